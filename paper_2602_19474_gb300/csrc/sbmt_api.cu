@@ -1878,71 +1878,54 @@ int mesh_quality(sbmt_ctx* ctx, sbmt_mesh mesh, sbmt_quality* out) {
   float* ar;
   unsigned long long* mm;
   double* part;
+  float2* ext;
   u32* hist;
   int rc;
+  const size_t sel_words = quality_select_words();
   if ((rc = aalloc(lane, &ar, T)) || (rc = aalloc(lane, &mm, 8)) || (rc = aalloc(lane, &part, 2 * NBLK)) ||
-      (rc = aalloc(lane, &hist, 32 + 2 * 4096))) {
+      (rc = aalloc(lane, &ext, NBLK)) || (rc = aalloc(lane, &hist, 32 + sel_words))) {
     arena_end(lane);
     return rc;
   }
   unsigned long long* cnt = mm + 3;
-  u32* h0 = hist + 32;
-  u32* h1 = h0 + 4096;
+  u32* select = hist + 32;
   const unsigned long long init[5] = {0x7FF0000000000000ull, 0x7FF0000000000000ull, 0ull, 0ull, 0ull};
+  // nearest-rank percentiles: the select's state starts with both ranks and
+  // no bits chosen
+  struct {
+    u32 pre[2];
+    u64 rank[2];
+  } sel = {{0, 0}, {(T + 1) / 2, (u64)std::ceil(0.95 * (double)T)}};
+  sel.rank[1] = std::max<u64>(1, std::min<u64>(sel.rank[1], T));
   std::vector<double> hpart(2 * NBLK);
   unsigned long long hmm[5];
   u32 hh[32];
   CK(cudaMemcpyAsync(mm, init, sizeof init, cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(hist, 0, 32 * sizeof(u32), st));
-  launch_quality(m->xy, m->tri, T, ar, mm, cnt, part, NBLK, hist, st);
+  CK(cudaMemsetAsync(hist, 0, (32 + sel_words) * sizeof(u32), st));
+  CK(cudaMemcpyAsync(select, &sel, sizeof sel, cudaMemcpyHostToDevice, st));
+  launch_quality(m->xy, m->tri, T, ar, mm, cnt, part, NBLK, hist, ext, select, st);
+  CK(cudaGetLastError());
   CK(cudaMemcpyAsync(hmm, mm, sizeof hmm, cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(hpart.data(), part, hpart.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(hh, hist, sizeof hh, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&sel, select, sizeof sel, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   auto dbl = [](unsigned long long b) {
     double d;
     std::memcpy(&d, &b, sizeof d);
     return d;
   };
-  out->min_angle_deg = dbl(hmm[0]), out->min_area = dbl(hmm[1]), out->ar_max = dbl(hmm[2]);
+  // the areas come doubled (the cross product): halving is exact
+  out->min_angle_deg = dbl(hmm[0]), out->min_area = 0.5 * dbl(hmm[1]), out->ar_max = dbl(hmm[2]);
   out->slivers = (int64_t)hmm[3], out->equilateral = (int64_t)hmm[4];
   double sa = 0.0, sa2 = 0.0;
   for (int b = 0; b < NBLK; ++b) sa += hpart[2 * b], sa2 += hpart[2 * b + 1];
+  sa *= 0.5, sa2 *= 0.25;
   out->area_mean = sa / (double)T;
   out->area_var = std::max(0.0, sa2 / (double)T - out->area_mean * out->area_mean);
   for (int k = 0; k < 30; ++k) out->angle_hist[k] = hh[k];
-  // nearest-rank percentiles: a radix select over the float bits in three
-  // levels, both ranks at once
-  u64 rank[2] = {(T + 1) / 2, (u64)std::ceil(0.95 * (double)T)};
-  rank[1] = std::max<u64>(1, std::min<u64>(rank[1], T));
-  u32 pre[2] = {0, 0};
-  const int lo_of[3] = {20, 10, 0}, width_of[3] = {12, 10, 10};
-  std::vector<u32> a0(4096), a1(4096);
-  for (int lev = 0; lev < 3; ++lev) {
-    const int lo = lo_of[lev], width = width_of[lev], nb = 1 << width;
-    CK(cudaMemsetAsync(h0, 0, 2 * 4096 * sizeof(u32), st));
-    launch_select_hist(ar, T, lo, width, pre[0], pre[1], lo + width, h0, h1, st);
-    CK(cudaMemcpyAsync(a0.data(), h0, nb * sizeof(u32), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(a1.data(), h1, nb * sizeof(u32), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    for (int r = 0; r < 2; ++r) {
-      const std::vector<u32>& h = r == 0 ? a0 : a1;
-      u64 cum = 0;
-      int bin = nb - 1;
-      for (int k = 0; k < nb; ++k) {
-        if (cum + h[k] >= rank[r]) {
-          bin = k;
-          break;
-        }
-        cum += h[k];
-      }
-      rank[r] -= cum;
-      pre[r] = (pre[r] << width) | (u32)bin;
-    }
-  }
   float f[2];
-  std::memcpy(&f[0], &pre[0], 4);
-  std::memcpy(&f[1], &pre[1], 4);
+  std::memcpy(f, sel.pre, sizeof f);
   out->ar_median = f[0], out->ar_p95 = f[1];
   arena_end(lane);
   return SBMT_OK;

@@ -210,13 +210,15 @@ size_t walk_chunks(u32 NP);
 size_t scan_scratch_words(u32 n);
 int launch_scan(const u32* in, int stride, u32* out, u32 n, u32* scratch, cudaStream_t st);
 
-// quality measures: per-triangle pass (mm: min angle, min area, max AR as
-// double bits; cnt: slivers, equilateral; part: per-block area sums; ar:
-// AR per triangle as float) and one level of the radix select of two ranks
+// quality measures of T triangles: mm [0] min angle, [1] min doubled area,
+// [2] max AR as double bits; cnt [0] slivers, [1] equilateral; part per block
+// (sum of doubled areas, of their squares); hist the 30 angle bins; ext per
+// block float extremes; select the percentiles' radix select (its ranks on
+// entry, the chosen floats' bits on return), quality_select_words() words
+size_t quality_select_words();
 int launch_quality(const double* xy, const int* tri, u64 T, float* ar, unsigned long long* mm,
-                   unsigned long long* cnt, double* part, int nblocks, u32* hist, cudaStream_t st);
-int launch_select_hist(const float* v, u64 T, int lo, int width, u32 pre0, u32 pre1, int above, u32* h0, u32* h1,
-                       cudaStream_t st);
+                   unsigned long long* cnt, double* part, int nblocks, u32* hist, float2* ext, u32* select,
+                   cudaStream_t st);
 
 // projection of a float pixel field (row pitch fpitch bytes): per-triangle
 // means into tri_value and bilinear vertex values into vertex_value (either

@@ -71,3 +71,31 @@ def test_paper_regime_quality(name):
     # uncut cells are equilateral: the median AR is 2 / sqrt(3)
     assert abs(q["ar_median"] - float(np.float32(2 / math.sqrt(3)))) == 0.0
     assert q["equilateral"] > q["triangles"] // 2
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 255, 257, 513, 4099])
+def test_shapes_at_the_filter_edges(n):
+    """Triangles at the edges of the single-precision decisions, on an imported
+    mesh: exact lattice cells, 30-60-90 and 45-degree shapes (on and off a bin
+    edge), side lengths within and beyond the equilateral tolerance, slivers
+    thinner than the filters take, and triangle counts around the block's and
+    the vector loads' remainders.  The tolerances are check_against_oracle's."""
+    rng = np.random.default_rng(n)
+    s3 = math.sqrt(3.0)
+    shapes = [
+        [(0, 0), (2, 0), (1, s3)], [(0, 0), (1, 0), (0, s3)], [(0, 0), (1, 0), (0, 1)],
+        [(0, 0), (2, 0), (1, s3 * (1 + 3e-10))], [(0, 0), (2, 0), (1, s3 * (1 + 3e-9))],
+        [(0, 0), (1, 0), (0.5, 1e-4)], [(0, 0), (4, 0), (3.9, 1e-7)], [(0, 0), (1, 0), (math.cos(math.radians(5)), math.sin(math.radians(5)))],
+        [(0, 0), (300, 0), (0, 0.01)], [(0, 0), (1e-4, 0), (0, 1e-4)],
+    ]
+    pts = []
+    for k in range(n):
+        p = np.array(shapes[k % len(shapes)] if k % 3 else rng.uniform(0, 2, (3, 2)), float)
+        pts.append(p + (rng.integers(0, 4096, 2) if k % 2 else 0))
+    xy = np.concatenate(pts)
+    c = ctx()
+    m = sb.mesh_import(c, xy, np.arange(3 * n, dtype=np.int32).reshape(n, 3))
+    mesh = sb.view_numpy(sb.mesh_query(c, m, -1))
+    q = sb.mesh_quality(c, m)
+    sb.mesh_release(c, m)
+    check_against_oracle(mesh, q)
