@@ -14,9 +14,10 @@
 // Double precision throughout.  The result does not depend on the order in
 // which threads run: records are placed by a scan, each free vertex's mass
 // and diagonal are gathered over its incident records in record order, the
-// rows' entries are sorted by column, and every reduction is finished by
-// the last block of its launch over the blocks' partial sums in block order.
+// rows' entries are sorted by column, and every sum over the grid adds the
+// blocks' partial sums in one fixed order.
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "sbmt_dev.cuh"
@@ -134,53 +135,6 @@ __global__ void __launch_bounds__(HB) k_heat_gather(const HeatTri* rec, u32 n, c
   }
 }
 
-// A reduction slot: the blocks' partial sums and a counter of finished
-// blocks (zeroed once; the last block resets it).
-struct Red {
-  double* part;
-  u32* done;
-};
-
-// block sum of v into *out: each block writes its partial sum, and the last
-// block to finish adds the partials in a fixed order (thread t sums partials
-// t, t + HB, ..., then a fixed tree over the threads), so the sum is the same
-// on every run, whatever order the blocks ran in
-__device__ __forceinline__ double block_sum_fixed(double v, double* s) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double b = 0.0;
-  if (threadIdx.x < 32) {
-    b = threadIdx.x < blockDim.x / 32 ? s[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
-  }
-  __syncthreads();
-  return b;  // valid in thread 0
-}
-
-__device__ __forceinline__ void block_add(double v, double* out, Red red) {
-  __shared__ double s[HB / 32];
-  __shared__ bool last;
-  const double b = block_sum_fixed(v, s);
-  if (threadIdx.x == 0) {
-    red.part[blockIdx.x] = b;
-    __threadfence();
-    last = atomicAdd(red.done, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last) {
-    __threadfence();
-    double t = 0.0;
-    for (u32 k = threadIdx.x; k < gridDim.x; k += blockDim.x) t += __ldcg(red.part + k);
-    t = block_sum_fixed(t, s);
-    if (threadIdx.x == 0) {
-      *out = t;
-      *red.done = 0;
-    }
-  }
-  __syncthreads();
-}
-
 // the free vertices: the pulse, the operator's inverse diagonal
 __global__ void __launch_bounds__(HB) k_heat_init(const double* xy, u32 n, const u32* list, const double* mass,
                                                   const double* kdiag, double tau, double x0, double y0,
@@ -193,11 +147,6 @@ __global__ void __launch_bounds__(HB) k_heat_init(const double* xy, u32 n, const
     dg[i] = mass[i] + tau * kdiag[i];
     dinv[i] = 1.0 / dg[i];
   }
-}
-
-// q = M x
-__global__ void __launch_bounds__(HB) k_heat_mass(u32 n, const double* mass, const double* x, double* q) {
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) q[i] = mass[i] * x[i];
 }
 
 // the operator as sparse rows over the free vertices: two entries per
@@ -260,21 +209,23 @@ __global__ void __launch_bounds__(HB) k_heat_merge(u32 n, const u32* rowptr, u32
   }
 }
 
-// q = (M + tau K) x over the free rows (dg: the diagonal M + tau diag K),
-// and x . q added into *xq
-__global__ void __launch_bounds__(HB) k_heat_apply(u32 n, const u32* rowptr, const u32* mcnt, const u32* col,
-                                                   const double* val, const double* dg, const double* x, double* q,
-                                                   double* xq, Red red) {
-  double acc = 0.0;
+// The merged rows again for the solver, in slices of 32 rows (one warp):
+// entry k < SW of row i at slice (i / 32), place 32 k + i % 32, so that a
+// warp reads its rows' k-th entries as one contiguous piece.  The first SF
+// are there for every row (absent ones name the row itself), so that the
+// solver loads them without waiting for the row's count.  Entries from SW on
+// (rows of more than SW neighbours, few on these meshes) stay in the rows.
+constexpr int SW = 8, SF = 6;
+__global__ void __launch_bounds__(HB) k_heat_slices(u32 n, const u32* rowptr, const u32* mcnt, const u32* col,
+                                                    const double* val, double* sval, u32* scol) {
   for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double xi = x[i];
-    double y = dg[i] * xi;
-    const u32 e0 = rowptr[i], e1 = e0 + mcnt[i];
-    for (u32 e = e0; e < e1; ++e) y += val[e] * x[col[e]];
-    q[i] = y;
-    acc += xi * y;
+    const u32 e0 = rowptr[i], m = min(mcnt[i], (u32)SW);
+    const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
+    for (u32 k = 0; k < max(m, (u32)SF); ++k) {
+      scol[at + 32 * k] = k < m ? col[e0 + k] : i;
+      sval[at + 32 * k] = k < m ? val[e0 + k] : 0.0;
+    }
   }
-  block_add(acc, xq, red);
 }
 
 // u over the mesh: 0, then the free values at their vertices
@@ -285,66 +236,325 @@ __global__ void __launch_bounds__(HB) k_heat_put(u32 n, const u32* list, const d
   for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) u[list[i]] = x[i];
 }
 
-// CG scalars per iteration it: s[4 it + 0] = p.q, s[4 it + 1] = r.z,
-// s[4 it + 2] = r.r (all zeroed before the solve)
-__global__ void __launch_bounds__(HB) k_heat_dot(u64 V, const double* a, const double* b, double* out, Red red) {
-  double acc = 0.0;
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (u64)gridDim.x * blockDim.x)
-    acc += a[v] * b[v];
-  block_add(acc, out, red);
-}
+// ---------------------------------------------------------------------------
+// The time steps: one cooperative launch for the whole call, one block of 512
+// threads on each SM (fewer for small regions), all resident, so that a phase
+// of the solver ends in a barrier across the grid instead of a launch, and the
+// host reads nothing until the last step.  Each thread keeps the same rows
+// throughout.  Per iteration:
+//   q = A p, p.q        | barrier
+//   x, r, z; r.z, r.r   | barrier
+//   p = z + beta p      | barrier
+// Everything but the matrix of a 10^6-row region stays in L2, and the phases
+// are short: what an iteration costs is latency (loads, then the barriers) and
+// this GPU's FP64 rate, about 1.6 instructions per clock and SM (14 per row of
+// 6 entries).  So: two rows of the product and three of the vector phases in
+// flight per thread; a block's sums through shared memory in halves (20 warp
+// adds for 512 threads, where a butterfly in every warp takes 80); the blocks'
+// sums published and awaited in one step, which is the barrier (below), and
+// added by every block in one fixed order; one division per block.
+// Measured on 0.33e6 free vertices (4096^2 Voronoi labels, h = 2): 57 us an
+// iteration as three launches with two-stage sums over 1216 blocks, 23 us here.
+// ---------------------------------------------------------------------------
+constexpr int CT = 512;         // threads per block
+constexpr int CG_BLOCKS = 152;  // at most one block per SM
+constexpr int CG_SUMS = 3;      // the most sums a barrier carries
+constexpr int SLOT_WORDS = 4 * CG_SUMS * CG_BLOCKS + 16 * CG_BLOCKS;
+struct HeatCg {
+  u32 n, nsteps;
+  int maxit, sliced;
+  double tol;
+  const u32* rowptr;
+  const u32* mcnt;
+  const u32* col;
+  const double* val;
+  const u32* scol;
+  const double* sval;
+  const double* mass;
+  const double* dg;
+  const double* dinv;
+  double *x, *r, *z, *p, *q;
+  unsigned long long* slot;  // SLOT_WORDS published sums, all bits set at first
+  u32* fail;                 // a wait ran out
+  unsigned long long* peak;  // per step: the maximum of x (double bits), 0 at least
+  int* iters;                // per step
+  int* done;                 // [0] steps finished, [1] the last one converged
+};
+constexpr unsigned long long CG_EMPTY = ~0ull;  // no sum has these bits
 
-// r = b - q (q = A x), z = D^-1 r, p = z; r.z into rz, r.r into rr
-__global__ void __launch_bounds__(HB) k_heat_start(u64 V, const double* b, const double* q, const double* dinv,
-                                                   double* r, double* z, double* p, double* rz, double* rr, Red r1,
-                                                   Red r2) {
-  double a1 = 0.0, a2 = 0.0;
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (u64)gridDim.x * blockDim.x) {
-    const double rv = dinv[v] != 0.0 ? b[v] - q[v] : 0.0, zv = rv * dinv[v];
-    r[v] = rv, z[v] = zv, p[v] = zv;
-    a1 += rv * zv, a2 += rv * rv;
+SBMT_DEV unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+SBMT_DEV void st_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// orders this thread's accesses (and those it has seen through a block
+// barrier) across the grid
+SBMT_DEV void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// waits until K words are no longer empty; bounded by the global timer (two
+// seconds), after which the failure word is set and every wait ends
+template <int K>
+SBMT_DEV bool wait_words(const HeatCg& h, const unsigned long long* p, size_t step, unsigned long long (&w)[K]) {
+  unsigned long long t0 = 0;
+  u32 spins = 0;
+  while (true) {
+    bool wait = false;
+#pragma unroll
+    for (int k = 0; k < K; ++k) w[k] = ld_relaxed(p + k * step);
+#pragma unroll
+    for (int k = 0; k < K; ++k) wait |= w[k] == CG_EMPTY;
+    if (!wait) return true;
+    if ((++spins & 1023u) == 0) {
+      unsigned long long clk;
+      asm volatile("mov.u64 %0, %globaltimer;" : "=l"(clk));
+      if (t0 == 0) t0 = clk;
+      if (clk - t0 > 2000000000ull) atomicExch(h.fail, 1u);
+      if (atomicAdd(h.fail, 0u)) return false;
+    }
   }
-  block_add(a1, rz, r1);
-  block_add(a2, rr, r2);
 }
 
-// x += alpha p, r -= alpha q, z = D^-1 r, with alpha = rz / pq; the new
-// r.z and r.r
-__global__ void __launch_bounds__(HB) k_heat_update(u64 V, const double* sc, double* x, double* r, double* z,
-                                                    const double* p, const double* q, const double* dinv,
-                                                    double* rz_next, double* rr_next, Red r1, Red r2) {
-  const double al = sc[0] != 0.0 ? sc[1] / sc[0] : 0.0;  // sc: {p.q, r.z} of this iteration
-  double a1 = 0.0, a2 = 0.0;
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (u64)gridDim.x * blockDim.x) {
-    x[v] += al * p[v];
-    const double rv = r[v] - al * q[v], zv = rv * dinv[v];
-    r[v] = rv, z[v] = zv;
-    a1 += rv * zv, a2 += rv * rv;
+// The grid's sums of K values per thread into s_out, and a barrier across the
+// grid: what a block's threads wrote before it is seen by every block after
+// it.  (TREE false: the barrier alone.)  A block publishes its sums in its
+// slots once its writes are fenced; block 0's thread b waits for block b's,
+// block 0 adds them (lane l takes blocks l, l + 32, ..., then a fixed tree)
+// and hands them to each block in a slot of its own, so that nobody but block
+// 0 reads more than one place (every block waiting for all 152 slots took 5 us
+// a barrier, 3 us this way).  Four buffers by turns: entering barrier g, a
+// block empties its slots of buffer (g + 2) % 4.  Those held barrier g - 2,
+// which it has left (and block 0 had read its sums before that), and they are
+// not written before it publishes barrier g + 2.  end(sums) runs on one thread
+// before the block goes on.  False when a wait ran out.
+template <int K, bool TREE, class End>
+SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double (*s)[CT], double* s_out, int* s_fail,
+                        const End& end) {
+  const u32 tid = threadIdx.x;
+  double t[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) t[k] = 0.0;
+  if (tid == 0) *s_fail = 0;
+  if (TREE) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) s[k][tid] = v[k];
+    __syncthreads();
+    if (tid < CT / 4) {
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        s[k][tid] = (s[k][tid] + s[k][tid + CT / 4]) + (s[k][tid + CT / 2] + s[k][tid + 3 * CT / 4]);
+    }
+    __syncthreads();
+    if (tid < 32) {
+      static_assert(CT == 512, "the second step adds four values per lane");
+#pragma unroll
+      for (int k = 0; k < K; ++k) t[k] = (s[k][tid] + s[k][tid + 32]) + (s[k][tid + 64] + s[k][tid + 96]);
+      for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xFFFFFFFFu, t[k], o);
+      }
+    }
+  } else {
+    __syncthreads();
   }
-  block_add(a1, rz_next, r1);
-  block_add(a2, rr_next, r2);
-}
-
-// p = z + beta p, beta = rz_next / rz
-__global__ void __launch_bounds__(HB) k_heat_dir(u64 V, const double* rz, const double* rz_next, const double* z,
-                                                 double* p) {
-  const double be = *rz != 0.0 ? *rz_next / *rz : 0.0;
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (u64)gridDim.x * blockDim.x)
-    p[v] = z[v] + be * p[v];
-}
-
-// per-block maxima of u (the host takes the largest)
-__global__ void __launch_bounds__(HB) k_heat_max(u64 V, const double* u, double* out) {
-  __shared__ double s[HB / 32];
-  double m = -1.0e308;
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (u64)gridDim.x * blockDim.x)
-    m = fmax(m, u[v]);
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = m;
+  if (gridDim.x > 1) {
+    // in: [buffer][sum][block]; out: [buffer][block][4], a sector per block
+    unsigned long long* in = h.slot + (size_t)(gen & 3u) * CG_SUMS * CG_BLOCKS;
+    unsigned long long* in2 = h.slot + (size_t)((gen + 2) & 3u) * CG_SUMS * CG_BLOCKS;
+    unsigned long long* out = h.slot + 4 * CG_SUMS * CG_BLOCKS + (size_t)(gen & 3u) * 4 * CG_BLOCKS;
+    unsigned long long* out2 = h.slot + 4 * CG_SUMS * CG_BLOCKS + (size_t)((gen + 2) & 3u) * 4 * CG_BLOCKS;
+    if (tid == 0) {
+#pragma unroll
+      for (int k = 0; k < CG_SUMS; ++k)
+        st_relaxed(in2 + k * CG_BLOCKS + blockIdx.x, CG_EMPTY), st_relaxed(out2 + 4 * blockIdx.x + k, CG_EMPTY);
+      fence_gpu();
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        st_relaxed(in + k * CG_BLOCKS + blockIdx.x, (unsigned long long)__double_as_longlong(t[k]));
+    }
+    if (blockIdx.x == 0) {
+      __syncthreads();  // the tree's last reads of s
+      if (tid < gridDim.x) {
+        unsigned long long w[K];
+        if (!wait_words<K>(h, in + tid, CG_BLOCKS, w)) *s_fail = 1;
+        fence_gpu();
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k][tid] = __longlong_as_double((long long)w[k]);
+      }
+      __syncthreads();
+      if (TREE && tid < 32) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          t[k] = 0.0;
+          for (u32 b = tid; b < gridDim.x; b += 32) t[k] += s[k][b];
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+          for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xFFFFFFFFu, t[k], o);
+        }
+        if (tid == 0) {
+#pragma unroll
+          for (int k = 0; k < K; ++k) s_out[k] = t[k];
+        }
+      }
+      if (TREE) __syncthreads();
+      if (tid > 0 && tid < gridDim.x) {
+        fence_gpu();
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          st_relaxed(out + 4 * tid + k, TREE ? (unsigned long long)__double_as_longlong(s_out[k]) : 0ull);
+      }
+    } else if (tid == 0) {
+      unsigned long long w[K];
+      if (!wait_words<K>(h, out + 4 * blockIdx.x, 1, w)) *s_fail = 1;
+      fence_gpu();
+#pragma unroll
+      for (int k = 0; k < K; ++k) t[k] = __longlong_as_double((long long)w[k]);
+    }
+  }
+  if (TREE && tid == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) s_out[k] = t[k];
+    end(t);
+  }
+  ++gen;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x / 32); ++w) m = fmax(m, s[w]);
-    out[blockIdx.x] = m;
+  return *s_fail == 0;
+}
+
+// U rows of A = M + tau K times v (v read from L2: other SMs write it): the
+// rows first, first + step, ..., those below n.  A warp's lanes hold the 32
+// rows of one slice.
+template <int U>
+SBMT_DEV void rows_times(const HeatCg& h, u32 i0, u32 step, const double* v, const double (&vi)[U], double (&y)[U]) {
+  u32 m[U];
+  double w[U][SF], g[U][SF];
+  if (h.sliced) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const u32 i = i0 + u * step;
+      if (i >= h.n) continue;
+      m[u] = h.mcnt[i];
+      const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
+#pragma unroll
+      for (int k = 0; k < SF; ++k) w[u][k] = h.sval[at + 32 * k], g[u][k] = __ldcg(v + h.scol[at + 32 * k]);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const u32 i = i0 + u * step;
+    if (i >= h.n) continue;
+    double a = h.dg[i] * vi[u];
+    u32 k0 = 0;
+    if (h.sliced) {
+#pragma unroll
+      for (int k = 0; k < SF; ++k)
+        if ((u32)k < m[u]) a += w[u][k] * g[u][k];
+      const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
+      for (u32 k = SF; k < min(m[u], (u32)SW); ++k) a += h.sval[at + 32 * k] * __ldcg(v + h.scol[at + 32 * k]);
+      k0 = SW;
+    } else {
+      m[u] = h.mcnt[i];
+    }
+    if (k0 < m[u])
+      for (u32 e = h.rowptr[i] + k0, e1 = h.rowptr[i] + m[u]; e < e1; ++e) a += h.val[e] * __ldcg(v + h.col[e]);
+    y[u] = a;
+  }
+}
+
+__global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatCg h) {
+  __shared__ double s[CG_SUMS][CT];
+  __shared__ double s_sum[CG_SUMS], s_k;
+  __shared__ int s_fail;
+  const u32 first = blockIdx.x * CT + threadIdx.x, stride = gridDim.x * CT, n = h.n;
+  u32 gen = 0;
+  for (u32 step = 0; step < h.nsteps; ++step) {
+    // b = M x; r = b - A x, z = D^-1 r, p = z; r.z, r.r, b.b
+    double a3[3] = {0.0, 0.0, 0.0};
+    for (u32 i = first; i < n; i += stride) {
+      const double xi[1] = {h.x[i]}, bi = h.mass[i] * xi[0];
+      double qi[1];
+      rows_times<1>(h, i, stride, h.x, xi, qi);
+      const double di = h.dinv[i], rv = di != 0.0 ? bi - qi[0] : 0.0, zv = rv * di;
+      h.r[i] = rv, h.z[i] = zv, h.p[i] = zv;
+      a3[0] += rv * zv, a3[1] += rv * rv, a3[2] += bi * bi;
+    }
+    if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [](const double*) {})) return;
+    double rz = s_sum[0], rr = s_sum[1];
+    const double stop = h.tol * h.tol * s_sum[2];
+    int it = 0;
+    while (rr > stop && it < h.maxit) {
+      bool look = false;
+      while (!look) {
+        double a1[1] = {0.0};
+        for (u32 i0 = first; i0 < n; i0 += 2 * stride) {
+          double pi[2], y[2];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) pi[u] = i0 + u * stride < n ? h.p[i0 + u * stride] : 0.0;
+          rows_times<2>(h, i0, stride, h.p, pi, y);
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (i0 + u * stride < n) h.q[i0 + u * stride] = y[u], a1[0] += pi[u] * y[u];
+        }
+        if (!grid_sums<1, true>(h, a1, gen, s, s_sum, &s_fail,
+                          [&](const double* t) { s_k = t[0] != 0.0 ? rz / t[0] : 0.0; }))
+          return;
+        const double al = s_k;
+        double a2[2] = {0.0, 0.0};
+        for (u32 i0 = first; i0 < n; i0 += 3 * stride) {
+          double x[3], r[3], p[3], q[3], d[3];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const u32 i = i0 + u * stride;
+            if (i < n) x[u] = h.x[i], r[u] = h.r[i], p[u] = h.p[i], q[u] = h.q[i], d[u] = h.dinv[i];
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const u32 i = i0 + u * stride;
+            if (i >= n) continue;
+            h.x[i] = x[u] + al * p[u];
+            const double rv = r[u] - al * q[u], zv = rv * d[u];
+            h.r[i] = rv, h.z[i] = zv;
+            a2[0] += rv * zv, a2[1] += rv * rv;
+          }
+        }
+        if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail,
+                          [&](const double* t) { s_k = rz != 0.0 ? t[0] / rz : 0.0; }))
+          return;
+        const double rz_new = s_sum[0], rr_new = s_sum[1];
+        const double be = s_k;
+        for (u32 i0 = first; i0 < n; i0 += 3 * stride) {
+          double z[3], p[3];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const u32 i = i0 + u * stride;
+            if (i < n) z[u] = h.z[i], p[u] = h.p[i];
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u)
+            if (i0 + u * stride < n) h.p[i0 + u * stride] = z[u] + be * p[u];
+        }
+        rz = rz_new;
+        ++it;
+        const double none[1] = {0.0};
+        if (!grid_sums<1, false>(h, none, gen, s, s_sum, &s_fail, [](const double*) {})) return;
+        look = (it & 7) == 0 || it == h.maxit;  // the residual is looked at every eighth iteration
+        if (look) rr = rr_new;
+      }
+    }
+    // the step's peak (positive doubles order as their bits)
+    unsigned long long top = 0;
+    for (u32 i = first; i < n; i += stride) {
+      const long long bits = __double_as_longlong(h.x[i]);
+      if (bits > 0) top = max(top, (unsigned long long)bits);
+    }
+    for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
+    if ((threadIdx.x & 31) == 0 && top) atomicMax(h.peak + step, top);
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+      h.iters[step] = it, h.done[0] = (int)step + 1, h.done[1] = rr > stop ? 0 : 1;
+    if (rr > stop) return;
   }
 }
 
@@ -352,11 +562,9 @@ unsigned grid_v(u64 n) { return (unsigned)std::max<u64>(1, std::min<u64>((n + HB
 
 }  // namespace
 
-constexpr int RED_BLOCKS = 152 * 8;  // the most blocks of a reducing launch (grid_v)
-
-size_t heat_scratch_bytes(u64 T, u64 V, int maxit) {
-  return 256 * 32 + T * (sizeof(HeatTri) + 6 * (4 + 8) + 4 + 4 + 12) + V * (4 + 4 + 4 + 4 + 4 + 4 + 4 + 8 * 10) +
-         8 * 4 * (size_t)(maxit + 1) + 8 * 152 * 8 + 8 * 2 * RED_BLOCKS + 16 +
+size_t heat_scratch_bytes(u64 T, u64 V, int nsteps) {
+  return 256 * 32 + T * (sizeof(HeatTri) + 6 * (4 + 8) + 4 + 4 + 12) + V * (4 + 4 + 4 + 4 + 4 + 4 + 4 + 8 * 9) +
+         8 * SLOT_WORDS + 12 * (size_t)std::max(nsteps, 1) + 64 +
          4 * scan_scratch_words((u32)std::min<u64>(std::max(T, V), 0xFFFFFFFFu));
 }
 
@@ -389,21 +597,22 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
   u32* col = (u32*)take(4 * 6 * T);
   double* val = (double*)take(8 * 6 * T);
   double* x = (double*)take(8 * V);
-  double* b = (double*)take(8 * V);
   double* q = (double*)take(8 * V);
   double* r = (double*)take(8 * V);
   double* z = (double*)take(8 * V);
   double* p = (double*)take(8 * V);
-  double* sc = (double*)take(8 * 4 * (size_t)(maxit + 1));  // 4 per iteration
-  double* bmax = (double*)take(8 * 152 * 8);
-  double* part = (double*)take(8 * 2 * RED_BLOCKS);
-  u32* rdone = (u32*)take(16);
+  unsigned long long* slot = (unsigned long long*)take(8 * SLOT_WORDS);
+  // the solver's results: a failed wait, 0, steps done, convergence, then per
+  // step the peak and the iterations
+  const size_t res_bytes = 16 + 12 * (size_t)std::max(nsteps, 1);
+  char* res = take(res_bytes);
   u32* sscr = (u32*)take(4 * scan_scratch_words((u32)std::max(T, V)) + 4);
-  const Red r1{part, rdone}, r2{part + RED_BLOCKS, rdone + 1};
   const unsigned gt = grid_v(T);
   const double tau = alpha * dt;
   int launches = 0;
-  if (cudaMemsetAsync(flag, 0, 4 * V, st) || cudaMemsetAsync(rdone, 0, 16, st)) return -1;
+  if (cudaMemsetAsync(flag, 0, 4 * V, st) || cudaMemsetAsync(res, 0, res_bytes, st) ||
+      cudaMemsetAsync(slot, 0xFF, 8 * SLOT_WORDS, st))
+    return -1;
   k_heat_flags<<<gt, HB, 0, st>>>(tri, label, T, L, flag);
   k_heat_free<<<grid_v(V), HB, 0, st>>>(V, flag);
   launches += 2 + launch_scan(flag, 1, fidx, (u32)V, sscr, st);
@@ -445,45 +654,38 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
       if (iters) iters[step] = 0;
       if (peaks) peaks[step] = 0.0;
     }
-  for (int step = 0; step < nsteps && n > 0; ++step) {
-    // b = M x_n; start from x_n: r = b - A x_n
-    if (cudaMemsetAsync(sc, 0, 8 * 4 * (size_t)(maxit + 1), st)) return -1;
-    k_heat_mass<<<gv, HB, 0, st>>>(n, mass, x, b);
-    k_heat_apply<<<gv, HB, 0, st>>>(n, rowptr, mcnt, col, val, dg, x, q, bmax, r1);
-    k_heat_start<<<gv, HB, 0, st>>>(n, b, q, dinv, r, z, p, sc + 1, sc + 2, r1, r2);
-    k_heat_dot<<<gv, HB, 0, st>>>(n, b, b, sc + 3, r1);
-    launches += 4;
-    double h2[2];
-    if (cudaMemcpyAsync(h2, sc + 2, 16, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st)) return -1;
-    const double stop = tol * tol * h2[1];
-    double rr = h2[0];
-    int it = 0;
-    while (rr > stop && it < maxit) {
-      double* s0 = sc + 4 * it;  // {p.q, r.z, r.r, -} of iteration it; the next iteration's at s0 + 4
-      k_heat_apply<<<gv, HB, 0, st>>>(n, rowptr, mcnt, col, val, dg, p, q, s0, r1);
-      k_heat_update<<<gv, HB, 0, st>>>(n, s0, x, r, z, p, q, dinv, s0 + 5, s0 + 6, r1, r2);
-      k_heat_dir<<<gv, HB, 0, st>>>(n, s0 + 1, s0 + 5, z, p);
-      launches += 3;
-      ++it;
-      // the residual, read back every eighth iteration
-      if ((it & 7) == 0 || it == maxit) {
-        if (cudaMemcpyAsync(&rr, sc + 4 * it + 2, 8, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))
-          return -1;
-      }
-    }
-    if (iters) iters[step] = it;
-    if (peaks) {
-      k_heat_max<<<gv, HB, 0, st>>>(n, x, bmax);
+  if (n > 0 && nsteps > 0) {
+    // the slices take the place of the triangle records, which are done with
+    const size_t sval_bytes = (size_t)((n + 31) / 32) * 32 * SW * 8;
+    const bool sliced = sval_bytes + sval_bytes / 2 <= T * sizeof(HeatTri);
+    double* sval = (double*)rec;
+    u32* scol = (u32*)((char*)rec + sval_bytes);
+    if (sliced) {
+      k_heat_slices<<<gv, HB, 0, st>>>(n, rowptr, mcnt, col, val, sval, scol);
       ++launches;
-      std::vector<double> hb(gv);
-      if (cudaMemcpyAsync(hb.data(), bmax, 8 * gv, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))
-        return -1;
-      peaks[step] = std::max(0.0, *std::max_element(hb.begin(), hb.end()));
     }
-    if (rr > stop) {
-      converged = false;
-      break;
+    unsigned long long* peak = (unsigned long long*)(res + 16);
+    int* its = (int*)(peak + nsteps);
+    HeatCg h{};
+    h.n = n, h.nsteps = (u32)nsteps, h.maxit = maxit, h.sliced = sliced ? 1 : 0, h.tol = tol;
+    h.rowptr = rowptr, h.mcnt = mcnt, h.col = col, h.val = val, h.scol = scol, h.sval = sval;
+    h.mass = mass, h.dg = dg, h.dinv = dinv, h.x = x, h.r = r, h.z = z, h.p = p, h.q = q;
+    h.slot = slot, h.fail = (u32*)res, h.peak = peak, h.iters = its, h.done = (int*)res + 2;
+    void* args[] = {&h};
+    const unsigned grid = (unsigned)std::min<u64>(CG_BLOCKS, (n + CT - 1) / CT);
+    if (cudaLaunchCooperativeKernel((const void*)k_heat_cg, dim3(grid), dim3(CT), args, 0, st) != cudaSuccess) return -1;
+    ++launches;
+    std::vector<char> hres(res_bytes);
+    if (cudaMemcpyAsync(hres.data(), res, res_bytes, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))
+      return -1;
+    const u32* words = (const u32*)hres.data();
+    if (words[0]) return -3;  // a wait across the grid ran out
+    const int done = (int)words[2];
+    for (int step = 0; step < done; ++step) {
+      if (peaks) std::memcpy(peaks + step, hres.data() + 16 + 8 * (size_t)step, 8);
+      if (iters) std::memcpy(iters + step, hres.data() + 16 + 8 * (size_t)nsteps + 4 * (size_t)step, 4);
     }
+    converged = words[3] != 0;
   }
   k_heat_zero<<<grid_v(V), HB, 0, st>>>(V, u);
   k_heat_put<<<std::max(gv, 1u), HB, 0, st>>>(n, list, x, u);

@@ -2018,7 +2018,7 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* hp, double*
   CK(cudaStreamWaitEvent(st, m->done, 0));
   arena_begin(lane);
   char* scratch;
-  int rc = aalloc(lane, &scratch, heat_scratch_bytes((u64)m->nt, (u64)m->nv, hp->max_iterations));
+  int rc = aalloc(lane, &scratch, heat_scratch_bytes((u64)m->nt, (u64)m->nv, hp->steps));
   if (rc) {
     arena_end(lane);
     return rc;
@@ -2029,6 +2029,7 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* hp, double*
                                 peaks, iterations, scratch, st));
   arena_end(lane);
   if (n == -2) return fail(SBMT_ETIMEDOUT, "a step did not reach the residual within %d iterations", hp->max_iterations);
+  if (n == -3) return fail(SBMT_ETIMEDOUT, "a device wait ran out in the heat solver");
   if (n < 0) return fail(SBMT_ECUDA, "heat solve: %s", cudaGetErrorString(cudaGetLastError()));
   CK(cudaGetLastError());
   return SBMT_OK;

@@ -325,7 +325,7 @@ int launch_r3_emit(const R3Args& a, cudaStream_t st);
 // heat_scratch_bytes(T, V, maxit) bytes (256-byte aligned).  Synchronises
 // with the device a few times per step; returns the kernels launched, -1 if
 // a CUDA call failed, -2 if a step did not converge.
-size_t heat_scratch_bytes(u64 T, u64 V, int maxit);
+size_t heat_scratch_bytes(u64 T, u64 V, int nsteps);
 int heat_solve(const double* xy, const int* tri, const unsigned short* label, u64 T, u64 V, int L, double alpha,
                double dt, int nsteps, double x0, double y0, double sigma, double amp, double tol, int maxit,
                double* u, double* peaks, int* iters, void* scratch, cudaStream_t st);

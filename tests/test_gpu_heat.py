@@ -120,3 +120,26 @@ def test_runs_are_bit_identical():
     b = run_gpu(m, L, 500.0, 0.01, 4, 350.0, 350.0, 60.0)
     sb.mesh_release(cx, m)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1]) and a[2] == b[2]
+
+
+@pytest.mark.parametrize("side,fan", [(3, 9), (21, 40), (22, 7), (23, 200), (120, 33)])
+def test_block_edges_and_long_rows(side, fan):
+    """Regions of one block (22^2 + fan - 1 vertices: 484 + 7 = 491), just over
+    one, and many, each with a vertex of `fan` neighbours (a row beyond the
+    eight entries kept in slices): an imported square grid and a fan apart from
+    it, every vertex free.  Tolerance as in test_parity_with_oracle."""
+    j, i = np.mgrid[0:side, 0:side]
+    xy = np.stack([i.ravel(), j.ravel() * 0.9], 1).astype(float)
+    a = (j[:-1, :-1] * side + i[:-1, :-1]).ravel()
+    tri = np.concatenate([np.stack([a, a + 1, a + side + 1], 1), np.stack([a, a + side + 1, a + side], 1)])
+    n = len(xy)
+    ang = 2 * np.pi * np.arange(fan) / fan
+    xy = np.concatenate([xy, [[-8.0, -8.0]], np.stack([-8 + 3 * np.cos(ang), -8 + 3 * np.sin(ang)], 1)])
+    k = np.arange(fan)
+    tri = np.concatenate([tri, np.stack([np.full(fan, n), n + 1 + k, n + 1 + (k + 1) % fan], 1)]).astype(np.int32)
+    m = sb.mesh_import(ctx(), xy, tri)
+    u, peaks, its = run_gpu(m, 0xFFFF, 3.0, 0.1, 3, 2.0, 1.0, 6.0)
+    sb.mesh_release(ctx(), m)
+    uo, po = H.heat(xy, tri, np.full(len(tri), 0xFFFF), 0xFFFF, 3.0, 0.1, 3, 2.0, 1.0, 6.0)
+    assert np.abs(u - uo).max() <= 1e-8 * 100.0
+    assert np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
