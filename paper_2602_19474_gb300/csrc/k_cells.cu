@@ -312,7 +312,7 @@ SBMT_DEV u32 stage_tier_t(const GridP& g, const CellGeo& cg, const CutRec& rec, 
 // Tier-T / Tier-G, triangle and inside-vertex counts) added to the bucket's
 // totals, for a Tier-T cell its staged patch, and a Tier-G cell counted
 // (cells in ngcell, triangles in ngtri, cells per local vertex count in
-// gcnt, counts above TIERG_WN pooled at TIERG_WN + 1).
+// gcnt, tierg_size).
 // The records of every job form one work queue, handed out in chunks of
 // CUT_CHUNK records of one job and one piece class (recpre[njobs + 1 + k]:
 // the chunks before job k), so that a block works for one job at a time with
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(128, 8) k_cutcells_b(const __grid_constant__ J
       const int lane = threadIdx.x & 31, lead = __ffs(act) - 1;
       const u32 t = __reduce_add_sync(act, kl.ntri);
       if (lane == lead) atomicAdd(jc(J, JC_NGCELL), (u32)__popc(act)), atomicAdd(jc(J, JC_NGTRI), t);
-      const u32 n = kl.ntri + 2 - kl.nchain, key = n > TIERG_WN ? TIERG_WN + 1 : n;
+      const u32 key = (u32)tierg_size((int)(kl.ntri + 2 - kl.nchain));
       const unsigned peers = __match_any_sync(act, key);
       if (lane == __ffs(peers) - 1) atomicAdd(&bd->gcnt[key], (u32)__popc(peers));
     }

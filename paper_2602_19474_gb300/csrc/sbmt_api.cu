@@ -627,7 +627,7 @@ int check_params(const sbmt_image* img, const sbmt_params* pr, bool pre = false,
 GridP grid_of(const sbmt_image& img, const sbmt_params& pr) {
   GridP g{};
   g.W = img.width, g.H = img.height;
-  g.p = pr.h_num, g.q = pr.h_den, g.S = 6 * g.q;
+  g.p = pr.h_num, g.q = pr.h_den, g.S = 6 * g.q, g.invS = 1.0 / (double)g.S;
   g.ox = 3 * g.q * (i64)pr.origin2x, g.oy = 3 * g.q * (i64)pr.origin2y;
   return g;
 }
@@ -904,6 +904,7 @@ int mesh_run(sbmt_ctx* ctx, Lane* lane, const sbmt_image* imgs, int n, const sbm
       (rc = aalloc(lane, &bp.wlist, std::max<u64>(np_all, 1))) ||
       (rc = aalloc(lane, &bp.big, std::max<u64>(nbe_all, 1))))
     return bail(rc);
+  bp.wlast = bp.wlist + std::max<u64>(np_all, 1) - 1;
   std::vector<ScanJob> sj1(2 * n), sj2;
   const size_t bdw = (batch_dev_words(n) + 63) & ~(size_t)63;
   std::vector<u32> t1pre(2 * n + 1, 0), t2pre;
@@ -1177,7 +1178,7 @@ int pre_one(sbmt_ctx* ctx, Lane* lane, const sbmt_image* img, const sbmt_params*
   CK(cudaSetDevice(ctx->device));
   GridP g{};
   g.W = img->width, g.H = img->height;
-  g.p = pr->h_num, g.q = pr->h_den, g.S = 6 * g.q;
+  g.p = pr->h_num, g.q = pr->h_den, g.S = 6 * g.q, g.invS = 1.0 / (double)g.S;
   g.ox = 3 * g.q * (i64)pr->origin2x, g.oy = 3 * g.q * (i64)pr->origin2y;
   const Tables* tbp;
   const i64* dt;
@@ -1495,7 +1496,6 @@ int mesh_create(sbmt_ctx** out, int device, size_t pool_bytes, void* cuda_stream
   if (cudaGetDeviceCount(&n) != cudaSuccess || n == 0) return fail(SBMT_ECUDA, "no CUDA device");
   if (device < 0 || device >= n) return fail(SBMT_EINVAL, "device %d of %d", device, n);
   CK(cudaSetDevice(device));
-  if (tierg_init()) return fail(SBMT_ECUDA, "kernel attributes");
   sbmt_ctx* ctx = new sbmt_ctx();
   ctx->device = device;
   if (cuda_stream) {

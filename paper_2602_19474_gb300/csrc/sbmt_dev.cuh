@@ -23,8 +23,10 @@ constexpr u32 NONE = 0xFFFFFFFFu;
 constexpr int OUTSIDE = 0x10000;  // label outside the image: above every pixel label
 constexpr int CB_LOG = 10;        // base cells per cell bucket (2^10)
 constexpr int EB_LOG = 11;        // grid-edge ids per event bucket (2^11)
-constexpr int TIERG_TN = 9;      // Tier-G cells up to this many local vertices may run one thread each
-constexpr int TIERG_WN = 16;     // Tier-G cells up to this many local vertices fit the warp path's small state
+constexpr int TIERG_TN = 8;       // Tier-G cells up to this many local vertices run 8 lanes each
+constexpr int TIERG_WN = 16;      // Tier-G cells up to this many run 16 lanes each
+constexpr int TIERG_SIZES = TIERG_WN + 3;  // counted per size up to TIERG_WN, then up to 32 and above together
+SBMT_HD int tierg_size(int n) { return n <= TIERG_WN ? n : n <= 32 ? TIERG_WN + 1 : TIERG_WN + 2; }
 constexpr u32 OVER_CAP = 1024;   // ids of cells over the Tier-G vertex limit kept per mesh
 constexpr u32 RANK_SMALL = 256;  // event buckets up to this size are ranked by one small block each
 
@@ -188,6 +190,7 @@ struct __align__(16) TStage {
 struct GridP {
   int W, H;
   i64 p, q, S, ox, oy;  // h = p/q, S = 6q, origin scaled by S
+  double invS;          // 1 / S
   int j0, nrows;        // strip rows meeting the image rectangle
   int vj0, nvrows;      // lattice vertex rows used
   const i64* clo;       // per strip row: first cell index c

@@ -109,10 +109,9 @@ SBMT_DEV int job_of(const u32* bpre, int njobs, u32 b) {
 
 // batch-wide state of the persistent stages
 struct BatchDev {
-  u32 gcnt[TIERG_WN + 2];  // Tier-G cells per local vertex count (above TIERG_WN pooled)
-  u32 gcur[TIERG_WN + 2];  // cursors while ordering
-  u32 nolist, nwlist, nbig, err;
-  u32 nslist;              // cells of the small-state warp list
+  u32 gcnt[TIERG_SIZES];  // Tier-G cells per local vertex count (tierg_size)
+  u32 gcur[TIERG_SIZES];  // cursors while ordering: in the end the lists' lengths
+  u32 nolist, nslist, nbig, err;
   u32 recpre[1];           // 2 (njobs + 1) entries: prefix of the jobs' cut-cell records, then of
                            // their chunks of CUT_CHUNK records
 };
@@ -122,7 +121,8 @@ struct BatchPtrs {
   BatchDev* bd;
   uint2* olist;  // (job, record) of Tier-G cells of at most TIERG_TN vertices, largest first
   uint2* slist;  // (job, record) of Tier-G cells of TIERG_TN + 1 .. TIERG_WN vertices, largest first
-  uint2* wlist;  // (job, record) of Tier-G cells above TIERG_WN vertices
+  uint2* wlist;  // (job, record) of Tier-G cells of TIERG_WN + 1 .. 32 vertices, from the front
+  uint2* wlast;  // wlist's last entry: those above 32 vertices, backwards from here
   uint2* big;    // (job, event bucket) of registry buckets above RANK_SMALL events
 };
 
@@ -179,15 +179,12 @@ int launch_cutcells_b(const Job* one, const Job* jobs, int njobs, const BatchPtr
 int launch_emit_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, cudaStream_t st);
 int launch_lattice_b(const Job* jobs, const u32* bpre_tab, u32 nb_tab, const u32* bpre_xy, u32 nb_xy, int njobs,
                      cudaStream_t st);
-// Tier-G: ordering (bpre over warps of buckets), then the persistent thread
-// and warp kernels over the batch's lists (warp kernels on st2 when given).
-// Cells of at most TIERG_TN vertices run one thread each, larger ones one warp
-// each (a small-state kernel up to TIERG_WN vertices, a large-state one above).
+// Tier-G: ordering (bpre over warps of buckets), then persistent kernels over
+// the batch's lists: groups of 8 lanes for cells of at most TIERG_TN vertices
+// (blocks_per_sm blocks of 64 threads an SM), of 16 up to TIERG_WN and of 32
+// up to 32, and a warp on vertex lists above (these on st2 when given).
 int launch_tierg_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, const BatchPtrs& bp,
-                   int thread_blocks_per_sm, cudaStream_t st, cudaStream_t st2, cudaEvent_t ev_order,
-                   cudaEvent_t ev_warp);
-// kernel attributes set once per device (outside any stream capture)
-int tierg_init();
+                   int blocks_per_sm, cudaStream_t st, cudaStream_t st2, cudaEvent_t ev_order, cudaEvent_t ev_warp);
 // status words of every job into its mapped host slot
 int launch_status_b(const Job* jobs, int njobs, const BatchPtrs& bp, cudaStream_t st);
 

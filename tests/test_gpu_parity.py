@@ -118,3 +118,18 @@ def test_serving_pool_images_all_h():
         run_both(img, hn, stages=False)
     for k in (order[len(order) // 4], order[len(order) // 2], order[(3 * len(order)) // 4]):
         run_both(synth.serving_image(specs[k]), specs[k][2], stages=False)
+
+
+@pytest.mark.parametrize("seed,h,sigma,sizes", [
+    (0, 4, 1.0, (7, 8, 9, 16, 17)),
+    (0, 8, 1.5, (8, 9, 16, 17)),
+    (0, 14, 2.0, (8, 9, 16, 17, 32, 33, 37)),
+])
+def test_tier_g_cells_of_every_group_size(seed, h, sigma, sizes):
+    """Tier-G cells of as many vertices as a group of 8, 16 or 32 lanes takes,
+    and of one more (the list form above 32): the mesh is the oracle's."""
+    img = synth.noise_bitmap(np.random.default_rng(seed), 260, 230, sigma)
+    g, o = run_both(img, h)
+    cut = o["cut"][o["cut"][:, 4] == 1]
+    have = set((cut[:, 2] + 2 - cut[:, 3]).tolist())
+    assert have.issuperset(sizes), sorted(have)
