@@ -38,11 +38,19 @@
 // (every cell: a cell whose pixel box carries one label is uncut and takes
 // that label, with no double-precision work; the others are listed);
 // k_r3_count (the listed cells: triangles, events on the edges each owns --
-// the smaller of the two cells beside an edge -- and inside vertices); three
-// scans; k_r3_emit_uncut; k_r3_emit (the listed cells: Tier-T patches, the
-// greedy rule for Tier-G cells of at most 12 nodes, larger ones queued);
-// k_r3_tierg (one warp per queued cell).
+// the smaller of the two cells beside an edge -- and inside vertices; a
+// record of what it found for each cut cell); three scans; k_r3_emit_uncut;
+// k_r3_cells (the cut cells of at most 32 nodes: Tier-T patches and the
+// greedy rule, a group of lanes a cell, from the records); k_r3_tierg (one
+// warp per larger cell).
+//
+// One thread per cut cell rebuilt the cell's graph in double formulas, twice
+// for a Tier-G cell, with 3 of 32 lanes active: 1.20 + 0.71 ms for the 1.9e5 cut
+// cells of a 4096^2 label image at h = 2.  With the records, and one event,
+// line, candidate or triangle per lane, 0.59 ms (0.54 -> 0.62 ms for the count
+// that writes them).
 #include "sbmt_cell.cuh"
+#include "sbmt_greedy.cuh"
 #include "sbmt_keys.cuh"
 #include "sbmt_launch.h"
 
@@ -180,12 +188,18 @@ SBMT_DEV R3Split r3_split(double v) {
   s.f = __fmul_rn(__fsub_rn(__int_as_float(0x4B000000 | n23), 8388608.0f), 1.1920928955078125e-7f);  // n23 2^-23
   return s;
 }
+struct R3Corner {  // what the line tests need of it
+  i64 fx;
+  bool inexact;
+};
 // v against the pixel line k - 1/2, exactly, from fx = floor(v 2^36):
 // below iff fx < (k - 1/2) 2^36; above iff fx is greater, or equal with
 // bits dropped
 SBMT_DEV i64 r3_line36(i64 k) { return (k << 36) - (1ll << 35); }
-SBMT_DEV bool r3_lt(const R3Split& v, i64 k) { return v.fx < r3_line36(k); }
-SBMT_DEV bool r3_gt(const R3Split& v, i64 k) {
+template <class V>
+SBMT_DEV bool r3_lt(const V& v, i64 k) { return v.fx < r3_line36(k); }
+template <class V>
+SBMT_DEV bool r3_gt(const V& v, i64 k) {
   const i64 t = r3_line36(k);
   return v.fx > t || (v.fx == t && v.inexact);
 }
@@ -217,11 +231,17 @@ __device__ __noinline__ void r3_cross_exact(double2 P, double2 Q, double c0, boo
   *corner = r3_at_corner(vert ? r3_vy(P, Q, c0) : r3_hx(P, Q, c0), j);
 }
 
+// an event as the count pass records it: pixel indices m, k (at most 32768),
+// the cell's edge and the kind; an inside vertex has kind 3, edge 3
+SBMT_DEV u64 r3_entry(int edge, int kind, int m, int k) {
+  return (u64)(u32)m | (u64)(u32)k << 16 | (u64)(edge << 2 | kind) << 32;
+}
+
 // the number of events of the edge from P (its lower-id end) to Q, or -1
 // past R3_MAXE, through the filters (the count pass's form: positions are
-// not needed there); ev receives the events' kinds and pixel indices, for
+// not needed there); ev receives the events (r3_entry), for the record and for
 // the corner found on both line families to count once
-SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, R3Ev* ev) {
+SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, int edge, u64* ev) {
   int n = 0;
   const bool hz = P.y == Q.y, vt = P.x == Q.x;
   const R3Split px = r3_split(P.x), py = r3_split(P.y), qx = r3_split(Q.x), qy = r3_split(Q.y);
@@ -244,8 +264,7 @@ SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, R3Ev* ev) {
       else r3_cross_exact(P, Q, (double)k - 0.5, false, &j, &corner);
       if (corner ? r3_corner_event(a, j, k, hz, vt) : r3_hb(a, j, k)) {
         if (n == R3_MAXE) return -1;
-        ev[n].kind = corner ? 2 : 0, ev[n].m = (int)j, ev[n].k = (int)k;
-        ++n;
+        ev[n++] = r3_entry(edge, corner ? 2 : 0, (int)j, (int)k);
       }
     }
   }
@@ -267,14 +286,13 @@ SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, R3Ev* ev) {
       if (corner) {
         bool dup = false;
         for (int t = 0; t < n; ++t)
-          if (ev[t].kind == 2 && ev[t].m == (int)m && ev[t].k == (int)j) dup = true;
+          if (ev[t] == r3_entry(edge, 2, (int)m, (int)j)) dup = true;
         if (dup || !r3_corner_event(a, m, j, hz, vt)) continue;
       } else if (!r3_vb(a, m, j)) {
         continue;
       }
       if (n == R3_MAXE) return -1;
-      ev[n].kind = corner ? 2 : 1, ev[n].m = (int)m, ev[n].k = (int)j;
-      ++n;
+      ev[n++] = r3_entry(edge, corner ? 2 : 1, (int)m, (int)j);
     }
   }
   return n;
@@ -372,8 +390,8 @@ SBMT_DEV bool r3_ccw(const double2* K, const i64* X, const i64* Y) {
   return r3_orient(K[0], K[1], K[2]) > 0.0;
 }
 
-// the boundary vertices strictly inside the cell, as corner ids y (W+1) + x
-// in id order; the count, -1 past R3_MAXI, -2 for a row the cell meets in
+// the boundary vertices strictly inside the cell (r3_entry), in corner-id
+// order; the count, -1 past R3_MAXI, -2 for a row the cell meets in
 // other than two points.  Rows strictly inside the cell's y-range; on each,
 // the chord's two ends (a corner on the row, or an edge crossing it, as in
 // r3_chord): a corner compared with the pixel corners exactly through its
@@ -410,7 +428,7 @@ SBMT_DEV bool r3_end_above(const R3Cell& C, const R3Split* sx, const R3End& e, i
   if (__fsub_rn(h, e.w) > e.T) return false;
   return r3_end_cmp_exact(C, e.src, cx, c0) > 0;
 }
-SBMT_DEV int r3_inside(const R3Args& a, const R3Cell& C, u32* out) {
+SBMT_DEV int r3_inside(const R3Args& a, const R3Cell& C, u64* out) {
   R3Split sx[3], sy[3];
   for (int q = 0; q < 3; ++q) sx[q] = r3_split(C.K[q].x), sy[q] = r3_split(C.K[q].y);
   float sl[3], D[3];
@@ -456,11 +474,222 @@ SBMT_DEV int r3_inside(const R3Args& a, const R3Cell& C, u32* out) {
       if (!inside) continue;
       if (!r3_is_vertex(r3_cmask(a, cx, cy))) continue;
       if (n == R3_MAXI) return -1;
-      if (out) out[n] = (u32)(cy * (a.W + 1) + cx);
+      out[n] = r3_entry(3, 3, (int)cx, (int)cy);
       ++n;
     }
   }
   return n;
+}
+
+// ---------------------------------------------------------------------------
+// the same for a cut cell without a record (the count pass ran out of room),
+// by a group of G lanes (sbmt_greedy.cuh): the crossings of its edges with the
+// pixel lines and the pixel corners of its bounding box are shared out over the
+// lanes
+// ---------------------------------------------------------------------------
+// a bounded list of the events found on the cell's edges, in no order
+constexpr int R3_LIST = R3_MAXN;
+struct R3Found {
+  int2 mk[R3_LIST];              // the pixel indices (m, k)
+  unsigned char jk[R3_LIST];     // edge << 2 | kind
+  u32 ins[R3_MAXI];              // inside vertices: corner ids, in id order
+};
+// the pixel lines strictly between two coordinates (closed: or through one of
+// them), within [0, most]: the first, and their number
+template <class V>
+SBMT_DEV int r3_lines(const V& a, const V& b, int most, int* first, bool closed = false) {
+  const bool sw = b.fx < a.fx || (b.fx == a.fx && a.inexact);  // the lower of the two first
+  const i64 lo = sw ? b.fx : a.fx, hi = sw ? a.fx : b.fx;
+  const bool hx = sw ? a.inexact : b.inexact;
+  constexpr i64 HALF = 1ll << 35;
+  const bool lx = sw ? b.inexact : a.inexact;
+  const i64 k0 = max(((lo + HALF - (closed && !lx ? 1 : 0)) >> 36) + 1, (i64)0);
+  const i64 k1 = min((hi + HALF - (hx || closed ? 0 : 1)) >> 36, (i64)most);
+  *first = (int)k0;
+  return k1 < k0 ? 0 : (int)(k1 - k0 + 1);
+}
+struct R3Geo2 {  // the cell in the filters' numbers
+  R3Split x[3], y[3];
+};
+SBMT_DEV bool r3_same(double a, double b) {  // a == b without an FP64 compare (finite numbers)
+  const i64 p = __double_as_longlong(a), q = __double_as_longlong(b);
+  return p == q || ((p | q) << 1) == 0;
+}
+
+// the cell's events into F (up to R3_LIST of them) and their number per edge,
+// the same in every lane; each through the float filter of r3_cross_tol, with
+// the double formula where it does not decide.  n = 0 cells: live false.
+template <int G>
+SBMT_DEV int r3_events(const R3Args& a, const R3Cell& C, const R3Geo2& S, bool live, const GLane<G>& me, R3Found& F,
+                       int (&cnt)[3]) {
+  int ne = 0;
+  cnt[0] = cnt[1] = cnt[2] = 0;
+#pragma unroll
+  for (int vert = 0; vert < 2; ++vert) {
+    int first[3], num[3], total = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int w = j == 2 ? 0 : j + 1;
+      num[j] = !live ? 0 : vert ? r3_lines(S.x[j], S.x[w], a.W, &first[j]) : r3_lines(S.y[j], S.y[w], a.H, &first[j]);
+      total += num[j];
+    }
+    const int most = warp_max(total);
+    const int ne_h = ne;  // vertical lines: the corners found on the horizontal ones count once
+    for (int i0 = 0; i0 < most; i0 += G) {
+      const int i = i0 + me.l;
+      bool found = false;
+      int kind = 0, m = 0, k = 0, j = 0;
+      if (i < total) {
+        j = i < num[0] ? 0 : i < num[0] + num[1] ? 1 : 2;
+        const int line = i - (j > 0 ? num[0] : 0) - (j > 1 ? num[1] : 0) + (j == 0 ? first[0] : j == 1 ? first[1] : first[2]);
+        const int u = j, w = j == 2 ? 0 : j + 1;
+        const bool fwd = (u == 0 ? C.id[0] : u == 1 ? C.id[1] : C.id[2]) < (w == 0 ? C.id[0] : w == 1 ? C.id[1] : C.id[2]);
+        const int pi = fwd ? u : w, qi = fwd ? w : u;
+        const R3Split px = pi == 0 ? S.x[0] : pi == 1 ? S.x[1] : S.x[2], py = pi == 0 ? S.y[0] : pi == 1 ? S.y[1] : S.y[2];
+        const R3Split qx = qi == 0 ? S.x[0] : qi == 1 ? S.x[1] : S.x[2], qy = qi == 0 ? S.y[0] : qi == 1 ? S.y[1] : S.y[2];
+        const float dxf = r3_fdiff(qx, px), dyf = r3_fdiff(qy, py), D = fmaxf(fabsf(dxf), fabsf(dyf));
+        const float sl = vert ? __fdiv_rn(dyf, dxf) : __fdiv_rn(dxf, dyf);
+        const R3Split& pc = vert ? px : py;  // across the line, and along it
+        const R3Split& pl = vert ? py : px;
+        const float hp = r3_i2f((int)(line - pc.i)) - 0.5f;
+        const float z0 = __fadd_rn(pl.f, __fmul_rn(__fsub_rn(hp, pc.f), sl));
+        const float z = __fadd_rn(z0, 0.5f);
+        const int zi = r3_ffloor(z);
+        const float fr = __fsub_rn(z, r3_i2f(zi)), T = r3_cross_tol(D, sl, z0);
+        i64 jj;
+        bool corner = false;
+        if (fr > T && fr < 1.0f - T) {
+          jj = pl.i + zi;
+        } else {
+          const double2 P = pi == 0 ? C.K[0] : pi == 1 ? C.K[1] : C.K[2], Q = qi == 0 ? C.K[0] : qi == 1 ? C.K[1] : C.K[2];
+          r3_cross_exact(P, Q, (double)line - 0.5, vert, &jj, &corner);
+        }
+        m = vert ? line : (int)jj, k = vert ? (int)jj : line;
+        if (corner) {
+          const bool hz = py.fx == qy.fx && py.inexact == qy.inexact && (!py.inexact || r3_same(C.K[u].y, C.K[w].y));
+          const bool vt = px.fx == qx.fx && px.inexact == qx.inexact && (!px.inexact || r3_same(C.K[u].x, C.K[w].x));
+          kind = 2;
+          found = r3_corner_event(a, m, k, hz, vt);
+          if (vert)
+            for (int t = 0; t < min(ne_h, R3_LIST); ++t)
+              if (F.jk[t] == (unsigned char)(j << 2 | 2) && F.mk[t].x == m && F.mk[t].y == k) found = false;
+        } else {
+          kind = vert;
+          found = vert ? r3_vb(a, m, k) : r3_hb(a, m, k);
+        }
+      }
+      const u32 bal = me.ballot(found);
+      if (found) {
+        const int at = ne + __popc(bal & me.below());
+        if (at < R3_LIST) F.mk[at] = make_int2(m, k), F.jk[at] = (unsigned char)(j << 2 | kind);
+      }
+      ne += __popc(bal);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) cnt[q] += __popc(me.ballot(found && j == q));
+    }
+    __syncwarp();
+  }
+  return ne;
+}
+
+// the boundary vertices strictly inside the cell, as corner ids y (W+1) + x in
+// id order in F.ins (R3_MAXI at most); their number, the same in every lane
+template <int G>
+SBMT_DEV int r3_inside_g(const R3Args& a, const R3Cell& C, const R3Geo2& S, bool live, const GLane<G>& me, R3Found& F) {
+  // rows strictly between the extreme corners, columns through or between them
+  int cy0 = 0, cx0 = 0, rows = 0, cols = 0;
+  if (live) {
+    R3Split lo = S.y[0], hi = S.y[0];
+#pragma unroll
+    for (int q = 1; q < 3; ++q) {
+      if (S.y[q].fx < lo.fx) lo = S.y[q];
+      if (S.y[q].fx > hi.fx || (S.y[q].fx == hi.fx && S.y[q].inexact)) hi = S.y[q];
+    }
+    rows = r3_lines(lo, hi, a.H, &cy0);
+    lo = S.x[0], hi = S.x[0];
+#pragma unroll
+    for (int q = 1; q < 3; ++q) {
+      if (S.x[q].fx < lo.fx) lo = S.x[q];
+      if (S.x[q].fx > hi.fx || (S.x[q].fx == hi.fx && S.x[q].inexact)) hi = S.x[q];
+    }
+    cols = r3_lines(lo, hi, a.W, &cx0, true);
+  }
+  const int total = rows * cols, most = warp_max(total);
+  int n = 0;
+  for (int i0 = 0; i0 < most; i0 += G) {
+    const int i = i0 + me.l;
+    bool inside = false;
+    int cy = 0, cx = 0;
+    if (i < total) {
+      cy = cy0 + i / cols, cx = cx0 + i % cols;
+      if (r3_is_vertex(r3_cmask(a, cx, cy))) {
+        const double c0 = (double)cy - 0.5;
+        bool lt[3], gt[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) lt[q] = r3_lt(S.y[q], cy), gt[q] = r3_gt(S.y[q], cy);
+        // inside when one chord end is below the corner and the other above
+        bool some_below = false, some_above = false;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          if (!lt[q] && !gt[q]) some_below |= r3_lt(S.x[q], cx), some_above |= r3_gt(S.x[q], cx);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const int u = j, v = j == 2 ? 0 : j + 1;
+          if (!((lt[u] && gt[v]) || (lt[v] && gt[u]))) continue;
+          const bool fwd = C.id[u] < C.id[v];
+          const R3Split &px = fwd ? S.x[u] : S.x[v], &py = fwd ? S.y[u] : S.y[v];
+          const R3Split &qx = fwd ? S.x[v] : S.x[u], &qy = fwd ? S.y[v] : S.y[u];
+          const float dxf = r3_fdiff(qx, px), dyf = r3_fdiff(qy, py), sl = __fdiv_rn(dxf, dyf);
+          const float hP = r3_i2f((int)(cy - py.i)) - 0.5f;
+          const float w = __fadd_rn(px.f, __fmul_rn(__fsub_rn(hP, py.f), sl));
+          const float T = r3_cross_tol(fmaxf(fabsf(dxf), fabsf(dyf)), sl, w), h = r3_i2f((int)(cx - px.i)) - 0.5f;
+          if (__fsub_rn(h, w) > T) some_below = true;
+          else if (__fsub_rn(w, h) > T) some_above = true;
+          else {
+            const int o = r3_end_cmp_exact(C, 3 + j, cx, c0);
+            some_below |= o < 0, some_above |= o > 0;
+          }
+        }
+        inside = some_below && some_above;
+      }
+    }
+    const u32 bal = me.ballot(inside);
+    if (inside) {
+      const int at = n + __popc(bal & me.below());
+      if (at < R3_MAXI) F.ins[at] = (u32)cy * (u32)(a.W + 1) + (u32)cx;
+    }
+    n += __popc(bal);
+  }
+  __syncwarp();
+  return n;
+}
+
+// the other cells beside the cell's edges with events (need: bit j): -1 on the
+// outer boundary, -2 when more than one other cell has the edge; the lanes
+// look at the cells around one end
+template <int G>
+SBMT_DEV void r3_neighbours(const R3Args& a, u32 c, const R3Cell& C, int need, const GLane<G>& me, int (&nb)[3]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int u = C.id[j], w = C.id[j == 2 ? 0 : j + 1];
+    u32 e0 = 0, e1 = 0;
+    if ((need >> j) & 1) e0 = a.vptr[u], e1 = a.vptr[u + 1];
+    const int most = warp_max((int)(e1 - e0));
+    int found = -1;
+    for (int i0 = 0; i0 < most; i0 += G) {
+      const u32 e = e0 + (u32)(i0 + me.l);
+      int c2 = -1;
+      if (e < e1) {
+        c2 = (int)a.inc[e];
+        const int* t = a.ttri + 3 * (i64)c2;
+        if ((u32)c2 == c || !(t[0] == w || t[1] == w || t[2] == w)) c2 = -1;
+      }
+      const u32 bal = me.ballot(c2 >= 0);
+      const int got = __shfl_sync(0xffffffffu, c2, me.base + (bal ? __ffs(bal) - 1 : 0));
+      if (bal) found = found != -1 || (bal & (bal - 1)) ? -2 : got;
+    }
+    nb[j] = found;
+  }
 }
 
 // events of the edge from P (its lower-id end) to Q, in order from P, with
@@ -633,10 +862,27 @@ __global__ void __launch_bounds__(256) k_r3_screen(R3Args a) {
   }
 }
 
+// The lists of the cut cells, by node count: at most 8 and at most 16 from the
+// two ends of cutl, at most 32 and above from the two ends of glist, and those
+// of at most 32 nodes without a record in ovl; ncls[q] is the length of list q.
+// Lists 0 to 2 hold records' places, the others cells.
+SBMT_DEV u32* r3_list(const R3Args& a, int q, u32 i) {
+  u32* base = q < 2 ? a.cutl : q < 4 ? a.glist : a.ovl;
+  return (q & 1) ? base + (a.nt - 1 - i) : base + i;
+}
+// A cut cell's record, in 64-bit words of rec: {cell, neighbour of edge 0},
+// {neighbours of edges 1 and 2} (-1: none), {counts: events per edge and inside
+// vertices, a byte each}, then the events' and the inside vertices' entries.
+// The room is one word per cell of the mesh (a few percent of them are cut);
+// a cell for which it is used up is listed without a record.
+constexpr int R3_HEAD = 3;
+
 // the candidates: events on the edges, inside vertices, the cells beside
-// the edges that carry events
+// the edges that carry events.  (Eight lanes a candidate, as in k_r3_cells,
+// took 0.99 ms against 0.54: here the cells are alike, and what every lane
+// needs is computed once.)
 __global__ void __launch_bounds__(128) k_r3_count(R3Args a) {
-  R3Ev ev[R3_MAXE];
+  u64 ev[3 * R3_MAXE + R3_MAXI];
   const u32 n = *a.ncand;
   for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
     const u32 c = a.cand[q];
@@ -646,31 +892,52 @@ __global__ void __launch_bounds__(128) k_r3_count(R3Args a) {
     for (int j = 0; j < 3; ++j) {
       const int u = j, w = j == 2 ? 0 : j + 1;
       const bool fwd = C.id[u] < C.id[w];
-      cnt[j] = r3_edge_count(a, fwd ? C.K[u] : C.K[w], fwd ? C.K[w] : C.K[u], ev);
+      cnt[j] = r3_edge_count(a, fwd ? C.K[u] : C.K[w], fwd ? C.K[w] : C.K[u], j, ev + ne);
       if (cnt[j] < 0) bad = true;
       else ne += cnt[j];
     }
-    const int ni = bad ? 0 : r3_inside(a, C, nullptr);
+    const int ni = bad ? 0 : r3_inside(a, C, ev + ne);
     if (bad || ni == -1 || 3 + ne + ni > R3_MAXN) {
       atomicOr(a.err, R3_CAPACITY);
     } else if (ni < 0) {
       atomicOr(a.err, R3_GEOMETRY);
     } else if (ne + ni > 0) {
-      // the cut cells' list for the emission, one atomic per group of lanes
       const unsigned act = __activemask();
       const int lane = threadIdx.x & 31, lead = __ffs(act) - 1;
-      u32 base = 0;
-      if (lane == lead) base = atomicAdd(a.ncut, (u32)__popc(act));
-      base = __shfl_sync(act, base, lead);
-      a.cutl[base + __popc(act & ((1u << lane) - 1u))] = c;
+      if (lane == lead) atomicAdd(a.ncut, (u32)__popc(act));
+      int nb[3] = {-1, -1, -1};
       u32 nown = 0, own3 = 0;
       for (int j = 0; j < 3; ++j) {
         if (cnt[j] == 0) continue;
-        const int nb = r3_neighbour(a, c, C, j);
-        if (nb == -2) atomicOr(a.err, R3_GEOMETRY);
-        if (nb < 0 || (u32)nb > c) nown += (u32)cnt[j], own3 |= (u32)cnt[j] << (8 * j);
+        nb[j] = r3_neighbour(a, c, C, j);
+        if (nb[j] == -2) atomicOr(a.err, R3_GEOMETRY);
+        if (nb[j] < 0 || (u32)nb[j] > c) nown += (u32)cnt[j], own3 |= (u32)cnt[j] << (8 * j);
       }
       a.ntri[c] = (u32)(2 * ni + 3 + ne - 2), a.nin[c] = (u32)ni, a.nown[c] = nown, a.own3[c] = own3;
+      // the record, and the cell's place in its list: one atomic per list and
+      // group of lanes
+      const int nodes = 3 + ne + ni;
+      int cls = nodes <= 8 ? 0 : nodes <= 16 ? 1 : nodes <= 32 ? 2 : 3;
+      u32 item = c;
+      if (cls < 3) {
+        const u32 words = (u32)(R3_HEAD + ne + ni);
+        const unsigned long long at = atomicAdd(a.nrec, (unsigned long long)words);
+        if (at + words <= a.nt) {
+          u64* r = a.rec + at;
+          r[0] = (u64)c | (u64)(u32)nb[0] << 32, r[1] = (u64)(u32)nb[1] | (u64)(u32)nb[2] << 32;
+          r[2] = (u64)(cnt[0] | cnt[1] << 8 | cnt[2] << 16 | ni << 24);
+          for (int t = 0; t < ne + ni; ++t) r[R3_HEAD + t] = ev[t];
+          item = (u32)at;
+        } else {
+          cls = 4;
+        }
+      }
+      const unsigned peers = __match_any_sync(__activemask(), cls);
+      const int first = __ffs(peers) - 1;
+      u32 base = 0;
+      if (lane == first) base = atomicAdd(a.ncls + cls, (u32)__popc(peers));
+      base = __shfl_sync(peers, base, first);
+      *r3_list(a, cls, base + __popc(peers & ((1u << lane) - 1u))) = item;
     }
   }
 }
@@ -866,189 +1133,6 @@ SBMT_DEV unsigned short r3_label(const R3Args& a, double2 p, double2 q, double2 
   return l == R3_OUTSIDE ? (unsigned short)0xFFFF : (unsigned short)l;
 }
 
-// Tier-T: the key and rotation of the cell in the table's regime, or key 0
-SBMT_DEV int r3_tier_t(const R3Local& L, int* sigma_out) {
-  if (L.ni > 1) return 0;
-  int deg[R3_MAXN];
-  for (int w = 0; w < L.n; ++w) deg[w] = 0;
-  for (int t = 0; t < L.np; ++t) {
-    if (L.pa[t] < 3 || L.pb[t] < 3) return 0;
-    deg[L.pa[t]]++, deg[L.pb[t]]++;
-  }
-  for (int w = 3; w < 3 + L.ne; ++w)
-    if (deg[w] != 1) return 0;
-  const int P = 3 + L.ne;
-  if (L.ni == 0 && !(L.np == 1 || L.np == 2)) return 0;
-  if (L.ni == 1)
-    for (int t = 0; t < L.np; ++t)
-      if (L.pa[t] != P && L.pb[t] != P) return 0;
-  auto edge_of = [&](int w) -> int {
-    int k = w - 3;
-    for (int j = 0; j < 3; ++j) {
-      if (k < L.nev[j]) return j;
-      k -= L.nev[j];
-    }
-    return -1;
-  };
-  int dir = 0;
-  if (L.ni == 0 && L.np == 2) {
-    int X[2];
-    for (int c = 0; c < 2; ++c) {
-      const int ea = edge_of(L.pa[c]), eb = edge_of(L.pb[c]);
-      if (ea == eb) return -1;  // a chord with both ends on one edge
-      X[c] = eb == (ea + 1) % 3 ? eb : ea;
-    }
-    if (X[0] == X[1]) {  // nested chords at corner X
-      const int ein = (X[0] + 2) % 3, eout = X[0];
-      int near = -1, best = -1;
-      for (int c = 0; c < 2; ++c)
-        for (int end = 0; end < 2; ++end) {
-          const int w = end ? L.pb[c] : L.pa[c];
-          if (edge_of(w) == ein && w > best) best = w, near = c;
-        }
-      dir = (edge_of(L.pa[near]) == ein && edge_of(L.pb[near]) == eout) ? 1 : 0;
-    }
-  }
-  const int st = L.ni == 1 ? 1 : 0, n0 = L.nev[0], n1 = L.nev[1], n2 = L.nev[2];
-  const int cr0 = (st << 10) | (n0 << 7) | (n1 << 4) | (n2 << 1) | dir;
-  const int cr1 = (st << 10) | (n1 << 7) | (n2 << 4) | (n0 << 1) | dir;
-  const int cr2 = (st << 10) | (n2 << 7) | (n0 << 4) | (n1 << 1) | dir;
-  int best = cr0, sigma = 0;
-  if (cr1 < best) best = cr1, sigma = 1;
-  if (cr2 < best) best = cr2, sigma = 2;
-  for (int k = 0; k < NKEYS; ++k)
-    if (g_keys.code[k] == best) {
-      *sigma_out = sigma;
-      return k + 1;
-    }
-  return -1;
-}
-
-// ---------------------------------------------------------------------------
-// the greedy rule for a small cell (n <= R3_SMALL nodes) in one thread:
-// candidate pairs by (squared length rounded to single precision, u, w),
-// each kept when its open segment holds no node and it crosses no kept edge;
-// the faces (3-cycles with no node inside, smallest index first,
-// counter-clockwise) in sorted order.  Returns the face count, -1 past the
-// limits.
-// ---------------------------------------------------------------------------
-constexpr int R3_SMALL = 12;
-
-// Orientation signs with a single-precision filter.  The nodes' coordinates
-// relative to the first corner, rounded once to float, are within
-// 2^-24 M (1 + 2^-23) of the exact differences (M: the largest of them);
-// a float orientation of three such points is then within 48 2^-24 M^2 of
-// the exact orientation of the doubles, and the double-precision formula
-// within 32 2^-53 M^2 of it.  Outside 80 2^-24 M^2 the float sign is the
-// sign the double formula gives; inside it the double formula decides.
-struct R3Filt {
-  float2 l[R3_SMALL];
-  float T;
-};
-SBMT_DEV void r3_filt_init(const R3Local& L, R3Filt& F) {
-  float M = 0.0f;
-  for (int k = 0; k < L.n; ++k) {
-    F.l[k] = make_float2(__double2float_rn(dsb(L.v[k].x, L.v[0].x)), __double2float_rn(dsb(L.v[k].y, L.v[0].y)));
-    M = fmaxf(M, fmaxf(fabsf(F.l[k].x), fabsf(F.l[k].y)));
-  }
-  F.T = 80.0f * 5.9604645e-8f * M * M * 1.0001f;  // 80 2^-24 M^2, rounded up
-}
-__device__ __noinline__ int r3_osgn_exact(const R3Local& L, int p, int q, int r) {
-  return r3_sgn(r3_orient(L.v[p], L.v[q], L.v[r]));
-}
-SBMT_DEV int r3_osgn(const R3Local& L, const R3Filt& F, int p, int q, int r) {
-  const float2 a = F.l[p], b = F.l[q], c = F.l[r];
-  const float o = __fsub_rn(__fmul_rn(__fsub_rn(b.x, a.x), __fsub_rn(c.y, a.y)),
-                            __fmul_rn(__fsub_rn(b.y, a.y), __fsub_rn(c.x, a.x)));
-  if (o > F.T) return 1;
-  if (o < -F.T) return -1;
-  return r3_osgn_exact(L, p, q, r);  // within the filter's bound: the double formula
-}
-
-SBMT_DEV int r3_greedy_small(const R3Local& L, int* face) {
-  const int n = L.n;
-  R3Filt F;
-  r3_filt_init(L, F);
-  unsigned short adj[R3_SMALL];
-  unsigned char ea[3 * R3_SMALL], eb[3 * R3_SMALL];
-  int ne = 0;
-  for (int w = 0; w < n; ++w) adj[w] = 0;
-  auto add = [&](int p, int q) {
-    if ((adj[p] >> q) & 1) return;
-    adj[p] |= (unsigned short)(1 << q), adj[q] |= (unsigned short)(1 << p);
-    if (ne < 3 * R3_SMALL) ea[ne] = (unsigned char)p, eb[ne] = (unsigned char)q;
-    ++ne;
-  };
-  for (int t = 0; t < L.np; ++t) add(L.pa[t], L.pb[t]);
-  {
-    int prev = 0, b = 3;
-    for (int j = 0; j < 3; ++j) {
-      if (j) add(prev, j), prev = j;
-      for (int t = 0; t < L.nev[j]; ++t) add(prev, b + t), prev = b + t;
-      b += L.nev[j];
-    }
-    add(prev, 0);
-  }
-  // candidates, insertion-sorted by (key, u, w)
-  float key[R3_SMALL * (R3_SMALL - 1) / 2];
-  unsigned char pr[R3_SMALL * (R3_SMALL - 1) / 2];
-  int nc = 0;
-  for (int u = 0; u < n; ++u)
-    for (int w = u + 1; w < n; ++w) {
-      if (((adj[u] >> w) & 1) || (L.on_edge[u] & L.on_edge[w])) continue;
-      const double dx = dsb(L.v[w].x, L.v[u].x), dy = dsb(L.v[w].y, L.v[u].y);
-      const float k = __double2float_rn(dad(dml(dx, dx), dml(dy, dy)));
-      const unsigned char code = (unsigned char)(u << 4 | w);
-      int t = nc++;
-      while (t > 0 && (key[t - 1] > k || (key[t - 1] == k && pr[t - 1] > code))) key[t] = key[t - 1], pr[t] = pr[t - 1], --t;
-      key[t] = k, pr[t] = code;
-    }
-  for (int r = 0; r < nc; ++r) {
-    const int u = pr[r] >> 4, w = pr[r] & 15;
-    const double2 pu = L.v[u], pw = L.v[w];
-    const double ex = dsb(pw.x, pu.x), ey = dsb(pw.y, pu.y), len2 = dad(dml(ex, ex), dml(ey, ey));
-    bool bad = false;
-    for (int k = 0; k < n && !bad; ++k) {
-      if (k == u || k == w || r3_osgn(L, F, u, w, k) != 0) continue;
-      const double t = dad(dml(dsb(L.v[k].x, pu.x), ex), dml(dsb(L.v[k].y, pu.y), ey));
-      if (t > 0.0 && t < len2) bad = true;
-    }
-    for (int t = 0; t < ne && t < 3 * R3_SMALL && !bad; ++t) {
-      const int p = ea[t], q = eb[t];
-      if (p == u || p == w || q == u || q == w) continue;
-      const int o1 = r3_osgn(L, F, u, w, p), o2 = r3_osgn(L, F, u, w, q);
-      if (o1 * o2 >= 0) continue;
-      const int o3 = r3_osgn(L, F, p, q, u), o4 = r3_osgn(L, F, p, q, w);
-      if (o3 * o4 < 0) bad = true;
-    }
-    if (!bad) add(u, w);
-  }
-  if (ne > 3 * R3_SMALL) return -1;
-  int nf = 0;
-  for (int p = 0; p < n; ++p)
-    for (int q = p + 1; q < n; ++q) {
-      if (!((adj[p] >> q) & 1)) continue;
-      for (int r = q + 1; r < n; ++r) {
-        if (!((adj[p] >> r) & 1) || !((adj[q] >> r) & 1)) continue;
-        const int o = r3_osgn(L, F, p, q, r);
-        if (o == 0) continue;
-        bool empty = true;
-        for (int k = 0; k < n && empty; ++k) {
-          if (k == p || k == q || k == r) continue;
-          if (r3_osgn(L, F, p, q, k) == o && r3_osgn(L, F, q, r, k) == o && r3_osgn(L, F, r, p, k) == o)
-            empty = false;
-        }
-        if (!empty) continue;
-        if (nf == 2 * R3_SMALL) return -1;
-        const int f = o > 0 ? (p << 12 | q << 6 | r) : (p << 12 | r << 6 | q);
-        int t = nf++;
-        while (t > 0 && face[t - 1] > f) face[t] = face[t - 1], --t;
-        face[t] = f;
-      }
-    }
-  return nf;
-}
-
 // ---------------------------------------------------------------------------
 // the cells left as they are: uncut cells of one label, labelled by their
 // pixel box, and candidates the boundary only touches (at a corner or along
@@ -1074,110 +1158,520 @@ __global__ void __launch_bounds__(256) k_r3_emit_uncut(R3Args a) {
 }
 
 // ---------------------------------------------------------------------------
-// the cut cells (k_r3_count's list): Tier-T cells take their template;
-// Tier-G cells are queued (those over R3_SMALL nodes
-// flagged) for the greedy kernels, so that this kernel's warps stay on the
-// short template path and the greedy runs in warps of Tier-G cells only
+// the cut cells of at most 32 nodes: a group of 8, 16 or 32 lanes each builds
+// the local boundary graph and takes the template of a Tier-T cell or the
+// greedy rule (sbmt_greedy.cuh) of a Tier-G one.  The double formulas run one
+// event, candidate or piece per lane; positions on pixel lines, orientations
+// and centroid labels are decided in fixed point or single precision where a
+// bound allows.
 // ---------------------------------------------------------------------------
-constexpr u32 R3_BIG = 0x80000000u;  // a queued cell over R3_SMALL nodes (cell ids stay below 2^31)
-
-struct R3EvBuf {
-  R3Ev e[3][R3_MAXE];
-  SBMT_DEV R3Ev* operator[](int j) { return e[j]; }
+template <int G>
+struct R3State {
+  GCell<G> c;
+  R3Found F;                  // a cell without a record
+  unsigned char ix[3];        // corners: whether x, y are off the fixed-point grid
+  unsigned char tj[G];        // the events as found: edge << 2 | kind, pixel indices
+  int2 tmk[G];
+  double vx[G], vy[G];  // the nodes: corners, events counter-clockwise, inside vertices
+  i64 X[G], Y[G];       // floor(v 2^36)
+  double s[G];          // while ordering: the events' parameters along their edges
+  u32 gid[G];
+  int2 mk[G];             // events: pixel indices and kind, in node order
+  unsigned char kind[G];
+  unsigned char pa[3 * G], pb[3 * G];  // the pieces
 };
 
-__global__ void __launch_bounds__(128) k_r3_emit(R3Args a) {
-  R3EvBuf ev;
-  R3Local L;
-  const u32 n = *a.ncut;
-  for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-    const u32 c = a.cutl[q];
-    const R3Cell C = r3_load(a, c);
-    const u32 t0 = a.toff[c];
-    int3* tri = reinterpret_cast<int3*>(a.tri);
-    const u32 e = r3_build(a, c, C, L, ev, true);
-    if (e) {
-      atomicOr(a.err, e);
-      continue;
+// the geometry for the greedy rule: the filter decides outside its band, and
+// the double formula of each test, taken as the rule states it, inside.  The
+// float coordinates are within 2^-24 M + 2^-35 of the differences from the
+// first corner (M: the largest), so a float determinant is within
+// 48 2^-24 M^2 + 8 2^-35 M of the doubles' exact one and the double formula
+// within 32 2^-53 M^2 of it.
+template <int G>
+struct R3Geo {
+  const R3State<G>* s;
+  float T;
+  SBMT_DEV float tol() const { return T; }
+  SBMT_DEV double2 pt(int k) const { return make_double2(s->vx[k], s->vy[k]); }
+  SBMT_DEV bool resolve(int, int, int, int*) const { return false; }
+  SBMT_DEV int late(int u, int v, int w) const { return r3_sgn(r3_orient(pt(u), pt(v), pt(w))); }
+  SBMT_DEV bool between(int u, int w, int k) const {
+    const double2 pu = pt(u), pw = pt(w), pk = pt(k);
+    const double ex = dsb(pw.x, pu.x), ey = dsb(pw.y, pu.y), len2 = dad(dml(ex, ex), dml(ey, ey));
+    const double t = dad(dml(dsb(pk.x, pu.x), ex), dml(dsb(pk.y, pu.y), ey));
+    return t > 0.0 && t < len2;
+  }
+  SBMT_DEV float key(int u, int w, int) const {
+    const double dx = dsb(s->vx[w], s->vx[u]), dy = dsb(s->vy[w], s->vy[u]);
+    return __double2float_rn(dad(dml(dx, dx), dml(dy, dy)));
+  }
+  SBMT_DEV bool less(float kx, unsigned short x, int, float ky, unsigned short y, int) const {
+    return kx < ky || (kx == ky && x < y);
+  }
+};
+
+// r3_at_corner through the fixed-point value
+SBMT_DEV bool r3_at_corner36(double t, i64* idx) {
+  bool inexact;
+  const i64 f = r3_fix36(t, &inexact), fl = f >> 36, fr = f & ((1ll << 36) - 1);
+  constexpr i64 HALF = 1ll << 35;
+  *idx = fr < HALF ? fl : fl + 1;
+  return fr == HALF && !inexact;
+}
+
+// the label of the pixel holding ((x1 + x2) + x3) / 3, from the fixed-point
+// values: floor((X1 + X2 + X3) / 3 + 1/2) is the double formula's unless the
+// sum is within a bound of a pixel line (three floors, 3 2^-36 below the exact
+// sum at most; the double formula's roundings, below 2^-26 px at 2^24)
+template <int G>
+SBMT_DEV unsigned short r3_label36(const R3Args& a, const R3State<G>& s, int p, int q, int r) {
+  constexpr i64 ONE3 = 3ll << 36, BAND = 1ll << 14;  // 3 px; 2^-22 px
+  i64 at[2];
+  bool near = false;
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    const i64 sum = (d ? s.Y[p] + s.Y[q] + s.Y[r] : s.X[p] + s.X[q] + s.X[r]) + (ONE3 >> 1);
+    const i64 f = (sum >= 0 ? sum : sum - (ONE3 - 1)) / ONE3, rem = sum - f * ONE3;
+    at[d] = f;
+    near |= rem < BAND || rem > ONE3 - BAND;
+  }
+  if (near)
+    return r3_label(a, make_double2(s.vx[p], s.vy[p]), make_double2(s.vx[q], s.vy[q]), make_double2(s.vx[r], s.vy[r]));
+  const int l = r3_px(a, at[0], at[1]);
+  return l == R3_OUTSIDE ? (unsigned short)0xFFFF : (unsigned short)l;
+}
+
+// Tier-T: the key and rotation of the cell in the table's regime, or key 0
+// (-1: a graph outside the table where none can be)
+template <int G>
+SBMT_DEV int r3_tier_t(const R3State<G>& s, int ni, int ne, int np, int n0, int n1, int n2, int* sigma_out) {
+  if (ni > 1 || np > 8) return 0;
+  const int P = 3 + ne;
+  u32 once = 0, twice = 0;
+  for (int t = 0; t < np; ++t) {
+    if (s.pa[t] < 3 || s.pb[t] < 3) return 0;
+    const u32 x = 1u << s.pa[t], y = 1u << s.pb[t];
+    twice |= once & x, once |= x;
+    twice |= once & y, once |= y;
+  }
+  const u32 evs = ((1u << ne) - 1u) << 3;
+  if ((once & evs) != evs || (twice & evs)) return 0;
+  if (ni == 0 && !(np == 1 || np == 2)) return 0;
+  if (ni == 1)
+    for (int t = 0; t < np; ++t)
+      if (s.pa[t] != P && s.pb[t] != P) return 0;
+  auto edge_of = [&](int w) -> int { return w - 3 < n0 ? 0 : w - 3 < n0 + n1 ? 1 : w - 3 < n0 + n1 + n2 ? 2 : -1; };
+  int dir = 0;
+  if (ni == 0 && np == 2) {
+    int X[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int ea = edge_of(s.pa[c]), eb = edge_of(s.pb[c]);
+      if (ea == eb) return -1;  // a chord with both ends on one edge
+      X[c] = eb == (ea + 1) % 3 ? eb : ea;
     }
-    const int nt = 2 * L.ni + 3 + L.ne - 2;
-    if ((u32)nt != a.toff[c + 1] - t0) {
-      atomicOr(a.err, R3_COUNT);
-      continue;
+    if (X[0] == X[1]) {  // nested chords at corner X
+      const int ein = (X[0] + 2) % 3, eout = X[0];
+      int near = -1, best = -1;
+      for (int c = 0; c < 2; ++c)
+        for (int end = 0; end < 2; ++end) {
+          const int w = end ? s.pb[c] : s.pa[c];
+          if (edge_of(w) == ein && w > best) best = w, near = c;
+        }
+      dir = (edge_of(s.pa[near]) == ein && edge_of(s.pb[near]) == eout) ? 1 : 0;
     }
-    int sigma = 0;
-    const int key = r3_tier_t(L, &sigma);
-    if (key < 0) {
-      atomicOr(a.err, R3_GEOMETRY);
-      continue;
+  }
+  const int st = ni == 1 ? 1 : 0;
+  const int cr0 = (st << 10) | (n0 << 7) | (n1 << 4) | (n2 << 1) | dir;
+  const int cr1 = (st << 10) | (n1 << 7) | (n2 << 4) | (n0 << 1) | dir;
+  const int cr2 = (st << 10) | (n2 << 7) | (n0 << 4) | (n1 << 1) | dir;
+  int best = cr0, sigma = 0;
+  if (cr1 < best) best = cr1, sigma = 1;
+  if (cr2 < best) best = cr2, sigma = 2;
+  for (int k = 0; k < NKEYS; ++k)
+    if (g_keys.code[k] == best) {
+      *sigma_out = sigma;
+      return k + 1;
     }
-    if (key == 0) {
-      // one queue slot per lane, one atomic per group of lanes here
-      const unsigned act = __activemask();
-      const int lane = threadIdx.x & 31, lead = __ffs(act) - 1;
-      u32 base = 0;
-      if (lane == lead) base = atomicAdd(a.ng, (u32)__popc(act));
-      base = __shfl_sync(act, base, lead);
-      a.glist[base + __popc(act & ((1u << lane) - 1u))] = c | (L.n > R3_SMALL ? R3_BIG : 0u);
-      continue;
-    }
-    const unsigned long long w = g_keys.tris[(key - 1) * 3 + sigma];
-    const unsigned short code =
-        (unsigned short)((L.mask & 15) | (sigma << 4) | (key << 6) | (L.klass << 12));
-    for (int k = 0; k < nt; ++k) {
-      int q3[3];
-      for (int u = 0; u < 3; ++u) {
-        const int l = tri_label(w, k, u);
-        q3[u] = l == 7 ? 3 + L.ne : l;
+  return -1;
+}
+
+// LIST: which list; REC: whether its cells come with the count pass's records
+template <int G, int LIST, bool REC>
+__global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
+  constexpr int C_ = 64 / G;
+  __shared__ R3State<G> sm[C_];
+  const GLane<G> me;
+  R3State<G>& s = sm[threadIdx.x / G];
+  const u32 total = a.ncls[LIST];
+  u32 ngc = 0, ngt = 0;
+  for (u32 q = blockIdx.x * C_ + threadIdx.x / G;; q += gridDim.x * C_) {
+    bool live = q < total;
+    if (!__any_sync(0xffffffffu, live)) break;
+    u32 err = 0, c = 0;
+    int cnt[3] = {0, 0, 0}, nb[3] = {-1, -1, -1}, ne, ni;
+    u64 entry = 0;  // this lane's event or inside vertex
+    auto put = [&](int v, double x, double y, u32 gid, int em) {
+      bool ix, iy;
+      s.vx[v] = x, s.vy[v] = y, s.X[v] = r3_fix36(x, &ix), s.Y[v] = r3_fix36(y, &iy);
+      s.gid[v] = gid, s.c.em[v] = (unsigned char)em;
+      if (v < 3) s.ix[v] = (unsigned char)((ix ? 1 : 0) | (iy ? 2 : 0));
+    };
+    if (REC) {
+      const u64* r = a.rec + (live ? *r3_list(a, LIST, q) : 0u);
+      if (live) {
+        const u64 h0 = r[0], h1 = r[1], h2 = r[2];
+        c = (u32)h0, nb[0] = (int)(u32)(h0 >> 32), nb[1] = (int)(u32)h1, nb[2] = (int)(u32)(h1 >> 32);
+        cnt[0] = (int)(h2 & 255u), cnt[1] = (int)((h2 >> 8) & 255u), cnt[2] = (int)((h2 >> 16) & 255u);
+        ni = (int)((h2 >> 24) & 255u);
+      } else {
+        ni = 0;
       }
-      tri[t0 + k] = make_int3((int)L.gid[q3[0]], (int)L.gid[q3[1]], (int)L.gid[q3[2]]);
-      a.label[t0 + k] = r3_label(a, L.v[q3[0]], L.v[q3[1]], L.v[q3[2]]);
-      a.code[t0 + k] = code;
+      ne = cnt[0] + cnt[1] + cnt[2];
+      if (live && me.l < ne + ni) entry = r[R3_HEAD + me.l];
+    } else {
+      c = live ? *r3_list(a, LIST, q) : 0u;
+      const R3Cell C = r3_load_k(a, c);
+      R3Geo2 S;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) S.x[t] = r3_split(C.K[t].x), S.y[t] = r3_split(C.K[t].y);
+      ne = r3_events<G>(a, C, S, live, me, s.F, cnt);
+      ni = r3_inside_g<G>(a, C, S, live, me, s.F);
+      r3_neighbours<G>(a, c, C, live ? (cnt[0] > 0) | (cnt[1] > 0) << 1 | (cnt[2] > 0) << 2 : 0, me, nb);
+      if (me.l < ne) {
+        entry = r3_entry(s.F.jk[me.l] >> 2, s.F.jk[me.l] & 3, s.F.mk[me.l].x, s.F.mk[me.l].y);
+      } else if (me.l < ne + ni) {
+        const u32 cid = s.F.ins[me.l - ne];
+        entry = r3_entry(3, 3, (int)(cid % (u32)(a.W + 1)), (int)(cid / (u32)(a.W + 1)));
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (nb[j] == -2) err |= R3_GEOMETRY;
     }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Tier-G cells of at most R3_SMALL nodes: one thread per queued cell, the
-// local graph rebuilt (the event and inside-vertex coordinates are written
-// by k_r3_emit), the greedy rule, the faces written in sorted order
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_r3_gsmall(R3Args a) {
-  R3EvBuf ev;
-  R3Local L;
-  const u32 n = *a.ng;
-  for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-    const u32 c = a.glist[q];
-    if (c & R3_BIG) continue;
-    const R3Cell C = r3_load(a, c);
-    const u32 e = r3_build(a, c, C, L, ev, false);
-    if (e) {
-      atomicOr(a.err, e);
-      continue;
+    const int n = live ? 3 + ne + ni : 0;
+    const u32 t0 = live ? a.toff[c] : 0u, nt = live ? a.toff[c + 1] - t0 : 0u;
+    if (live && (n > G || (u32)(2 * ni + ne + 1) != nt)) err |= R3_COUNT;  // the count pass found others
+    if (err) {
+      if (me.l == 0) atomicOr(a.err, err);
+      live = false;
     }
-    const u32 t0 = a.toff[c];
-    int face[2 * R3_SMALL];
-    const int nf = r3_greedy_small(L, face);
-    if (nf != (int)(a.toff[c + 1] - t0)) {
-      atomicOr(a.err, nf < 0 ? R3_CAPACITY : R3_COUNT);
-      continue;
+    // the corners
+    if (live && me.l < 3) {
+      const int k = me.l, id = a.ttri[3 * (u64)c + (u32)k];
+      const double2 K = reinterpret_cast<const double2*>(a.txy)[id];
+      put(k, K.x, K.y, (u32)id, (1 << k) | (1 << (k == 0 ? 2 : k - 1)));
     }
-    const unsigned short code = (unsigned short)((L.mask & 15) | (63 << 6) | (L.klass << 12));
-    atomicAdd(a.ngtri, (u32)nf);
-    atomicAdd(a.ngsmall, 1u);
+    // the events: one lane each (n <= G), with their position on their edge
+    double ex = 0.0, ey = 0.0, es = 0.0;
+    const int ej = (int)(entry >> 34), ekind = (int)(entry >> 32) & 3;
+    const int2 emk = make_int2((int)(entry & 0xFFFFu), (int)((entry >> 16) & 0xFFFFu));
+    bool fwd = true;
+    const bool isev = live && me.l < ne;
+    if (isev) s.tj[me.l] = (unsigned char)(ej << 2 | ekind), s.tmk[me.l] = emk;
+    __syncwarp();
+    if (isev) {
+      const int w = ej == 2 ? 0 : ej + 1;
+      fwd = (int)s.gid[ej] < (int)s.gid[w];
+      const int pi = fwd ? ej : w, qi = fwd ? w : ej;
+      const double2 P = make_double2(s.vx[pi], s.vy[pi]), Q = make_double2(s.vx[qi], s.vy[qi]);
+      const double dx = dsb(Q.x, P.x), dy = dsb(Q.y, P.y);
+      ex = (double)emk.x - 0.5, ey = (double)emk.y - 0.5;  // a corner; else one of the two from the other
+      if (ekind != 2) {  // one division for either kind
+        const bool v = ekind == 1;
+        const double t = ddv(dml(v ? dsb(ex, P.x) : dsb(ey, P.y), v ? dy : dx), v ? dx : dy);
+        if (v) ey = dad(P.y, t);
+        else ex = dad(P.x, t);
+      }
+      const bool alongx = fabs(dx) >= fabs(dy);
+      es = ddv(alongx ? dsb(ex, P.x) : dsb(ey, P.y), alongx ? dx : dy);
+      s.s[me.l] = es;
+    }
+    __syncwarp();
+    // rank on the edge by (s, kind, k, m); node order runs counter-clockwise
+    if (isev) {
+      int r = 0;
+      for (int t = 0; t < ne; ++t) {
+        if (t == me.l || (s.tj[t] >> 2) != ej) continue;
+        const double f = s.s[t];
+        const int tk = s.tj[t] & 3;
+        const int2 tm = s.tmk[t];
+        r += (f != es ? f < es : tk != ekind ? tk < ekind : tm.y != emk.y ? tm.y < emk.y : tm.x < emk.x) ? 1 : 0;
+      }
+      const int own = ej == 0 ? cnt[0] : ej == 1 ? cnt[1] : cnt[2], other = ej == 0 ? nb[0] : ej == 1 ? nb[1] : nb[2];
+      const int b0 = ej == 0 ? 0 : ej == 1 ? cnt[0] : cnt[0] + cnt[1];
+      const int v = 3 + b0 + (fwd ? r : own - 1 - r);
+      u32 base;
+      if (other < 0 || (u32)other > c) {
+        base = r3_edge_base(a, c, ej) + (u32)r;
+        reinterpret_cast<double2*>(a.xy)[base] = make_double2(ex, ey);
+      } else {
+        const int j2 = r3_edge_in(a, (u32)other, (int)s.gid[ej], (int)s.gid[ej == 2 ? 0 : ej + 1]);
+        if (j2 < 0) err |= R3_GEOMETRY;
+        base = r3_edge_base(a, (u32)other, max(j2, 0)) + (u32)r;
+      }
+      put(v, ex, ey, base, 1 << ej);
+      s.mk[v] = emk, s.kind[v] = (unsigned char)ekind;
+    }
+    // inside vertices
+    if (live && me.l >= ne && me.l < ne + ni) {
+      const u32 id = a.nv + a.ne_total + a.ioff[c] + (u32)(me.l - ne);
+      const int v = 3 + me.l;
+      const double2 p = make_double2((double)emk.x - 0.5, (double)emk.y - 0.5);
+      reinterpret_cast<double2*>(a.xy)[id] = p;
+      put(v, p.x, p.y, id, 0);
+      s.mk[v] = emk, s.kind[v] = 3;
+    }
+    if (me.ballot(err != 0)) {
+      if (err) atomicOr(a.err, err);
+      live = false;
+    }
+    __syncwarp();
+    R3Corner Sx[3], Sy[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+      Sx[t] = R3Corner{s.X[t], (s.ix[t] & 1) != 0}, Sy[t] = R3Corner{s.Y[t], (s.ix[t] & 2) != 0};
+    // the filter's frame
+    float M = 0.0f;
+    if (live && me.l < n) {
+      const float fx = __fmul_rn((float)(s.X[me.l] - s.X[0]), 1.4551915228366852e-11f);
+      const float fy = __fmul_rn((float)(s.Y[me.l] - s.Y[0]), 1.4551915228366852e-11f);
+      s.c.f[me.l] = make_float2(fx, fy);
+      M = fmaxf(fabsf(fx), fabsf(fy));
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    // pieces: horizontal lines by y, then vertical lines by x, one line per
+    // lane: its nodes in order, and a piece between two consecutive ones when
+    // the pixel edge at their middle is a boundary; lower label on the left
+    int np = 0;
+    {
+      int f0[2], nl[2];
+#pragma unroll
+      for (int vert = 0; vert < 2; ++vert) {
+        R3Corner lo = vert ? Sx[0] : Sy[0], hi = lo;
+#pragma unroll
+        for (int t = 1; t < 3; ++t) {
+          const R3Corner v = vert ? Sx[t] : Sy[t];
+          if (v.fx < lo.fx) lo = v;
+          if (v.fx > hi.fx || (v.fx == hi.fx && v.inexact)) hi = v;
+        }
+        nl[vert] = live ? r3_lines(lo, hi, vert ? a.W : a.H, &f0[vert]) : 0;
+      }
+      const int lines = nl[0] + nl[1], most = warp_max(lines);
+      for (int i0 = 0; i0 < most; i0 += G) {
+        const int i = i0 + me.l;
+        const bool on = i < lines, vert = on && i >= nl[0];
+        const int line = on ? (vert ? f0[1] + i - nl[0] : f0[0] + i) : 0;
+        int end[2] = {-1, -1}, nend = 0;
+        u32 ins = 0;
+        if (on) {
+          bool lt[3], gt[3];
+#pragma unroll
+          for (int t = 0; t < 3; ++t) {
+            const R3Corner v{vert ? Sx[t].fx : Sy[t].fx, vert ? Sx[t].inexact : Sy[t].inexact};
+            lt[t] = r3_lt(v, line), gt[t] = r3_gt(v, line);
+          }
+#pragma unroll
+          for (int t = 0; t < 3; ++t)
+            if (!lt[t] && !gt[t]) {
+              if (nend < 2) end[nend] = t;
+              ++nend;
+            }
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const int w = j == 2 ? 0 : j + 1;
+            if (!((lt[j] && gt[w]) || (lt[w] && gt[j]))) continue;
+            int node = -1;
+            const int b0 = 3 + (j > 0 ? cnt[0] : 0) + (j > 1 ? cnt[1] : 0);
+            for (int v = b0 + cnt[j] - 1; v >= b0; --v)  // the first in order
+              if ((s.kind[v] == 2 || s.kind[v] == (vert ? 1 : 0)) && (vert ? s.mk[v].x : s.mk[v].y) == line) node = v;
+            if (nend < 2) end[nend] = node;
+            ++nend;
+          }
+          for (int v = 3 + ne; v < n; ++v)
+            if ((vert ? s.mk[v].x : s.mk[v].y) == line) ins |= 1u << v;
+          if (nend != 2) err |= R3_GEOMETRY, ins = 0, end[0] = end[1] = -1;
+        }
+        auto pos = [&](int v) { return vert ? s.vy[v] : s.vx[v]; };
+        // the ends around the inside vertices (which lie strictly between)
+        int lo = end[0], hi = end[1];
+        if (lo >= 0 && hi >= 0) {
+          if (pos(hi) < pos(lo)) lo = end[1], hi = end[0];
+        } else if (ins && (lo >= 0 || hi >= 0)) {
+          const int v = max(lo, hi);
+          const bool before = pos(v) < pos(__ffs(ins) - 1);
+          lo = before ? v : -1, hi = before ? -1 : v;
+        }
+        auto walk = [&](int at) {
+          int prev = lo, k = 0;
+          u32 rest = ins;
+          while (on) {
+            int cur;
+            if (rest) cur = __ffs(rest) - 1, rest &= rest - 1;
+            else if (hi >= 0) cur = hi, hi = -2;
+            else break;
+            if (prev >= 0) {
+              i64 j;
+              r3_at_corner36(dml(dad(pos(prev), pos(cur)), 0.5), &j);  // at a corner: the pixel edge starting there
+              int l0, l1;
+              if (!vert) l0 = r3_px(a, j, line - 1), l1 = r3_px(a, j, line);
+              else l0 = r3_px(a, line - 1, j), l1 = r3_px(a, line, j);
+              if (l0 != l1) {
+                const bool f = vert ? l0 < l1 : l1 < l0;  // going +x the left side is above, going +y it is -x
+                if (at >= 0 && at + k < 3 * G)
+                  s.pa[at + k] = (unsigned char)(f ? prev : cur), s.pb[at + k] = (unsigned char)(f ? cur : prev);
+                ++k;
+              }
+            }
+            prev = cur;
+          }
+          if (hi == -2) hi = prev;
+          return k;
+        };
+        const int k = walk(-1);
+        int before = k;
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, before, o, G);
+          if (me.l >= o) before += t;
+        }
+        const int sum = __shfl_sync(0xffffffffu, before, G - 1, G);
+        if (k) walk(np + before - k);
+        np += sum;
+      }
+    }
+    if (np + 3 + ne > 3 * G || np > R3_MAXP) err |= R3_CAPACITY;  // (no planar graph on n nodes has as many edges)
+    if (me.ballot(err != 0)) {
+      if (err) atomicOr(a.err, err);
+      live = false;
+    }
+    __syncwarp();
+    // Alg. 1 mask (a corner on a piece sets both its edges, an event its
+    // edge, an edge on a boundary run its own bit, bit 0 an inside vertex)
+    // and the (m, n) class of the first two pieces
+    int mask = 0, klass = 0, key = -1, sigma = 0;
+    if (live) {
+      mask = ni > 0 ? 1 : 0;
+      int pc0 = 0, pc1 = 0;
+      for (int t = 0; t < np; ++t) {
+        const int b = ((int)s.c.em[s.pa[t]] | (int)s.c.em[s.pb[t]]) << 1;
+        mask |= b;
+        if (t == 0) pc0 = __popc(b);
+        if (t == 1) pc1 = __popc(b);
+      }
+      klass = np == 1 ? thm32_class(0, pc0) : np == 2 ? thm32_class(pc0, pc1) : 0;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int w = j == 2 ? 0 : j + 1;
+#pragma unroll
+        for (int vert = 0; vert < 2; ++vert) {
+          // the edge on the pixel line `line`: the pixel edges (g - 1/2, g + 1/2)
+          // it has a stretch of
+          const R3Corner ca = vert ? Sx[j] : Sy[j], cb = vert ? Sx[w] : Sy[w];
+          constexpr i64 HALF = 1ll << 35, ONE = 1ll << 36;
+          if (ca.inexact || cb.inexact || ca.fx != cb.fx || (ca.fx & (ONE - 1)) != HALF) continue;
+          const i64 line = (ca.fx >> 36) + 1;
+          const R3Corner ta = vert ? Sy[j] : Sx[j], tb = vert ? Sy[w] : Sx[w];
+          const bool sw = tb.fx < ta.fx;
+          const i64 e0 = sw ? tb.fx : ta.fx, e1 = sw ? ta.fx : tb.fx;
+          const bool x1 = sw ? ta.inexact : tb.inexact;
+          // g + 1/2 > e0 and g - 1/2 < e1
+          for (i64 g = (e0 + HALF) >> 36; (g << 36) - HALF < e1 + (x1 ? 1 : 0); ++g)
+            if (vert ? r3_vb(a, line, g) : r3_hb(a, g, line)) mask |= 2 << j;
+        }
+      }
+      key = r3_tier_t<G>(s, ni, ne, np, cnt[0], cnt[1], cnt[2], &sigma);
+      if (key < 0) {
+        if (me.l == 0) atomicOr(a.err, R3_GEOMETRY);
+        live = false;
+      }
+    }
     int3* tri = reinterpret_cast<int3*>(a.tri);
-    for (int i = 0; i < nf; ++i) {
-      const int f = face[i], p = f >> 12, r2 = (f >> 6) & 63, s2 = f & 63;
-      tri[t0 + i] = make_int3((int)L.gid[p], (int)L.gid[r2], (int)L.gid[s2]);
-      a.label[t0 + i] = r3_label(a, L.v[p], L.v[r2], L.v[s2]);
-      a.code[t0 + i] = code;
+    if (live && key > 0) {
+      const unsigned long long w = g_keys.tris[(key - 1) * 3 + sigma];
+      const unsigned short code = (unsigned short)((mask & 15) | (sigma << 4) | (key << 6) | (klass << 12));
+      for (int k = me.l; k < (int)nt; k += G) {
+        int q3[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          const int l = tri_label(w, k, u);
+          q3[u] = l == 7 ? 3 + ne : l;
+        }
+        tri[t0 + k] = make_int3((int)s.gid[q3[0]], (int)s.gid[q3[1]], (int)s.gid[q3[2]]);
+        a.label[t0 + k] = r3_label36<G>(a, s, q3[0], q3[1], q3[2]);
+        a.code[t0 + k] = code;
+      }
     }
+    // Tier-G
+    const bool tg = live && key == 0;
+    __syncwarp();
+    if (!__any_sync(0xffffffffu, tg)) continue;
+    // constraints: the pieces and the boundary cycle, each an edge as the
+    // rule's list has it (above 12 nodes the smaller node first)
+    if (tg) {
+      const int v = me.l;
+      if (v < n) {
+        // the cycle's edge from node v to the next, and the one before
+        int next = -1, prev = -1;
+        if (v < 3) {
+          const int own = v == 0 ? cnt[0] : v == 1 ? cnt[1] : cnt[2], b0 = 3 + (v > 0 ? cnt[0] : 0) + (v > 1 ? cnt[1] : 0);
+          const int pk = v == 0 ? cnt[2] : v == 1 ? cnt[0] : cnt[1];
+          next = own ? b0 : (v == 2 ? 0 : v + 1);
+          prev = pk ? (v == 0 ? 2 + ne : b0 - 1) : (v == 0 ? 2 : v - 1);
+        } else if (v < 3 + ne) {
+          const int e = v - 3, k = e < cnt[0] ? 0 : e < cnt[0] + cnt[1] ? 1 : 2;
+          const int b0 = k == 0 ? 0 : k == 1 ? cnt[0] : cnt[0] + cnt[1], own = k == 0 ? cnt[0] : k == 1 ? cnt[1] : cnt[2];
+          next = e + 1 == b0 + own ? (k == 2 ? 0 : k + 1) : v + 1;
+          prev = e == b0 ? k : v - 1;
+        }
+        s.c.adj[v] = next >= 0 ? (1u << next) | (1u << prev) : 0u;
+        if (next >= 0) {
+          const bool sw = n > 12 && next < v;
+          s.c.ce[np + v] = (unsigned short)(sw ? (next << 8) | v : (v << 8) | next);
+        }
+      }
+      if (me.l == 0) s.c.nce = np + 3 + ne;
+    }
+    __syncwarp();
+    if (tg)
+      for (int t = me.l; t < np; t += G) {
+        const int p = s.pa[t], r = s.pb[t];
+        const bool sw = n > 12 && r < p;
+        s.c.ce[t] = (unsigned short)(sw ? (r << 8) | p : (p << 8) | r);
+        atomicOr(&s.c.adj[p], 1u << r);
+        atomicOr(&s.c.adj[r], 1u << p);
+      }
+    __syncwarp();
+    const R3Geo<G> geo{&s, 80.0f * 5.9604645e-8f * M * M * 1.0001f + 16.0f * 2.910383e-11f * M};
+    g_greedy<G, true>(s.c, geo, tg ? n : 0);
+    if (tg) {
+      const int nf = (int)s.c.nface;
+      if ((u32)nf != nt) {
+        if (me.l == 0) atomicOr(a.err, R3_COUNT);
+      } else {
+        const unsigned short code = (unsigned short)((mask & 15) | (63 << 6) | (klass << 12));
+        if (me.l == 0) ++ngc, ngt += (u32)nf;
+        for (int k = me.l; k < nf; k += G) {
+          const u32 f = s.c.face[k];
+          u32 r = 0;
+          for (int j = 0; j < nf; ++j) r += s.c.face[j] < f ? 1u : 0u;
+          const int p = (int)(f >> 16), u = (int)((f >> 8) & 255u), w = (int)(f & 255u);
+          tri[t0 + r] = make_int3((int)s.gid[p], (int)s.gid[u], (int)s.gid[w]);
+          a.label[t0 + r] = r3_label36<G>(a, s, p, u, w);
+          a.code[t0 + r] = code;
+        }
+      }
+    }
+    __syncwarp();
   }
+  // the counts, one atomic per warp
+  ngc = __reduce_add_sync(0xffffffffu, ngc), ngt = __reduce_add_sync(0xffffffffu, ngt);
+  if (me.lane == 0 && ngc) atomicAdd(a.ng, ngc), atomicAdd(a.ngtri, ngt);
 }
 
 // ---------------------------------------------------------------------------
-// Tier-G: one warp per cell.  Lane 0 builds the cell's boundary graph in
-// shared memory; the warp ranks the candidate pairs, runs the greedy pass
+// Cells of more than 32 nodes (all Tier-G): one warp each.  Lane 0 builds the
+// cell's boundary graph in shared memory; the warp ranks the candidate pairs, runs the greedy pass
 // (each candidate tested by the lanes against the nodes and the kept
 // edges), lists the faces and writes them in sorted order.
 // ---------------------------------------------------------------------------
@@ -1206,14 +1700,13 @@ __global__ void __launch_bounds__(32 * R3G_WARPS) k_r3_tierg(R3Args a) {
   __shared__ R3GShared sh[R3G_WARPS];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   R3GShared& S = sh[wid];
-  const u32 ng = *a.ng;
+  const u32 ng = a.ncls[3];
   for (u32 g = blockIdx.x * R3G_WARPS + wid; g < ng; g += gridDim.x * R3G_WARPS) {
-    const u32 c = a.glist[g] & ~R3_BIG;
-    if (!(a.glist[g] & R3_BIG)) continue;  // k_r3_gsmall's (the whole warp reads one entry)
+    const u32 c = *r3_list(a, 3, g);
     if (lane == 0) {
       const R3Cell C = r3_load(a, c);
       R3SharedEv ev{S.ev};
-      S.err = r3_build(a, c, C, S.L, ev, false);
+      S.err = r3_build(a, c, C, S.L, ev, true);
     }
     __syncwarp();
     if (S.err) {
@@ -1345,7 +1838,7 @@ __global__ void __launch_bounds__(32 * R3G_WARPS) k_r3_tierg(R3Args a) {
       continue;
     }
     const unsigned short code = (unsigned short)((L.mask & 15) | (63 << 6) | (L.klass << 12));
-    if (lane == 0) atomicAdd(a.ngtri, (u32)nf);
+    if (lane == 0) atomicAdd(a.ngtri, (u32)nf), atomicAdd(a.ng, 1u);
     int3* tri = reinterpret_cast<int3*>(a.tri);
     for (int i = lane; i < nf; i += 32) {
       const int f = S.face[i];
@@ -1380,10 +1873,12 @@ int launch_r3_count(const R3Args& a, cudaStream_t st) {
 int launch_r3_emit(const R3Args& a, cudaStream_t st) {
   const unsigned g = (unsigned)std::min<u64>((a.nt + 255) / 256, 152 * 16);
   k_r3_emit_uncut<<<std::max(g, 1u), 256, 0, st>>>(a);
-  k_r3_emit<<<152 * 16, 128, 0, st>>>(a);
-  k_r3_gsmall<<<152 * 16, 128, 0, st>>>(a);
   k_r3_tierg<<<152 * 8, 32 * R3G_WARPS, 0, st>>>(a);
-  return 4;
+  k_r3_cells<32, 4, false><<<152 * 5, 64, 0, st>>>(a);
+  k_r3_cells<32, 2, true><<<152 * 5, 64, 0, st>>>(a);
+  k_r3_cells<16, 1, true><<<152 * 10, 64, 0, st>>>(a);
+  k_r3_cells<8, 0, true><<<152 * 16, 64, 0, st>>>(a);
+  return 6;
 }
 
 }  // namespace sbmt

@@ -1366,14 +1366,15 @@ int r3_one(sbmt_ctx* ctx, Lane* lane, const unsigned char* dimg, i64 pitch, int 
   if ((rc = aalloc(lane, &a.deg, nv)) || (rc = aalloc(lane, &a.vptr, nv + 1)) || (rc = aalloc(lane, &a.inc, 3 * nt)) ||
       (rc = aalloc(lane, &a.ntri, nt)) || (rc = aalloc(lane, &a.nown, nt)) || (rc = aalloc(lane, &a.nin, nt)) ||
       (rc = aalloc(lane, &a.own3, nt)) || (rc = aalloc(lane, &a.toff, nt + 1)) || (rc = aalloc(lane, &a.eoff, nt + 1)) ||
-      (rc = aalloc(lane, &a.ioff, nt + 1)) || (rc = aalloc(lane, &a.glist, nt)) || (rc = aalloc(lane, &cnt, 8)) ||
+      (rc = aalloc(lane, &a.ioff, nt + 1)) || (rc = aalloc(lane, &a.glist, nt)) || (rc = aalloc(lane, &cnt, 16)) ||
       (rc = aalloc(lane, &scr, scr_words)) || (rc = aalloc(lane, &a.ulab, nt)) ||
       (rc = aalloc(lane, &a.cmark, (nt + 31) / 32)) || (rc = aalloc(lane, &a.cand, nt)) ||
-      (rc = aalloc(lane, &a.cutl, nt)))
+      (rc = aalloc(lane, &a.cutl, nt)) || (rc = aalloc(lane, &a.ovl, nt)) || (rc = aalloc(lane, &a.rec, nt)))
     return bail(rc);
-  a.err = cnt, a.ncut = cnt + 1, a.ng = cnt + 2, a.ngtri = cnt + 3, a.ncand = cnt + 4, a.ngsmall = cnt + 5;
+  a.err = cnt, a.ncut = cnt + 1, a.ng = cnt + 2, a.ngtri = cnt + 3, a.ncand = cnt + 4, a.ncls = cnt + 8;
+  a.nrec = (unsigned long long*)(cnt + 14);
   CK(cudaMemsetAsync(a.deg, 0, sizeof(u32) * (size_t)nv, st));
-  CK(cudaMemsetAsync(cnt, 0, 8 * sizeof(u32), st));
+  CK(cudaMemsetAsync(cnt, 0, 16 * sizeof(u32), st));
   int nk = 0;
   TRACE(KN_R3, nk = launch_r3_adjacency(a, scr, st));
   TRACE(KN_R3, nk = launch_r3_count(a, st));

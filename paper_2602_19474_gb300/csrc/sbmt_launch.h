@@ -303,12 +303,15 @@ struct R3Args {
   double* xy;
   int* tri;
   unsigned short *label, *code;
-  u32 *glist, *ng, *err, *ncut, *ngtri;  // glist: the Tier-G cells (bit 31: over 12 nodes), ng of them
+  u32 *ncut, *ng, *err, *ngtri;  // cut cells, Tier-G cells, error bits, Tier-G triangles
   unsigned short* ulab;  // per cell: the label of an uncut cell's pixel box
   u32* cmark;            // candidate bit-plane, (nt + 31) / 32 words
   u32 *cand, *ncand;     // the candidates (nt entries) and their count
-  u32* ngsmall;          // Tier-G cells done by one thread
-  u32* cutl;             // the cut cells (nt entries), ncut of them
+  u32 *cutl, *glist;     // the cut cells' lists by node count (nt entries each, two lists in each)
+  u32* ovl;              // cut cells without a record (nt entries)
+  u32* ncls;             // the five lists' lengths
+  u64* rec;              // the cut cells' records (nt words), nrec words of them asked for
+  unsigned long long* nrec;
 };
 int launch_r3_adjacency(const R3Args& a, u32* scr, cudaStream_t st);
 int launch_r3_count(const R3Args& a, cudaStream_t st);

@@ -349,3 +349,15 @@ def test_retriangulate_points_on_and_near_pixel_lines(seed):
     g = _imported(img, xy, tri)
     assert_same(g, o)
     assert o["n_cut_cells"] > 50
+
+
+@pytest.mark.parametrize("hn,sigma,w,h", [(4, 1.0, 61, 40), (8, 3.0, 150, 130), (10, 3.0, 170, 150)])
+def test_cells_of_every_group_size(hn, sigma, w, h):
+    """Cut cells from one chord to more nodes than a group of 16 lanes takes,
+    with and without room for every cell's record (about one 64-bit word a
+    cell: used up at h = 4 and above on these images): bit for bit the
+    oracle's mesh."""
+    img = synth.noise_bitmap(np.random.default_rng(hn), w, h, sigma)
+    g = gpu_full(img, hn, 1)
+    T, o = oracle_full(img, hn, 1)
+    assert_same(g, o)
