@@ -615,10 +615,10 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     return -1;
   k_heat_flags<<<gt, HB, 0, st>>>(tri, label, T, L, flag);
   k_heat_free<<<grid_v(V), HB, 0, st>>>(V, flag);
-  launches += 2 + launch_scan(flag, 1, fidx, (u32)V, sscr, st);
+  launches += 2 + launch_scan(flag, fidx, (u32)V, sscr, st);
   k_heat_list<<<grid_v(V), HB, 0, st>>>(V, flag, fidx, list);
   k_heat_tflag<<<gt, HB, 0, st>>>(label, T, L, tf);
-  launches += 2 + launch_scan(tf, 1, tpos, (u32)T, sscr, st);
+  launches += 2 + launch_scan(tf, tpos, (u32)T, sscr, st);
   u32 n = 0, nr = 0;
   if (cudaMemcpyAsync(&n, fidx + V, 4, cudaMemcpyDeviceToHost, st) ||
       cudaMemcpyAsync(&nr, tpos + T, 4, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))
@@ -630,7 +630,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
   launches += 1;
   if (n > 0) {
     // the free vertices' incident records, sorted, then their mass and diagonal
-    launches += launch_scan(vcnt, 1, vptr, n, sscr, st);
+    launches += launch_scan(vcnt, vptr, n, sscr, st);
     if (cudaMemcpyAsync(mcnt, vptr, 4 * (size_t)n, cudaMemcpyDeviceToDevice, st)) return -1;
     k_heat_inc<<<gr, HB, 0, st>>>(rec, nr, mcnt, inc);
     k_heat_gather<<<gv, HB, 0, st>>>(rec, n, vptr, inc, mass, kdiag);
@@ -642,7 +642,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
   if (n > 0) {
     if (cudaMemsetAsync(flag, 0, 4 * (size_t)n, st)) return -1;
     k_heat_rowcount<<<gr, HB, 0, st>>>(rec, nr, flag);
-    launches += 1 + launch_scan(flag, 1, rowptr, n, sscr, st);
+    launches += 1 + launch_scan(flag, rowptr, n, sscr, st);
     if (cudaMemcpyAsync(flag, rowptr, 4 * (size_t)n, cudaMemcpyDeviceToDevice, st)) return -1;
     k_heat_fill<<<gr, HB, 0, st>>>(rec, nr, tau, flag, col, val);
     k_heat_merge<<<gv, HB, 0, st>>>(n, rowptr, col, val, mcnt);

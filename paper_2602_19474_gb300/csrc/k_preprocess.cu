@@ -261,16 +261,20 @@ SBMT_DEV bool step2(const PreArgs& a, double x, double y, float xf, float yf, bo
 }
 
 // Region I, first pass: one block per vertex row.  A vertex whose nearby
-// pixels carry one label stays; the others are queued in the row's own part
-// of the queue (the row's vertex ids) for the second pass, which takes them
-// densely, so that the few near the boundary do not hold up warps of
-// vertices that stay.
-constexpr int PV_U = 1;  // vertices per thread per iteration (2 measured slower)
+// pixels carry one label stays; the others are queued for the second pass,
+// which takes them densely, so that the few near the boundary do not hold up
+// warps of vertices that stay.  (One queue: in a part per row the second pass
+// had a few dozen vertices per block of 128 threads, 64 us against 24 on
+// 4096^2 labels at h = 2, where gathering the places per block costs this pass
+// 14.)
+
+constexpr int PV_LIST = 1024;  // queued vertices gathered per block before a global place is taken
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_pre_vertex(PreArgs a) {
-  __shared__ u32 nslow;
-  if (threadIdx.x == 0) nslow = 0;
+  __shared__ u32 s_list[PV_LIST];
+  __shared__ u32 s_n, s_base;
+  if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
   const GridP& g = a.g;
   const int r = blockIdx.x, W = g.W, H = g.H;
@@ -318,35 +322,38 @@ __global__ void __launch_bounds__(256) k_pre_vertex(PreArgs a) {
     }
     return uniform;
   };
-  // the screen's loads before any store; whole warps in every iteration
-  for (i64 k0 = 0; k0 < n; k0 += PV_U * blockDim.x) {
-    bool slow[PV_U];
-#pragma unroll
-    for (int u = 0; u < PV_U; ++u) {
-      const i64 k = k0 + threadIdx.x + u * blockDim.x;
-      slow[u] = k < n && !uniform_at(2 * (lo + k) + j - a.m0);
+  u32 total = 0;  // vertices in s_list, the same in every thread
+  auto flush = [&]() {
+    if (threadIdx.x == 0) s_base = total ? atomicAdd(a.cnt + 7, total) : 0u;
+    __syncthreads();
+    for (u32 e = threadIdx.x; e < total; e += blockDim.x)
+      a.vq[s_base + e] = make_uint2((u32)base + s_list[e], (u32)r);
+    if (threadIdx.x == 0) s_n = 0;
+    total = 0;
+    __syncthreads();
+  };
+  // whole blocks in every iteration (2 vertices per thread measured slower)
+  for (i64 k0 = 0; k0 < n; k0 += blockDim.x) {
+    const i64 k = k0 + threadIdx.x;
+    const bool slow = k < n && !uniform_at(2 * (lo + k) + j - a.m0);
+    if (k < n && !slow) {
+      const i64 mi = 2 * (lo + k) + j - a.m0;
+      xy[base + k] = make_double2(a.tab[mi], y);
+      a.xyf[base + k] = make_float2(a.tabf[mi], yf);
+      a.status[base + k] = 0;
+      a.snap[base + k] = -1;
     }
-#pragma unroll
-    for (int u = 0; u < PV_U; ++u) {
-      const i64 k = k0 + threadIdx.x + u * blockDim.x;
-      if (k < n && !slow[u]) {
-        const i64 mi = 2 * (lo + k) + j - a.m0;
-        xy[base + k] = make_double2(a.tab[mi], y);
-        a.xyf[base + k] = make_float2(a.tabf[mi], yf);
-        a.status[base + k] = 0;
-        a.snap[base + k] = -1;
-      }
-      const u32 m = __ballot_sync(0xFFFFFFFFu, slow[u]);
-      if (m) {
-        u32 q0 = 0;
-        if (lane == 0) q0 = atomicAdd(&nslow, (u32)__popc(m));
-        q0 = __shfl_sync(0xFFFFFFFFu, q0, 0);
-        if (slow[u]) a.vq[base + q0 + __popc(m & ((1u << lane) - 1u))] = (u32)(base + k);
-      }
+    const u32 m = __ballot_sync(0xFFFFFFFFu, slow);
+    if (m) {
+      u32 q0 = 0;
+      if (lane == 0) q0 = atomicAdd(&s_n, (u32)__popc(m));
+      q0 = __shfl_sync(0xFFFFFFFFu, q0, 0);
+      if (slow) s_list[q0 + __popc(m & ((1u << lane) - 1u))] = (u32)k;
     }
+    total += (u32)__syncthreads_count(slow);
+    if (total > (u32)PV_LIST - blockDim.x) flush();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) a.vqn[r] = nslow;
+  flush();
 }
 
 // a vertex of the base mesh's outer boundary: one of the six cells around
@@ -370,60 +377,53 @@ SBMT_DEV bool border_safe(const PreArgs& a, int bx, int by) {
   return (double)side >= dadd(__ddiv_rn((double)g.p, (double)g.q), a.A);
 }
 
-// Region I, second pass: the queued vertices, one block per vertex row at a
-// time.  Step 1 in full; Step 2 only screened here: a vertex the float
-// distances leave within reach of c goes to the third pass, so that the
-// double-precision work of the moves runs in full warps.
-constexpr int PR_CHUNK = 1024;
-
+// Region I, second pass: the queued vertices.  Step 1 in full; Step 2 only
+// screened here: a vertex the float distances leave within reach of c goes to
+// the third pass, so that the double-precision work of the moves runs in full
+// warps.
 template <typename T>
 __global__ void __launch_bounds__(128) k_pre_region1(PreArgs a) {
-  __shared__ u32 rq[PR_CHUNK];
-  __shared__ u32 nrq, rq0;
   const GridP& g = a.g;
   double2* xy = reinterpret_cast<double2*>(a.xy);
+  const u32 nq = a.cnt[7];
+  const int lane = threadIdx.x & 31;
   u32 nsnap = 0;
-  for (int r = blockIdx.x; r < g.nvrows; r += gridDim.x) {
-    const u32 nq = a.vqn[r];
-    const i64 base = g.vbase[r], j = g.vj0 + r, lo = g.vlo[r];
-    const double y = a.ytab[r];
-    const float yf = a.ytabf[r];
-    for (u32 c0 = 0; c0 < nq; c0 += PR_CHUNK) {
-      if (threadIdx.x == 0) nrq = 0;
-      __syncthreads();
-      const u32 c1 = min(nq, c0 + PR_CHUNK);
-      for (u32 e = c0 + threadIdx.x; e < c1; e += blockDim.x) {
-        const i64 v = a.vq[base + e], mi = 2 * (lo + (v - base)) + j - a.m0;
-        const double x = a.tab[mi];
-        const float xf = a.tabf[mi];
-        int bx = -1, by = -1;
-        if (step1(a, x, y, xf, yf, bx, by) && (!outer_vertex(g, lo + (v - base), j) || border_safe(a, bx, by))) {
-          xy[v] = make_double2(half_minus(bx), half_minus(by));
-          a.xyf[v] = make_float2((float)bx - 0.5f, (float)by - 0.5f);
-          a.status[v] = 1;
-          a.snap[v] = by * (g.W + 1) + bx;
-          ++nsnap;
-          continue;
-        }
+  for (u32 e0 = blockIdx.x * blockDim.x; e0 < nq; e0 += gridDim.x * blockDim.x) {
+    const u32 e = e0 + threadIdx.x;
+    bool reach = false;
+    uint2 qe = make_uint2(0u, 0u);
+    if (e < nq) {
+      qe = a.vq[e];
+      const int r = (int)qe.y;
+      const i64 v = qe.x, j = g.vj0 + r, i = g.vlo[r] + (v - g.vbase[r]), mi = 2 * i + j - a.m0;
+      const double x = a.tab[mi], y = a.ytab[r];
+      const float xf = a.tabf[mi], yf = a.ytabf[r];
+      int bx = -1, by = -1;
+      if (step1(a, x, y, xf, yf, bx, by) && (!outer_vertex(g, i, j) || border_safe(a, bx, by))) {
+        xy[v] = make_double2(half_minus(bx), half_minus(by));
+        a.xyf[v] = make_float2((float)bx - 0.5f, (float)by - 0.5f);
+        a.status[v] = 1;
+        a.snap[v] = by * (g.W + 1) + bx;
+        ++nsnap;
+      } else {
         double2 dummy;
         xy[v] = make_double2(x, y);
         a.xyf[v] = make_float2(xf, yf);
         a.status[v] = 0;
         a.snap[v] = -1;
-        if (step2<T>(a, x, y, xf, yf, true, dummy)) rq[atomicAdd(&nrq, 1u)] = (u32)v;
+        reach = step2<T>(a, x, y, xf, yf, true, dummy);
       }
-      __syncthreads();
-      const u32 n = nrq;
-      if (threadIdx.x == 0 && n) rq0 = atomicAdd(a.cnt + 6, n);
-      __syncthreads();
-      for (u32 e = threadIdx.x; e < n; e += blockDim.x) {
-        a.rq[rq0 + e] = make_uint2(rq[e], (u32)r);
-      }
-      __syncthreads();
+    }
+    const u32 m = __ballot_sync(0xFFFFFFFFu, reach);
+    if (m) {
+      u32 q0 = 0;
+      if (lane == 0) q0 = atomicAdd(a.cnt + 6, (u32)__popc(m));
+      q0 = __shfl_sync(0xFFFFFFFFu, q0, 0);
+      if (reach) a.rq[q0 + __popc(m & ((1u << lane) - 1u))] = qe;
     }
   }
   nsnap = __reduce_add_sync(0xFFFFFFFFu, nsnap);
-  if ((threadIdx.x & 31) == 0 && nsnap) atomicAdd(a.cnt + 3, nsnap);
+  if (lane == 0 && nsnap) atomicAdd(a.cnt + 3, nsnap);
 }
 
 // Region I, third pass: Step 2 in doubles for the vertices the float
@@ -448,19 +448,6 @@ __global__ void __launch_bounds__(128) k_pre_repel(PreArgs a) {
   }
   nrep = __reduce_add_sync(0xFFFFFFFFu, nrep);
   if ((threadIdx.x & 31) == 0 && nrep) atomicAdd(a.cnt + 4, nrep);
-}
-
-// population counts of a bit-plane; with wpr > 0 the plane has rows of wpr
-// words and only the bits of corner columns 0..W count
-__global__ void __launch_bounds__(256) k_popc(const u32* words, u64 n, int wpr, int W, u32* out) {
-  for (u64 w = (u64)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (u64)gridDim.x * blockDim.x) {
-    u32 b = words[w];
-    if (wpr > 0) {
-      const int c0 = 32 * (int)(w % (u64)wpr);
-      if (W - c0 < 31) b &= (2u << (W - c0)) - 1u;
-    }
-    out[w] = __popc(b);
-  }
 }
 
 // the boundary points in corner-id order
@@ -724,31 +711,29 @@ unsigned grid_for(u64 n, int threads, unsigned cap) {
 
 }  // namespace
 
-int launch_preprocess(const PreArgs& a, u64 nw, u32* wpop, u32* wscan, u32* scr, cudaStream_t st) {
+int launch_preprocess(const PreArgs& a, u64 nw, u32* wscan, u32* scr, cudaStream_t st) {
   int n = 0;
   const GridP& g = a.g;
   k_pre_rows<<<grid_for((u64)std::max<i64>(a.nm, std::max(g.nrows, g.nvrows)), 256, 1024), 256, 0, st>>>(a), ++n;
   if (a.dtype == 1) {
     k_pre_vertex<unsigned char><<<g.nvrows, 256, 0, st>>>(a);
-    k_pre_region1<unsigned char><<<(unsigned)std::min(g.nvrows, 152 * 16), 128, 0, st>>>(a);
+    k_pre_region1<unsigned char><<<152 * 16, 128, 0, st>>>(a);
     k_pre_repel<unsigned char><<<152 * 8, 128, 0, st>>>(a);
   } else {
     k_pre_vertex<unsigned short><<<g.nvrows, 256, 0, st>>>(a);
-    k_pre_region1<unsigned short><<<(unsigned)std::min(g.nvrows, 152 * 16), 128, 0, st>>>(a);
+    k_pre_region1<unsigned short><<<152 * 16, 128, 0, st>>>(a);
     k_pre_repel<unsigned short><<<152 * 8, 128, 0, st>>>(a);
   }
   n += 3;
   // the boundary points, in corner-id order
-  k_popc<<<grid_for(nw, 256, 152 * 8), 256, 0, st>>>(a.vrow, nw, a.wpr, g.W, wpop), ++n;
-  n += launch_scan(wpop, 1, wscan, (u32)nw, scr, st);
+  n += launch_scan_bits(a.vrow, a.wpr, g.W, wscan, (u32)nw, scr, st);
   k_pre_points<<<grid_for(nw, 256, 152 * 8), 256, 0, st>>>(a, nw, wscan), ++n;
   // Step 3
   const u64 nsw = ((u64)g.ncells + 31) / 32;
   if (cudaMemsetAsync(a.sbit, 0, (nsw + 1) * sizeof(u32), st) != cudaSuccess) return -1;
   k_pre_step3<<<grid_for(a.np, 128, 152 * 16), 128, 0, st>>>(a), ++n;
-  n += launch_scan(a.appl, 1, a.ascan, a.np, scr, st);
-  k_popc<<<grid_for(nsw, 256, 152 * 8), 256, 0, st>>>(a.sbit, nsw, 0, 0, a.spop), ++n;
-  n += launch_scan(a.spop, 1, a.wpre, (u32)nsw, scr, st);
+  n += launch_scan(a.appl, a.ascan, a.np, scr, st);
+  n += launch_scan_bits(a.sbit, 0, 0, a.wpre, (u32)nsw, scr, st);
   // the preprocessed mesh
   if (a.dtype == 1) {
     k_pre_emit<unsigned char><<<(unsigned)std::min(g.nrows, 152 * 16), 256, 0, st>>>(a);

@@ -1,9 +1,8 @@
 // k_scan.cu -- exclusive prefix sums of u32 counts (offsets of the output
 // patches, of the (cell, segment) pairs and crossing events per segment, of
 // the bucket ranges).  The meshing path scans every array of a batch in one
-// single-pass launch (k_mscan); the preprocessing and heat paths use the
-// three-pass scan (one block for small inputs; else tile sums, a scan of the
-// tile sums, and the tiles with their offsets).
+// single-pass launch (k_mscan); the preprocessing, retriangulation and heat
+// paths use the two-kernel scan (one block for small inputs).
 #include "sbmt_cell.cuh"
 #include "sbmt_launch.h"
 
@@ -38,37 +37,88 @@ __global__ void __launch_bounds__(1024) k_scan_small(const u32* in, int stride, 
   if (t == 1023) out[n] = sh[1023];
 }
 
-__global__ void __launch_bounds__(256) k_tile_sums(const u32* in, int stride, u32 n, u32* part) {
-  __shared__ u32 s_sh[8];
-  const u64 base = (u64)blockIdx.x * TILE;
-  u32 s = 0;
-  for (int u = 0; u < 8; ++u) {
-    const u64 i = base + (u64)threadIdx.x * 8 + u;
-    if (i < n) s += in[i * stride];
+// Up to three arrays of one length at once (blockIdx.y: which), as two kernels:
+// the tiles' sums, then the tiles, every block adding the sums before its tile
+// itself.  For up to some thousand tiles that costs less than a launch of one
+// block for their scan (1.9e7 values: 22 us for the three-kernel form's middle
+// kernel and its gap alone); above, the sums are scanned in between.
+// A value is the word itself or, with BITS, the number of its bits (of a
+// bit-plane with rows of wpr words, those of columns 0 .. W; wpr 0: all).
+struct Scan3 {
+  const u32* in[3];
+  u32* out[3];
+  u32* part[3];
+  int wpr, W;
+};
+template <bool BITS>
+SBMT_DEV u32 scan_value(const Scan3& s, const u32* in, u64 i) {
+  u32 v = in[i];
+  if (BITS) {
+    if (s.wpr > 0) {
+      const int c0 = 32 * (int)((u32)i % (u32)s.wpr);
+      if (s.W - c0 < 31) v &= (2u << (s.W - c0)) - 1u;
+    }
+    v = __popc(v);
   }
-  u32 tot;
-  block_exscan256(s, &tot, s_sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
+  return v;
 }
-
-__global__ void __launch_bounds__(256) k_tile_scan(const u32* in, int stride, u32 n, const u32* part_scan,
-                                                   u32* out) {
+template <bool BITS>
+__global__ void __launch_bounds__(256) k_tile_sums(Scan3 s, u32 n) {
   __shared__ u32 s_sh[8];
-  const u64 base = (u64)blockIdx.x * TILE;
-  u32 v[8], s = 0;
+  const u32* in = s.in[blockIdx.y];
+  const u64 i0 = (u64)blockIdx.x * TILE + threadIdx.x;
+  u32 sum = 0;
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (i0 + 256 * u < n) sum += scan_value<BITS>(s, in, i0 + 256 * u);
+  u32 tot;
+  block_exscan256(sum, &tot, s_sh);
+  if (threadIdx.x == 0) s.part[blockIdx.y][blockIdx.x] = tot;
+}
+template <bool BITS, bool SCANNED>
+__global__ void __launch_bounds__(256) k_tile_scan(Scan3 s, u32 n) {
+  __shared__ u32 s_sh[8];
+  const u32* in = s.in[blockIdx.y];
+  const u32* part = s.part[blockIdx.y];
+  u32* out = s.out[blockIdx.y];
+  const u64 i0 = (u64)blockIdx.x * TILE + 8 * threadIdx.x;
+  u32 v[8], sum = 0;
+#pragma unroll
   for (int u = 0; u < 8; ++u) {
-    const u64 i = base + (u64)threadIdx.x * 8 + u;
-    v[u] = i < n ? in[i * stride] : 0u;
-    s += v[u];
+    v[u] = i0 + u < n ? scan_value<BITS>(s, in, i0 + u) : 0u;
+    sum += v[u];
+  }
+  u32 prefix;
+  if (SCANNED) {
+    prefix = part[blockIdx.x];
+  } else {
+    u32 before = 0;
+    for (u32 k = threadIdx.x; k < blockIdx.x; k += 256) before += part[k];
+    block_exscan256(before, &prefix, s_sh);
   }
   u32 tot;
-  u32 run = block_exscan256(s, &tot, s_sh) + part_scan[blockIdx.x];
+  u32 run = block_exscan256(sum, &tot, s_sh) + prefix;
+#pragma unroll
   for (int u = 0; u < 8; ++u) {
-    const u64 i = base + (u64)threadIdx.x * 8 + u;
-    if (i < n) out[i] = run;
+    if (i0 + u < n) out[i0 + u] = run;
     run += v[u];
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 255) out[n] = run;
+}
+
+constexpr u32 SELF_TILES = 8192;  // up to this many tiles a block adds the sums before it itself
+
+template <bool BITS>
+int run_scan(const Scan3& s, int arrays, u32 n, cudaStream_t st) {
+  const u32 tiles = n / TILE + 1;
+  k_tile_sums<BITS><<<dim3(tiles, arrays), 256, 0, st>>>(s, n);
+  if (tiles <= SELF_TILES) {
+    k_tile_scan<BITS, false><<<dim3(tiles, arrays), 256, 0, st>>>(s, n);
+    return 2;
+  }
+  for (int k = 0; k < arrays; ++k) k_scan_small<<<1, 1024, 0, st>>>(s.part[k], 1, s.part[k], tiles);
+  k_tile_scan<BITS, true><<<dim3(tiles, arrays), 256, 0, st>>>(s, n);
+  return 2 + arrays;
 }
 
 // ---------------------------------------------------------------------------
@@ -168,19 +218,30 @@ __global__ void __launch_bounds__(256) k_mscan(const ScanJob* __restrict__ sj, c
 
 }  // namespace
 
-size_t scan_scratch_words(u32 n) { return n <= 16384 ? 0 : (size_t)((n + TILE - 1) / TILE) + 1; }
+size_t scan_scratch_words(u32 n) { return (size_t)n / TILE + 2; }
 
-int launch_scan(const u32* in, int stride, u32* out, u32 n, u32* scratch, cudaStream_t st) {
-  if (n <= 16384 || scratch == nullptr) {
-    k_scan_small<<<1, 1024, 0, st>>>(in, stride, out, n);
+int launch_scan(const u32* in, u32* out, u32 n, u32* scratch, cudaStream_t st) {
+  if (n <= 4096) {
+    k_scan_small<<<1, 1024, 0, st>>>(in, 1, out, n);
     return 1;
   }
-  const u32 tiles = (n + TILE - 1) / TILE;
-  k_tile_sums<<<tiles, 256, 0, st>>>(in, stride, n, scratch);
-  // scan of the tile sums in place (tiles <= 65536 for any n < 2^27)
-  k_scan_small<<<1, 1024, 0, st>>>(scratch, 1, scratch, tiles);
-  k_tile_scan<<<tiles, 256, 0, st>>>(in, stride, n, scratch, out);
-  return 3;
+  Scan3 s{};
+  s.in[0] = in, s.out[0] = out, s.part[0] = scratch;
+  return run_scan<false>(s, 1, n, st);
+}
+
+int launch_scan_bits(const u32* in, int wpr, int W, u32* out, u32 n, u32* scratch, cudaStream_t st) {
+  Scan3 s{};
+  s.in[0] = in, s.out[0] = out, s.part[0] = scratch, s.wpr = wpr, s.W = W;
+  return run_scan<true>(s, 1, n, st);
+}
+
+size_t scan3_scratch_words(u32 n) { return 3 * scan_scratch_words(n); }
+
+int launch_scan3(const u32* const in[3], u32* const out[3], u32 n, u32* scratch, cudaStream_t st) {
+  Scan3 s{};
+  for (int k = 0; k < 3; ++k) s.in[k] = in[k], s.out[k] = out[k], s.part[k] = scratch + k * scan_scratch_words(n);
+  return run_scan<false>(s, 3, n, st);
 }
 
 int launch_mscan(const ScanJob* sj, const u32* tpre, int nsj, u32 ntiles, unsigned long long* flags, u32* ticket,

@@ -1250,18 +1250,18 @@ int pre_one(sbmt_ctx* ctx, Lane* lane, const sbmt_image* img, const sbmt_params*
   PreArgs a{};
   a.g = g, a.img = dimg, a.pitch = pitch, a.dtype = img->dtype, a.vrow = vrow, a.wpr = wpr, a.np = (u32)NP;
   a.m0 = m_lo, a.nm = (i64)nm;
-  u32 *wpop, *wscan, *scr;
+  u32 *wscan, *scr;
   const size_t scr_words =
       std::max({scan_scratch_words((u32)nw), scan_scratch_words((u32)NP), scan_scratch_words((u32)nsw)}) + 1;
   if ((rc = aalloc(lane, &a.tab, nm)) || (rc = aalloc(lane, &a.tabf, nm)) ||
       (rc = aalloc(lane, &a.prow, 2 * (size_t)nrows)) || (rc = aalloc(lane, &a.xyf, V)) ||
-      (rc = aalloc(lane, &wpop, nw)) || (rc = aalloc(lane, &wscan, nw + 1)) ||
+      (rc = aalloc(lane, &wscan, nw + 1)) ||
       (rc = aalloc(lane, &a.plist, std::max<u64>(NP, 1))) || (rc = aalloc(lane, &a.appl, std::max<u64>(NP, 1))) ||
       (rc = aalloc(lane, &a.ascan, NP + 1)) || (rc = aalloc(lane, &a.sbit, nsw + 1)) ||
-      (rc = aalloc(lane, &a.spop, nsw + 1)) || (rc = aalloc(lane, &a.wpre, nsw + 1)) ||
+      (rc = aalloc(lane, &a.wpre, nsw + 1)) ||
       (rc = aalloc(lane, &scr, scr_words)) || (rc = aalloc(lane, &a.ytab, (size_t)nvr)) ||
       (rc = aalloc(lane, &a.ytabf, (size_t)nvr)) || (rc = aalloc(lane, &a.vq, std::max<u64>(V, 1))) ||
-      (rc = aalloc(lane, &a.vqn, (size_t)nvr)) || (rc = aalloc(lane, &a.rq, std::max<u64>(V, 1))))
+      (rc = aalloc(lane, &a.rq, std::max<u64>(V, 1))))
     return bail(rc);
   char* candb;
   if ((rc = aalloc(lane, &candb, pre_cand_bytes((u32)NP)))) return bail(rc);
@@ -1303,7 +1303,7 @@ int pre_one(sbmt_ctx* ctx, Lane* lane, const sbmt_image* img, const sbmt_params*
   m->nv = (int64_t)V, m->nt = (int64_t)NCELL, m->ncells = (int64_t)NCELL, m->nvg = (int64_t)V;
   m->thr[0] = A, m->thr[1] = B, m->thr[2] = C, m->npts = (int64_t)NP;
   int nk = 0;
-  TRACE(KN_PRE, nk = launch_preprocess(a, nw, wpop, wscan, scr, st));
+  TRACE(KN_PRE, nk = launch_preprocess(a, nw, wscan, scr, st));
   if (nk < 0) return bail(fail(SBMT_ECUDA, "preprocess launch"));
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(m->h_info, a.cnt, 6 * sizeof(u32), cudaMemcpyDeviceToHost, st));
@@ -1362,31 +1362,33 @@ int r3_one(sbmt_ctx* ctx, Lane* lane, const unsigned char* dimg, i64 pitch, int 
   a.img = dimg, a.pitch = pitch, a.dtype = dtype, a.W = W, a.H = H;
   a.txy = txy, a.ttri = ttri, a.nv = (u32)nv, a.nt = (u64)nt;
   u32 *cnt, *scr;
-  const size_t scr_words = std::max(scan_scratch_words((u32)nv), scan_scratch_words((u32)nt)) + 1;
-  if ((rc = aalloc(lane, &a.deg, nv)) || (rc = aalloc(lane, &a.vptr, nv + 1)) || (rc = aalloc(lane, &a.inc, 3 * nt)) ||
+  const u32 nwords = (u32)((nt + 31) / 32);
+  const size_t scr_words = scan3_scratch_words(nwords);
+  u32* words;  // per word of 32 cells: the cut cells, three sums (zeroed), then their scans
+  if ((rc = aalloc(lane, &a.head, nv)) || (rc = aalloc(lane, &a.link, 3 * nt)) ||
       (rc = aalloc(lane, &a.ntri, nt)) || (rc = aalloc(lane, &a.nown, nt)) || (rc = aalloc(lane, &a.nin, nt)) ||
-      (rc = aalloc(lane, &a.own3, nt)) || (rc = aalloc(lane, &a.toff, nt + 1)) || (rc = aalloc(lane, &a.eoff, nt + 1)) ||
-      (rc = aalloc(lane, &a.ioff, nt + 1)) || (rc = aalloc(lane, &a.glist, nt)) || (rc = aalloc(lane, &cnt, 16)) ||
+      (rc = aalloc(lane, &a.own3, nt)) || (rc = aalloc(lane, &a.glist, nt)) || (rc = aalloc(lane, &cnt, 16)) ||
       (rc = aalloc(lane, &scr, scr_words)) || (rc = aalloc(lane, &a.ulab, nt)) ||
       (rc = aalloc(lane, &a.cmark, (nt + 31) / 32)) || (rc = aalloc(lane, &a.cand, nt)) ||
       (rc = aalloc(lane, &a.cutl, nt)) || (rc = aalloc(lane, &a.ovl, nt)) || (rc = aalloc(lane, &a.rec, nt)))
     return bail(rc);
   a.err = cnt, a.ncut = cnt + 1, a.ng = cnt + 2, a.ngtri = cnt + 3, a.ncand = cnt + 4, a.ncls = cnt + 8;
   a.nrec = (unsigned long long*)(cnt + 14);
-  CK(cudaMemsetAsync(a.deg, 0, sizeof(u32) * (size_t)nv, st));
+  if ((rc = aalloc(lane, &words, 4 * (size_t)nwords + 3 * ((size_t)nwords + 1)))) return bail(rc);
+  a.kmark = words;
+  for (int k = 0; k < 3; ++k)
+    a.wsum[k] = words + (k + 1) * (size_t)nwords, a.woff[k] = words + 4 * (size_t)nwords + k * ((size_t)nwords + 1);
+  CK(cudaMemsetAsync(words, 0, 4 * sizeof(u32) * (size_t)nwords, st));
+  CK(cudaMemsetAsync(a.head, 0xFF, sizeof(u32) * (size_t)nv, st));
   CK(cudaMemsetAsync(cnt, 0, 16 * sizeof(u32), st));
   int nk = 0;
-  TRACE(KN_R3, nk = launch_r3_adjacency(a, scr, st));
   TRACE(KN_R3, nk = launch_r3_count(a, st));
-  TRACE(KN_R3, nk = launch_scan(a.ntri, 1, a.toff, (u32)nt, scr, st));
-  TRACE(KN_R3, nk = launch_scan(a.nown, 1, a.eoff, (u32)nt, scr, st));
-  TRACE(KN_R3, nk = launch_scan(a.nin, 1, a.ioff, (u32)nt, scr, st));
+  TRACE(KN_R3, nk = launch_scan3(a.wsum, a.woff, nwords, scr, st));
   (void)nk;
   CK(cudaGetLastError());
   u32* h = m->h_info;
-  CK(cudaMemcpyAsync(h + 4, a.toff + nt, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h + 5, a.eoff + nt, sizeof(u32), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h + 6, a.ioff + nt, sizeof(u32), cudaMemcpyDeviceToHost, st));
+  for (int k = 0; k < 3; ++k)
+    CK(cudaMemcpyAsync(h + 4 + k, a.woff[k] + nwords, sizeof(u32), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(h, cnt, sizeof(u32), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (h[0]) {
@@ -1398,7 +1400,7 @@ int r3_one(sbmt_ctx* ctx, Lane* lane, const unsigned char* dimg, i64 pitch, int 
                                        : "an inconsistent mesh (a cell not counter-clockwise, an edge in three cells)",
                      e));
   }
-  const u64 NT = h[4], NE = h[5], NI = h[6], NV = (u64)nv + NE + NI;
+  const u64 NT = (u64)nt + h[4], NE = h[5], NI = h[6], NV = (u64)nv + NE + NI;
   if (NV >= (1ull << 31) || NT >= (1ull << 31)) return bail(fail(SBMT_EINVAL, "mesh too large"));
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t off_tri = up(16 * NV), off_lab = up(off_tri + 12 * NT), off_code = up(off_lab + 2 * NT);

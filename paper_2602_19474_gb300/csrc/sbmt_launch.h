@@ -201,11 +201,17 @@ int launch_segments(const unsigned char* img, i64 pitch, int dtype, int W, int H
 // pairs, one thread each.
 size_t walk_chunks(u32 NP);
 
-// exclusive scan of n u32 values with stride `stride` into out (n + 1
-// entries, out[n] = total); inputs above 65536 values need scratch of
-// scan_scratch_words(n) words
+// exclusive scan of n u32 values into out (n + 1 entries, out[n] = total),
+// with scratch of scan_scratch_words(n) words
 size_t scan_scratch_words(u32 n);
-int launch_scan(const u32* in, int stride, u32* out, u32 n, u32* scratch, cudaStream_t st);
+int launch_scan(const u32* in, u32* out, u32 n, u32* scratch, cudaStream_t st);
+// the same over the words' numbers of bits (rows of wpr words, columns 0 .. W
+// of each counted; wpr 0: every bit)
+int launch_scan_bits(const u32* in, int wpr, int W, u32* out, u32 n, u32* scratch, cudaStream_t st);
+// three exclusive scans of n values each (out[k][n]: the total), scratch of
+// scan3_scratch_words(n) words
+size_t scan3_scratch_words(u32 n);
+int launch_scan3(const u32* const in[3], u32* const out[3], u32 n, u32* scratch, cudaStream_t st);
 
 // quality measures of T triangles: mm [0] min angle, [1] min doubled area,
 // [2] max AR as double bits; cnt [0] slivers, [1] equilateral; part per block
@@ -232,11 +238,11 @@ int launch_project(const double* xy, const int* tri, u64 T, u64 V, const float* 
 // the coordinates), bscr2 = bscr^2.  Scratch: tab / tabf (nm entries, the
 // x table over m0 <= m < m0 + nm), prow (2 per strip row), xyf (float copy
 // of the moved lattice positions), plist (np boundary points), cand
-// (pre_cand_bytes(np)), appl / ascan (np and np + 1 words), sbit / spop /
-// wpre (split-cell bit-plane of ncells / 32 + 1 words, its counts and their
-// scan), ytab / ytabf / vqn (one per vertex row), vq / rq (nverts), cnt
-// (7 zeroed words: error, eliminations, split cells, snapped, repelled,
-// points with a candidate, the Step 2 queue length).  Outputs: xy (lattice vertices, then
+// (pre_cand_bytes(np)), appl / ascan (np and np + 1 words), sbit / wpre
+// (split-cell bit-plane of ncells / 32 + 1 words and the scan of its counts),
+// ytab / ytabf (one per vertex row), vq / rq (nverts), cnt (8 zeroed words:
+// error, eliminations, split cells, snapped, repelled, points with a
+// candidate, the Step 2 and Region I queues' lengths).  Outputs: xy (lattice vertices, then
 // the inserted points), tri / label / code (ncells + split cells
 // triangles), status and snap per lattice vertex, elim (3 per elimination).
 struct PreCand;
@@ -259,14 +265,13 @@ struct PreArgs {
   float* tabf;
   double* ytab;  // y of every vertex row, and its float copy
   float* ytabf;
-  u32* vq;       // Region I queue: vertex ids, in each row's own id range
-  u32* vqn;      // queued vertices per vertex row
+  uint2* vq;     // Region I queue: (vertex id, vertex row), nverts entries, cnt[7] of them
   uint2* rq;     // Step 2 queue: (vertex id, vertex row), nverts entries
   int* prow;
   float2* xyf;
   u32* plist;
   PreCand* cand;
-  u32 *appl, *ascan, *sbit, *spop, *wpre, *cnt;
+  u32 *appl, *ascan, *sbit, *wpre, *cnt;
   double* xy;
   int* tri;
   unsigned short *label, *code;
@@ -274,19 +279,17 @@ struct PreArgs {
   int *snap, *elim;
 };
 size_t pre_cand_bytes(u32 np);
-// nw vrow words; wpop / wscan: nw and nw + 1 words; scr: scan scratch for
+// nw vrow words; wscan: nw + 1 words; scr: scan scratch for
 // the largest of nw, np and ncells / 32 + 1.  Returns the kernels launched,
 // -1 if a CUDA call failed.
-int launch_preprocess(const PreArgs& a, u64 nw, u32* wpop, u32* wscan, u32* scr, cudaStream_t st);
+int launch_preprocess(const PreArgs& a, u64 nw, u32* wscan, u32* scr, cudaStream_t st);
 
 // Region III (Alg. 2 on an arbitrary counter-clockwise mesh T, the
 // preprocessed one): the image, T (nv vertices as double pairs, nt cells as
-// vertex-id triples), the per-vertex cell lists (deg: nv counts, vptr:
-// nv + 1 offsets, inc: 3 nt cell ids), per cell the triangle count, the
-// events on the edges it owns (the smaller cell beside an edge), the inside
-// vertices and the owned events per local edge (8 bits each), their
-// exclusive scans (nt + 1 each), the output mesh, the Tier-G queue (nt
-// entries) and its length, the error word and counters.
+// vertex-id triples), per vertex the list of candidate cells, per cut cell
+// the triangle count, the events on the edges it owns (the smaller cell beside an edge), the inside
+// vertices and the owned events per local edge (8 bits each), the output
+// mesh, the error word and counters.
 enum : u32 { R3_CAPACITY = 1u, R3_GEOMETRY = 2u, R3_COUNT = 4u };
 struct R3Args {
   const unsigned char* img;
@@ -296,9 +299,13 @@ struct R3Args {
   const int* ttri;
   u32 nv;
   u64 nt;
-  u32 *deg, *vptr, *inc;
+  u32* head;    // per vertex: its list of candidate cells (all bits set: none)
+  uint2* link;  // list entries (cell, next), 3 per candidate
+  // per cut cell (unset elsewhere): triangles, owned events (and per edge),
+  // inside vertices; per word of 32 cells: the cut cells, and the sums of their
+  // triangles beyond one, owned events and inside vertices with their scans
   u32 *ntri, *nown, *nin, *own3;
-  u32 *toff, *eoff, *ioff;
+  u32 *kmark, *wsum[3], *woff[3];
   u32 ne_total;
   double* xy;
   int* tri;
@@ -313,7 +320,6 @@ struct R3Args {
   u64* rec;              // the cut cells' records (nt words), nrec words of them asked for
   unsigned long long* nrec;
 };
-int launch_r3_adjacency(const R3Args& a, u32* scr, cudaStream_t st);
 int launch_r3_count(const R3Args& a, cudaStream_t st);
 int launch_r3_emit(const R3Args& a, cudaStream_t st);
 
