@@ -459,9 +459,13 @@ __global__ void __launch_bounds__(1024) k_rec_prefix(const Job* __restrict__ job
 //     earlier chunks) the label, so the warp's stores of neighbouring cells
 //     are adjacent;
 //  4. the cut cells, a lane per record, offsets from a scan over the records.
-constexpr int EMIT_W = 4;  // buckets (warps) per block
+// A mesh of few buckets leaves the device nearly empty while each warp goes
+// through its 32 chunks (72 us for 54 buckets, 39 us for two), so there SUB
+// warps share a bucket: each repeats steps 1 and 2 and takes every SUB-th chunk
+// and group of records (25 us and 18 us).  emit_sub gives SUB.
+constexpr int EMIT_W = 4;  // warps per block
 
-template <bool ONE>
+template <bool ONE, int SUB>
 __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant__ Job one,
                                                            const Job* __restrict__ jobs, const u32* __restrict__ bpre,
                                                            int njobs) {
@@ -470,7 +474,8 @@ __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant
   __shared__ __align__(16) u32 s_x[EMIT_W][NB];  // extra triangles per cell; a run start's label after step 2
   SBMT_BLOCK_JOB(ONE, one, jobs, bpre, njobs)
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const u32 b = lb * EMIT_W + (u32)w;
+  const u32 b = (lb * EMIT_W + (u32)w) / SUB;
+  const int sub = (int)((lb * EMIT_W + (u32)w) % SUB);
   if (b >= J.nbc) return;
   constexpr unsigned FULL = 0xFFFFFFFFu;
   const GridP& g = J.g;
@@ -568,7 +573,7 @@ __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant
   i64 clo_r = g.clo[rr], cb_r = g.cbase[rr];
   i64 vb0 = g.vbase[rr] - g.vlo[rr], vb1 = g.vbase[rr + 1] - g.vlo[rr + 1];
 #pragma unroll 4
-  for (int t = 0; t * 32 < nc; ++t) {
+  for (int t = sub; t * 32 < nc; t += SUB) {
     const int k = 32 * t + lane;
     const u32 cm = __shfl_sync(FULL, cutm, t), sm = __shfl_sync(FULL, startm, t);
     const u32 ext = __shfl_sync(FULL, xex, t), ct = __shfl_sync(FULL, carry, t);
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant
     }
     const u32 pe = ex_carry + ie - ex, cb = CB0 + ch_carry + ic - ch;
     ex_carry += __shfl_sync(FULL, ie, 31), ch_carry += __shfl_sync(FULL, ic, 31);
-    if (!valid) continue;
+    if (!valid || (SUB > 1 && (int)((base >> 5) % SUB) != sub)) continue;
     const u32 kl = rec.cell - (u32)c0;
     u32 off = T0 + kl + pe;
     if (cp.on) {
@@ -683,7 +688,7 @@ __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant
       reinterpret_cast<double2*>(J.xy)[cb - cp.xy0] = vv;
     }
   }
-  if (cp.on && b == J.nbc - 1 && lane == 0)
+  if (cp.on && b == J.nbc - 1 && lane == 0 && sub == 0)
     cp.patch_off[cp.cut_scan[J.nbc]] = J.extra_scan[J.nbc] + cp.cut_scan[J.nbc];
 }
 
@@ -738,10 +743,28 @@ int launch_cutcells_b(const Job* one, const Job* jobs, int njobs, const BatchPtr
   return 2;
 }
 
-int launch_emit_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, cudaStream_t st) {
+int emit_sub(u64 buckets) {
+  // one warp a bucket once that gives the SMs (152) 16 warps each; below, as
+  // many as 8 a bucket
+  int sub = 1;
+  while (sub < 8 && buckets * sub < 152 * 16) sub *= 2;
+  return sub;
+}
+
+namespace {
+template <bool ONE>
+void launch_emit(int sub, const Job& oj, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, cudaStream_t st) {
+  if (sub == 8) k_emit_b<ONE, 8><<<nblocks, 32 * EMIT_W, 0, st>>>(oj, jobs, bpre, njobs);
+  else if (sub == 4) k_emit_b<ONE, 4><<<nblocks, 32 * EMIT_W, 0, st>>>(oj, jobs, bpre, njobs);
+  else if (sub == 2) k_emit_b<ONE, 2><<<nblocks, 32 * EMIT_W, 0, st>>>(oj, jobs, bpre, njobs);
+  else k_emit_b<ONE, 1><<<nblocks, 32 * EMIT_W, 0, st>>>(oj, jobs, bpre, njobs);
+}
+}  // namespace
+
+int launch_emit_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, int sub, cudaStream_t st) {
   if (nblocks == 0) return 0;
-  if (one) k_emit_b<true><<<nblocks, 32 * EMIT_W, 0, st>>>(*one, jobs, bpre, njobs);
-  else k_emit_b<false><<<nblocks, 32 * EMIT_W, 0, st>>>(Job{}, jobs, bpre, njobs);
+  if (one) launch_emit<true>(sub, *one, jobs, bpre, njobs, nblocks, st);
+  else launch_emit<false>(sub, Job{}, jobs, bpre, njobs, nblocks, st);
   return 1;
 }
 

@@ -953,7 +953,10 @@ int mesh_run(sbmt_ctx* ctx, Lane* lane, const sbmt_image* imgs, int n, const sbm
   const std::vector<u32> p_walk = prefix_of(n, [&](int k) { return (u32)((walk_chunks(J[k].NP) + 255) / 256); });
   const std::vector<u32> p_sc = prefix_of(n, [&](int k) { return (std::max(J[k].NP, J[k].NE) + 255) / 256; });
   const std::vector<u32> p_rk = prefix_of(n, [&](int k) { return J[k].nbe; });
-  const std::vector<u32> p_so = prefix_of(n, [&](int k) { return (J[k].nbc + 3) / 4; });  // the emission: 4 buckets a block
+  u64 nbc_all = 0;
+  for (int k = 0; k < n; ++k) nbc_all += J[k].nbc;
+  const int sub = emit_sub(nbc_all);
+  const std::vector<u32> p_so = prefix_of(n, [&](int k) { return (u32)(((u64)J[k].nbc * sub + 3) / 4); });
   const std::vector<u32> p_sw = prefix_of(n, [&](int k) { return (J[k].nbc + 3) / 4; });  // the sort: 4 buckets a block
   const std::vector<u32> p_go = prefix_of(n, [&](int k) { return (J[k].nbc + 7) / 8; });
   const std::vector<u32> p_lt = prefix_of(n, [&](int k) {
@@ -1025,7 +1028,7 @@ int mesh_run(sbmt_ctx* ctx, Lane* lane, const sbmt_image* imgs, int n, const sbm
                                 fork ? lane->side2 : nullptr, lane->order, lane->warp));
   if (ntg < 0) kerr = 1;
   if (fork && cudaEventRecord(lane->join, lane->side) != cudaSuccess) kerr = 1;
-  TRACE(KN_EMIT, launch_emit_b(one, dj, dpre(4), n, p_so[n], st));
+  TRACE(KN_EMIT, launch_emit_b(one, dj, dpre(4), n, p_so[n], sub, st));
   if (!fork) TRACE(KN_XY, launch_lattice_b(dj, dpre(6), p_lt[n], dpre(7), p_lx[n], n, st));
   if (fork && cudaStreamWaitEvent(st, lane->join, 0) != cudaSuccess) kerr = 1;
   launch_status_b(dj, n, bp, st);

@@ -176,7 +176,9 @@ int launch_sort_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u
 // cut-cell classification, persistent over every job's records
 int launch_cutcells_b(const Job* one, const Job* jobs, int njobs, const BatchPtrs& bp, int blocks_per_sm,
                       cudaStream_t st);
-int launch_emit_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, cudaStream_t st);
+// the emission: sub warps a bucket (emit_sub of the batch's buckets), four to a block
+int emit_sub(u64 buckets);
+int launch_emit_b(const Job* one, const Job* jobs, const u32* bpre, int njobs, u32 nblocks, int sub, cudaStream_t st);
 int launch_lattice_b(const Job* jobs, const u32* bpre_tab, u32 nb_tab, const u32* bpre_xy, u32 nb_xy, int njobs,
                      cudaStream_t st);
 // Tier-G: ordering (bpre over warps of buckets), then persistent kernels over
