@@ -1774,15 +1774,20 @@ int mesh_query(sbmt_ctx* ctx, sbmt_mesh mesh, int wait_ms, sbmt_mesh_view* out) 
     if (it == ctx->meshes.end()) return fail(SBMT_ENOENT, "unknown mesh %llu", (unsigned long long)mesh);
     m = it->second;
   }
+  if (wait_ms < 0) {
+    // no limit: the driver's own wait, which returns within microseconds of
+    // the event (a sleep between polls overslept by some 50)
+    const cudaError_t q = cudaEventSynchronize(m->done);
+    if (q != cudaSuccess) return fail(SBMT_ECUDA, "mesh work failed: %s", cudaGetErrorString(q));
+  }
   const auto t0 = std::chrono::steady_clock::now();
-  while (true) {
+  while (wait_ms >= 0) {
     const cudaError_t q = cudaEventQuery(m->done);
     if (q == cudaSuccess) break;
     if (q != cudaErrorNotReady) return fail(SBMT_ECUDA, "mesh work failed: %s", cudaGetErrorString(q));
     if (wait_ms == 0) return SBMT_EPENDING;
-    if (wait_ms > 0 &&
-        std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(wait_ms))
-      return SBMT_ETIMEDOUT;
+    const auto waited = std::chrono::steady_clock::now() - t0;
+    if (waited > std::chrono::milliseconds(wait_ms)) return SBMT_ETIMEDOUT;
     std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
   int rc = settle(m);
