@@ -240,21 +240,24 @@ __global__ void __launch_bounds__(HB) k_heat_put(u32 n, const u32* list, const d
 // The time steps: one cooperative launch for the whole call, one block of 512
 // threads on each SM (fewer for small regions), all resident, so that a phase
 // of the solver ends in a barrier across the grid instead of a launch, and the
-// host reads nothing until the last step.  Each thread keeps the same rows
-// throughout.  Per iteration:
-//   q = A p, p.q        | barrier
-//   x, r, z; r.z, r.r   | barrier
-//   p = z + beta p      | barrier
-// Everything but the matrix of a 10^6-row region stays in L2, and the phases
-// are short: what an iteration costs is latency (loads, then the barriers) and
-// this GPU's FP64 rate, about 1.6 instructions per clock and SM (14 per row of
-// 6 entries).  So: two rows of the product and three of the vector phases in
-// flight per thread; a block's sums through shared memory in halves (20 warp
-// adds for 512 threads, where a butterfly in every warp takes 80); the blocks'
-// sums published and awaited in one step, which is the barrier (below), and
-// added by every block in one fixed order; one division per block.
-// Measured on 0.33e6 free vertices (4096^2 Voronoi labels, h = 2): 57 us an
-// iteration as three launches with two-stage sums over 1216 blocks, 23 us here.
+// host reads nothing until the last step.  Each block keeps the same rows
+// throughout, their vectors in shared memory.  Per iteration:
+//   q = A z + beta q, p = z + beta p; p.q        | barrier
+//   r, z; r.z (and r.r every eighth time)        | barrier, x meanwhile
+// What an iteration costs is this GPU's FP64 rate, about 1.6 instructions per
+// clock and SM (13 per row of 6 entries), and the two barriers.  So: the product
+// is taken of z, which is final before beta is known, and p and q follow by
+// recurrence, which saves the barrier that a new p would need before the next
+// product; no work that only sometimes counts (r.r); a block's sums through shared
+// memory in halves (a dependent FP64 add is some 100 clocks); the blocks' sums
+// published and awaited in one step, which is the barrier (below), and
+// added in one fixed order; one division per block.
+// Measured on 0.38e6 free vertices (4096^2 Voronoi labels, h = 2), clocks of an
+// iteration: products 14e3 and residuals 4.5e3 (both the FP64 rate), barriers
+// 9e3 and 11e3.  The call took 8.4 ms with three barriers and the vectors in L2 and
+// 5.8 ms now on the same GPU (5.9 and 4.2 ms on another).  Sums by integer limbs
+// instead of FP64 trees, every block waiting for all slots, and a smaller share of rows
+// for block 0 gained nothing.
 // ---------------------------------------------------------------------------
 constexpr int CT = 512;         // threads per block
 constexpr int CG_BLOCKS = 152;  // at most one block per SM
@@ -262,6 +265,7 @@ constexpr int CG_SUMS = 3;      // the most sums a barrier carries
 constexpr int SLOT_WORDS = 4 * CG_SUMS * CG_BLOCKS + 16 * CG_BLOCKS;
 struct HeatCg {
   u32 n, nsteps;
+  u32 block_rows;  // the most rows a block has, in whole slices
   int maxit, sliced;
   double tol;
   const u32* rowptr;
@@ -282,9 +286,9 @@ struct HeatCg {
 };
 constexpr unsigned long long CG_EMPTY = ~0ull;  // no sum has these bits
 
-SBMT_DEV unsigned long long ld_relaxed(const unsigned long long* p) {
+SBMT_DEV unsigned long long ld_acquire(const unsigned long long* p) {
   unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 SBMT_DEV void st_relaxed(unsigned long long* p, unsigned long long v) {
@@ -303,7 +307,7 @@ SBMT_DEV bool wait_words(const HeatCg& h, const unsigned long long* p, size_t st
   while (true) {
     bool wait = false;
 #pragma unroll
-    for (int k = 0; k < K; ++k) w[k] = ld_relaxed(p + k * step);
+    for (int k = 0; k < K; ++k) w[k] = ld_acquire(p + k * step);
 #pragma unroll
     for (int k = 0; k < K; ++k) wait |= w[k] == CG_EMPTY;
     if (!wait) return true;
@@ -327,11 +331,11 @@ SBMT_DEV bool wait_words(const HeatCg& h, const unsigned long long* p, size_t st
 // a barrier, 3 us this way).  Four buffers by turns: entering barrier g, a
 // block empties its slots of buffer (g + 2) % 4.  Those held barrier g - 2,
 // which it has left (and block 0 had read its sums before that), and they are
-// not written before it publishes barrier g + 2.  end(sums) runs on one thread
-// before the block goes on.  False when a wait ran out.
-template <int K, bool TREE, class End>
+// not written before it publishes barrier g + 2.  mid() runs between publishing
+// and waiting, end(sums) on one thread before the block goes on.  False when a wait ran out.
+template <int K, bool TREE, class Mid, class End>
 SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double (*s)[CT], double* s_out, int* s_fail,
-                        const End& end) {
+                        const Mid& mid, const End& end) {
   const u32 tid = threadIdx.x;
   double t[K];
 #pragma unroll
@@ -374,12 +378,12 @@ SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double 
       for (int k = 0; k < K; ++k)
         st_relaxed(in + k * CG_BLOCKS + blockIdx.x, (unsigned long long)__double_as_longlong(t[k]));
     }
+    mid();
     if (blockIdx.x == 0) {
       __syncthreads();  // the tree's last reads of s
       if (tid < gridDim.x) {
         unsigned long long w[K];
         if (!wait_words<K>(h, in + tid, CG_BLOCKS, w)) *s_fail = 1;
-        fence_gpu();
 #pragma unroll
         for (int k = 0; k < K; ++k) s[k][tid] = __longlong_as_double((long long)w[k]);
       }
@@ -409,11 +413,11 @@ SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double 
     } else if (tid == 0) {
       unsigned long long w[K];
       if (!wait_words<K>(h, out + 4 * blockIdx.x, 1, w)) *s_fail = 1;
-      fence_gpu();
 #pragma unroll
       for (int k = 0; k < K; ++k) t[k] = __longlong_as_double((long long)w[k]);
     }
   }
+  if (gridDim.x == 1) mid();
   if (TREE && tid == 0) {
 #pragma unroll
     for (int k = 0; k < K; ++k) s_out[k] = t[k];
@@ -424,130 +428,138 @@ SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double 
   return *s_fail == 0;
 }
 
-// U rows of A = M + tau K times v (v read from L2: other SMs write it): the
-// rows first, first + step, ..., those below n.  A warp's lanes hold the 32
-// rows of one slice.
-template <int U>
-SBMT_DEV void rows_times(const HeatCg& h, u32 i0, u32 step, const double* v, const double (&vi)[U], double (&y)[U]) {
-  u32 m[U];
-  double w[U][SF], g[U][SF];
+// Row i of A = M + tau K times v (v read from L2: other SMs write it); dd: the
+// diagonal's part.  A warp's lanes hold the 32 rows of one slice.  (Two or
+// three rows in flight per thread were no faster: 16 warps hide the loads behind
+// the FP64 pipe's 19 clocks an instruction.)
+SBMT_DEV double row_times(const HeatCg& h, u32 i, const double* v, double dd) {
+  const u32 m = h.mcnt[i];
+  double a = dd;
+  u32 k0 = 0;
   if (h.sliced) {
+    double w[SF], g[SF];
+    const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const u32 i = i0 + u * step;
-      if (i >= h.n) continue;
-      m[u] = h.mcnt[i];
-      const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
+    for (int k = 0; k < SF; ++k) w[k] = h.sval[at + 32 * k], g[k] = __ldcg(v + h.scol[at + 32 * k]);
 #pragma unroll
-      for (int k = 0; k < SF; ++k) w[u][k] = h.sval[at + 32 * k], g[u][k] = __ldcg(v + h.scol[at + 32 * k]);
-    }
+    for (int k = 0; k < SF; ++k)
+      if ((u32)k < m) a += w[k] * g[k];
+    for (u32 k = SF; k < min(m, (u32)SW); ++k) a += h.sval[at + 32 * k] * __ldcg(v + h.scol[at + 32 * k]);
+    k0 = SW;
   }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    const u32 i = i0 + u * step;
-    if (i >= h.n) continue;
-    double a = h.dg[i] * vi[u];
-    u32 k0 = 0;
-    if (h.sliced) {
-#pragma unroll
-      for (int k = 0; k < SF; ++k)
-        if ((u32)k < m[u]) a += w[u][k] * g[u][k];
-      const size_t at = (size_t)(i >> 5) * (32 * SW) + (i & 31u);
-      for (u32 k = SF; k < min(m[u], (u32)SW); ++k) a += h.sval[at + 32 * k] * __ldcg(v + h.scol[at + 32 * k]);
-      k0 = SW;
-    } else {
-      m[u] = h.mcnt[i];
-    }
-    if (k0 < m[u])
-      for (u32 e = h.rowptr[i] + k0, e1 = h.rowptr[i] + m[u]; e < e1; ++e) a += h.val[e] * __ldcg(v + h.col[e]);
-    y[u] = a;
-  }
+  if (k0 < m)
+    for (u32 e = h.rowptr[i] + k0, e1 = h.rowptr[i] + m; e < e1; ++e) a += h.val[e] * __ldcg(v + h.col[e]);
+  return a;
 }
 
+// Rows of a block: whole slices of 32, the same number (or one less) in every
+// block, so that the FP64 pipes of all SMs finish together (rows dealt out in
+// rounds of CT left most SMs idle in the last round).
+SBMT_HD u32 cg_slice(u32 n, u32 block, u32 blocks) { return (u32)((u64)((n + 31) / 32) * block / blocks); }
+constexpr int CG_VECS = 6;  // vectors of a block's rows held on chip
+constexpr size_t CG_SMEM = 227 * 1024 - 13 * 1024;  // what a block has for them, beside its sums
+
+// ONCHIP: the block's rows of x, r, z, p, q and the diagonals stay in shared
+// memory for the whole solve (48 B a row: up to 0.69e6 free vertices); only z, which the
+// product gathers, is also written through to L2.  Otherwise they stay in L2.
+//
+// Two barriers an iteration: the product is taken of z, which is final
+// before beta is known, and q = A z + beta q, p = z + beta p follow from it, so that
+// the new p needs no barrier of its own before the next product.
+template <bool ONCHIP>
 __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatCg h) {
+  extern __shared__ double s_vec[];
   __shared__ double s[CG_SUMS][CT];
   __shared__ double s_sum[CG_SUMS], s_k;
   __shared__ int s_fail;
-  const u32 first = blockIdx.x * CT + threadIdx.x, stride = gridDim.x * CT, n = h.n;
+  const u32 row0 = 32 * cg_slice(h.n, blockIdx.x, gridDim.x);
+  const u32 rows = min(32 * cg_slice(h.n, blockIdx.x + 1, gridDim.x), h.n) - row0;
+  const u32 R = h.block_rows, tid = threadIdx.x;
+  double* x = ONCHIP ? s_vec : h.x + row0;
+  double* r = ONCHIP ? s_vec + R : h.r + row0;
+  double* z = ONCHIP ? s_vec + 2 * R : h.z + row0;
+  double* p = ONCHIP ? s_vec + 3 * R : h.p + row0;
+  double* q = ONCHIP ? s_vec + 4 * R : h.q + row0;
+  double* dinv = ONCHIP ? s_vec + 5 * R : nullptr;
+  // (a thread touches only its own rows of these: no block barrier)
+  if (ONCHIP)
+    for (u32 l = tid; l < rows; l += CT) x[l] = h.x[row0 + l], dinv[l] = h.dinv[row0 + l];
+  auto dinv_at = [&](u32 l) { return ONCHIP ? dinv[l] : h.dinv[row0 + l]; };
   u32 gen = 0;
   for (u32 step = 0; step < h.nsteps; ++step) {
-    // b = M x; r = b - A x, z = D^-1 r, p = z; r.z, r.r, b.b
+    // b = M x; r = b - A x, z = D^-1 r; r.z, r.r, b.b
     double a3[3] = {0.0, 0.0, 0.0};
-    for (u32 i = first; i < n; i += stride) {
-      const double xi[1] = {h.x[i]}, bi = h.mass[i] * xi[0];
-      double qi[1];
-      rows_times<1>(h, i, stride, h.x, xi, qi);
-      const double di = h.dinv[i], rv = di != 0.0 ? bi - qi[0] : 0.0, zv = rv * di;
-      h.r[i] = rv, h.z[i] = zv, h.p[i] = zv;
+    for (u32 l = tid; l < rows; l += CT) {
+      const u32 i = row0 + l;
+      const double xi = x[l], bi = h.mass[i] * xi, dd = h.dg[i] * xi;
+      const double qi = row_times(h, i, h.x, dd);
+      const double di = dinv_at(l), rv = di != 0.0 ? bi - qi : 0.0, zv = rv * di;
+      r[l] = rv, z[l] = zv, p[l] = 0.0, q[l] = 0.0;
+      if (ONCHIP) h.z[i] = zv;
       a3[0] += rv * zv, a3[1] += rv * rv, a3[2] += bi * bi;
     }
-    if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [](const double*) {})) return;
-    double rz = s_sum[0], rr = s_sum[1];
+    if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
+    double rz = s_sum[0], rr = s_sum[1], be = 0.0;
     const double stop = h.tol * h.tol * s_sum[2];
     int it = 0;
     while (rr > stop && it < h.maxit) {
       bool look = false;
       while (!look) {
         double a1[1] = {0.0};
-        for (u32 i0 = first; i0 < n; i0 += 2 * stride) {
-          double pi[2], y[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) pi[u] = i0 + u * stride < n ? h.p[i0 + u * stride] : 0.0;
-          rows_times<2>(h, i0, stride, h.p, pi, y);
-#pragma unroll
-          for (int u = 0; u < 2; ++u)
-            if (i0 + u * stride < n) h.q[i0 + u * stride] = y[u], a1[0] += pi[u] * y[u];
+        for (u32 l = tid; l < rows; l += CT) {
+          // (the diagonal times z is r, up to z's rounding)
+          const double qv = row_times(h, row0 + l, h.z, r[l]) + be * q[l], pv = z[l] + be * p[l];
+          q[l] = qv, p[l] = pv;
+          a1[0] += pv * qv;
         }
-        if (!grid_sums<1, true>(h, a1, gen, s, s_sum, &s_fail,
-                          [&](const double* t) { s_k = t[0] != 0.0 ? rz / t[0] : 0.0; }))
+        if (!grid_sums<1, true>(h, a1, gen, s, s_sum, &s_fail, [] {},
+                                [&](const double* t) { s_k = t[0] != 0.0 ? rz / t[0] : 0.0; }))
           return;
         const double al = s_k;
-        double a2[2] = {0.0, 0.0};
-        for (u32 i0 = first; i0 < n; i0 += 3 * stride) {
-          double x[3], r[3], p[3], q[3], d[3];
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const u32 i = i0 + u * stride;
-            if (i < n) x[u] = h.x[i], r[u] = h.r[i], p[u] = h.p[i], q[u] = h.q[i], d[u] = h.dinv[i];
-          }
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const u32 i = i0 + u * stride;
-            if (i >= n) continue;
-            h.x[i] = x[u] + al * p[u];
-            const double rv = r[u] - al * q[u], zv = rv * d[u];
-            h.r[i] = rv, h.z[i] = zv;
-            a2[0] += rv * zv, a2[1] += rv * rv;
-          }
-        }
-        if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail,
-                          [&](const double* t) { s_k = rz != 0.0 ? t[0] / rz : 0.0; }))
-          return;
-        const double rz_new = s_sum[0], rr_new = s_sum[1];
-        const double be = s_k;
-        for (u32 i0 = first; i0 < n; i0 += 3 * stride) {
-          double z[3], p[3];
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const u32 i = i0 + u * stride;
-            if (i < n) z[u] = h.z[i], p[u] = h.p[i];
-          }
-#pragma unroll
-          for (int u = 0; u < 3; ++u)
-            if (i0 + u * stride < n) h.p[i0 + u * stride] = z[u] + be * p[u];
-        }
-        rz = rz_new;
         ++it;
-        const double none[1] = {0.0};
-        if (!grid_sums<1, false>(h, none, gen, s, s_sum, &s_fail, [](const double*) {})) return;
-        look = (it & 7) == 0 || it == h.maxit;  // the residual is looked at every eighth iteration
-        if (look) rr = rr_new;
+        look = (it & 7) == 0 || it == h.maxit;  // the residual is looked at (and summed) every eighth iteration
+        double a2[2] = {0.0, 0.0};
+        for (u32 l0 = tid; l0 < rows; l0 += 3 * CT) {
+          double rv[3], qv[3], dv[3];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const u32 l = l0 + u * CT;
+            if (l < rows) rv[u] = r[l], qv[u] = q[l], dv[u] = dinv_at(l);
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const u32 l = l0 + u * CT;
+            if (l >= rows) continue;
+            const double rn = rv[u] - al * qv[u], zn = rn * dv[u];
+            r[l] = rn, z[l] = zn;
+            if (ONCHIP) h.z[row0 + l] = zn;
+            a2[0] += rn * zn;
+            if (look) a2[1] += rn * rn;
+          }
+        }
+        // (x is not needed before the next step: updated while the sums travel)
+        auto update_x = [&] {
+#pragma unroll 4
+          for (u32 l = tid; l < rows; l += CT) x[l] += al * p[l];
+        };
+        const auto beta = [&](const double* t) { s_k = rz != 0.0 ? t[0] / rz : 0.0; };
+        if (look) {
+          if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail, update_x, beta)) return;
+        } else {
+          const double only[1] = {a2[0]};
+          if (!grid_sums<1, true>(h, only, gen, s, s_sum, &s_fail, update_x, beta)) return;
+        }
+        rz = s_sum[0], be = s_k;
+        if (look) rr = s_sum[1];
       }
     }
-    // the step's peak (positive doubles order as their bits)
+    // the step's peak (positive doubles order as their bits), and x for the
+    // next step's product
     unsigned long long top = 0;
-    for (u32 i = first; i < n; i += stride) {
-      const long long bits = __double_as_longlong(h.x[i]);
+    for (u32 l = tid; l < rows; l += CT) {
+      const double xv = x[l];
+      if (ONCHIP) h.x[row0 + l] = xv;
+      const long long bits = __double_as_longlong(xv);
       if (bits > 0) top = max(top, (unsigned long long)bits);
     }
     for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
@@ -555,6 +567,9 @@ __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatC
     if (blockIdx.x == 0 && threadIdx.x == 0)
       h.iters[step] = it, h.done[0] = (int)step + 1, h.done[1] = rr > stop ? 0 : 1;
     if (rr > stop) return;
+    if (step + 1 == h.nsteps) return;
+    const double none[1] = {0.0};
+    if (!grid_sums<1, false>(h, none, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
   }
 }
 
@@ -673,7 +688,14 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     h.slot = slot, h.fail = (u32*)res, h.peak = peak, h.iters = its, h.done = (int*)res + 2;
     void* args[] = {&h};
     const unsigned grid = (unsigned)std::min<u64>(CG_BLOCKS, (n + CT - 1) / CT);
-    if (cudaLaunchCooperativeKernel((const void*)k_heat_cg, dim3(grid), dim3(CT), args, 0, st) != cudaSuccess) return -1;
+    h.block_rows = 32 * (((n + 31) / 32 + grid - 1) / grid);
+    const size_t vec_bytes = (size_t)CG_VECS * 8 * h.block_rows;
+    const bool onchip = vec_bytes <= CG_SMEM;
+    const void* cg = onchip ? (const void*)k_heat_cg<true> : (const void*)k_heat_cg<false>;
+    if (onchip && cudaFuncSetAttribute(cg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM) != cudaSuccess)
+      return -1;
+    if (cudaLaunchCooperativeKernel(cg, dim3(grid), dim3(CT), args, onchip ? vec_bytes : 0, st) != cudaSuccess)
+      return -1;
     ++launches;
     std::vector<char> hres(res_bytes);
     if (cudaMemcpyAsync(hres.data(), res, res_bytes, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))
