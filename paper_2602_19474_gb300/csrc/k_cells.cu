@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(32 * EMIT_W, 8) k_emit_b(const __grid_constant
   const u32 startm = ~cutm & validm & (prevm | rowm);
   {
     const i64 twoS = 2 * g.S;
-    const float inv2S = 1.0f / (float)twoS;
+    const float inv2S = 1.0f / (float)(int)twoS;
     // four run starts at a time: their loads are in flight together
     for (u32 m = startm; m;) {
       int kk[4], lab[4];

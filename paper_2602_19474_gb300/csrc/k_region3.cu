@@ -132,10 +132,10 @@ SBMT_DEV bool r3_corner_event(const R3Args& a, i64 cx, i64 cy, bool hz, bool vt)
 // where it does not, so that every decision is the double formula's.
 // ---------------------------------------------------------------------------
 // This GPU converts from double to float, from 64-bit integers to double
-// and from float to 64-bit integers at about the rate of its FP64
-// arithmetic (a few per clock per SM, against about a hundred for float
-// arithmetic and for integer to float conversions), so the filters take
-// doubles apart with integer instructions.
+// from float to 64-bit integers and from 64-bit integers to float on its FP64
+// pipe (a few per clock per SM, against about a hundred for float arithmetic
+// and for 32-bit conversions), so the filters take doubles apart with integer
+// instructions, and 64-bit integers to float by their upper 32 bits.
 //
 // v (|v| <= 2^24) as a 64-bit fixed-point number with 36 fraction bits:
 // floor(v 2^36), exactly, and whether v 2^36 was not an integer (*inexact)
@@ -204,10 +204,9 @@ SBMT_DEV bool r3_gt(const V& v, i64 k) {
   return v.fx > t || (v.fx == t && v.inexact);
 }
 // the float of a coordinate difference from the fixed-point values (within
-// 2^-35 + 2^-24 |d| of the double difference's real value; integer to
-// float conversions run at the float rate)
+// 2^-35 + (2^-24 + 2^-31) |d| of the double difference's real value)
 SBMT_DEV float r3_fdiff(const R3Split& q, const R3Split& p) {
-  return __fmul_rn((float)(q.fx - p.fx), 1.4551915228366852e-11f);
+  return i64_float(q.fx - p.fx, -36);
 }
 
 // The crossing of the edge from P (its lower-id end) with the line at
@@ -229,6 +228,25 @@ SBMT_DEV float r3_cross_tol(float D, float s, float w) {
 // its pixel edge or corner index in *j, *corner set
 __device__ __noinline__ void r3_cross_exact(double2 P, double2 Q, double c0, bool vert, i64* j, bool* corner) {
   *corner = r3_at_corner(vert ? r3_vy(P, Q, c0) : r3_hx(P, Q, c0), j);
+}
+// The same in integers for an edge between two pixel corners (snapped vertices:
+// the usual reason for a crossing at a corner).  The formula's differences are
+// then integers of at most 2^15, its product exact, its quotient exact where it is an
+// integer and otherwise at least 2^-15 from one, far above its rounding.
+// a, b: across the line and along it, p the edge's first end, q the other.
+SBMT_DEV bool r3_corner_ends(const R3Split& px, const R3Split& py, const R3Split& qx, const R3Split& qy, float D) {
+  constexpr i64 M = (1ll << 36) - 1, HALF = 1ll << 35;
+  return ((px.fx ^ HALF) & M) == 0 && ((py.fx ^ HALF) & M) == 0 && ((qx.fx ^ HALF) & M) == 0 &&
+         ((qy.fx ^ HALF) & M) == 0 && !(px.inexact || py.inexact || qx.inexact || qy.inexact) && D <= 32768.0f;
+}
+SBMT_DEV void r3_cross_corners(const R3Split& pa, const R3Split& pb, const R3Split& qa, const R3Split& qb, int line,
+                               i64* j, bool* corner) {
+  int num = (line - (int)(pa.i + 1)) * (int)(qb.i - pb.i), den = (int)(qa.i - pa.i);
+  if (den < 0) num = -num, den = -den;
+  int q = num / den, r = num - q * den;
+  if (r < 0) --q;
+  *corner = r == 0;
+  *j = pb.i + 1 + q;
 }
 
 // the pixel lines strictly between two coordinates (closed: or through one of
@@ -261,6 +279,7 @@ SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, int edge, u64*
   const R3Split px = r3_split(P.x), py = r3_split(P.y), qx = r3_split(Q.x), qy = r3_split(Q.y);
   const float dxf = r3_fdiff(qx, px), dyf = r3_fdiff(qy, py);
   const float D = fmaxf(fabsf(dxf), fabsf(dyf));
+  const bool grid = r3_corner_ends(px, py, qx, qy, D);
   if (!hz) {
     // horizontal lines y = k - 1/2 strictly between P.y and Q.y
     const float sl = __fdiv_rn(dxf, dyf);
@@ -275,6 +294,7 @@ SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, int edge, u64*
       i64 j;
       bool corner = false;
       if (fr > T && fr < 1.0f - T) j = px.i + zi;
+      else if (grid) r3_cross_corners(py, px, qy, qx, k, &j, &corner);
       else r3_cross_exact(P, Q, (double)k - 0.5, false, &j, &corner);
       if (corner ? r3_corner_event(a, j, k, hz, vt) : r3_hb(a, j, k)) {
         if (n == R3_MAXE) return -1;
@@ -296,6 +316,7 @@ SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, int edge, u64*
       i64 j;
       bool corner = false;
       if (fr > T && fr < 1.0f - T) j = py.i + zi;
+      else if (grid) r3_cross_corners(px, py, qx, qy, m, &j, &corner);
       else r3_cross_exact(P, Q, (double)m - 0.5, true, &j, &corner);
       if (corner) {
         bool dup = false;
@@ -419,6 +440,8 @@ SBMT_DEV int r3_uniform(const R3Args& a, const i64* X, const i64* Y) {
 // float sign decides, else the double formula
 SBMT_DEV bool r3_ccw(const double2* K, const i64* X, const i64* Y) {
   constexpr float S36 = 1.4551915228366852e-11f;  // 2^-36
+  // (converted on the FP64 pipe: this kernel waits for loads, and the integer
+  // form took it from 205 to 238 us)
   const float ax = __fmul_rn((float)(X[1] - X[0]), S36), ay = __fmul_rn((float)(Y[1] - Y[0]), S36);
   const float bx = __fmul_rn((float)(X[2] - X[0]), S36), by = __fmul_rn((float)(Y[2] - Y[0]), S36);
   const float o = __fsub_rn(__fmul_rn(ax, by), __fmul_rn(ay, bx));
@@ -587,6 +610,8 @@ SBMT_DEV int r3_events(const R3Args& a, const R3Cell& C, const R3Geo2& S, bool l
         bool corner = false;
         if (fr > T && fr < 1.0f - T) {
           jj = pl.i + zi;
+        } else if (r3_corner_ends(px, py, qx, qy, D)) {
+          r3_cross_corners(pc, pl, vert ? qx : qy, vert ? qy : qx, line, &jj, &corner);
         } else {
           const double2 P = pi == 0 ? C.K[0] : pi == 1 ? C.K[1] : C.K[2], Q = qi == 0 ? C.K[0] : qi == 1 ? C.K[1] : C.K[2];
           r3_cross_exact(P, Q, (double)line - 0.5, vert, &jj, &corner);
@@ -1151,11 +1176,48 @@ SBMT_DEV unsigned short r3_label(const R3Args& a, double2 p, double2 q, double2 
   return l == R3_OUTSIDE ? (unsigned short)0xFFFF : (unsigned short)l;
 }
 
+__device__ __noinline__ unsigned short r3_label_d(const R3Args& a, double2 p, double2 q, double2 r) {
+  return r3_label(a, p, q, r);
+}
+// the same from the coordinates' fixed-point values, sx and sy their sums:
+// floor((X1 + X2 + X3) / 3 + 1/2) is the double formula's unless the sum is
+// within a bound of a pixel line (three floors, 3 2^-36 below the exact sum at
+// most; the double formula's roundings, below 2^-25 px at 2^24).  -1 when it is.
+SBMT_DEV int r3_label36(const R3Args& a, i64 sx, i64 sy) {
+  constexpr i64 ONE3 = 3ll << 36, BAND = 1ll << 14;  // 3 px; 2^-22 px
+  i64 at[2];
+  bool near = false;
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    // the quotient by 3 2^36: the upper part first, so that 32 bits divide
+    const i64 sum = (d ? sy : sx) + (ONE3 >> 1);
+    const int hi = (int)(sum >> 36);
+    const int f = (hi >= 0 ? hi : hi - 2) / 3;
+    const i64 rem = sum - (i64)f * ONE3;
+    at[d] = f;
+    near |= rem < BAND || rem > ONE3 - BAND;
+  }
+  if (near) return -1;
+  const int l = r3_px(a, at[0], at[1]);
+  return l == R3_OUTSIDE ? 0xFFFF : l;
+}
+
 // ---------------------------------------------------------------------------
 // the cells left as they are: uncut cells of one label, labelled by their
 // pixel box, and candidates the boundary only touches (at a corner or along
 // an edge), labelled by the pixel holding the centroid
 // ---------------------------------------------------------------------------
+// (the kernel took 148 us on 4096^2 labels with the double formula for every
+// candidate left as it is, 128 with the fixed-point one: its loads bound it now)
+__device__ __noinline__ unsigned short r3_cell_label(const R3Args& a, int u, int v, int w) {
+  const double2* K = reinterpret_cast<const double2*>(a.txy);
+  const double2 p = K[u], q = K[v], r = K[w];
+  bool ix;
+  const i64 sx = r3_fix36(p.x, &ix) + r3_fix36(q.x, &ix) + r3_fix36(r.x, &ix);
+  const i64 sy = r3_fix36(p.y, &ix) + r3_fix36(q.y, &ix) + r3_fix36(r.y, &ix);
+  const int l = r3_label36(a, sx, sy);
+  return l >= 0 ? (unsigned short)l : r3_label_d(a, p, q, r);
+}
 __global__ void __launch_bounds__(256) k_r3_emit_uncut(R3Args a) {
   const u32 lane = threadIdx.x & 31u;
   for (u64 c0 = (u64)blockIdx.x * blockDim.x; c0 < a.nt; c0 += (u64)gridDim.x * blockDim.x) {
@@ -1184,9 +1246,8 @@ __global__ void __launch_bounds__(256) k_r3_emit_uncut(R3Args a) {
       const u32 cm = a.cmark[word];
       unsigned short lab;
       if ((cm >> lane) & 1u) {
-        const double2* K = reinterpret_cast<const double2*>(a.txy);
         const int* t = a.ttri + 3 * c;
-        lab = r3_label(a, K[t[0]], K[t[1]], K[t[2]]);
+        lab = r3_cell_label(a, t[0], t[1], t[2]);
       } else {
         lab = a.ulab[c];
       }
@@ -1202,8 +1263,7 @@ __global__ void __launch_bounds__(256) k_r3_emit_uncut(R3Args a) {
     const int3 tv = make_int3(t[0], t[1], t[2]);
     unsigned short lab;
     if ((a.cmark[c >> 5] >> (c & 31)) & 1u) {
-      const double2* K = reinterpret_cast<const double2*>(a.txy);
-      lab = r3_label(a, K[tv.x], K[tv.y], K[tv.z]);
+      lab = r3_cell_label(a, tv.x, tv.y, tv.z);
     } else {
       lab = a.ulab[c];
     }
@@ -1237,6 +1297,14 @@ struct R3State {
   unsigned char pa[3 * G], pb[3 * G];  // the pieces
 };
 
+// The kernel is long: what it needs rarely or in several places is kept out of
+// line, and short loops stay loops (inlined and unrolled it waited for
+// instructions in 18 of 27 cycles per issue: 595 us against 527).
+__device__ __noinline__ int r3_late(const double* x, const double* y, int u, int v, int w) {
+  return r3_sgn(r3_orient(make_double2(x[u], y[u]), make_double2(x[v], y[v]), make_double2(x[w], y[w])));
+}
+__device__ __noinline__ int r3_pixel(const R3Args& a, int x, int y) { return r3_px(a, x, y); }
+
 // the geometry for the greedy rule: the filter decides outside its band, and
 // the double formula of each test, taken as the rule states it, inside.  The
 // float coordinates are within 2^-24 M + 2^-35 of the differences from the
@@ -1250,7 +1318,7 @@ struct R3Geo {
   SBMT_DEV float tol() const { return T; }
   SBMT_DEV double2 pt(int k) const { return make_double2(s->vx[k], s->vy[k]); }
   SBMT_DEV bool resolve(int, int, int, int*) const { return false; }
-  SBMT_DEV int late(int u, int v, int w) const { return r3_sgn(r3_orient(pt(u), pt(v), pt(w))); }
+  SBMT_DEV int late(int u, int v, int w) const { return r3_late(s->vx, s->vy, u, v, w); }
   SBMT_DEV bool between(int u, int w, int k) const {
     const double2 pu = pt(u), pw = pt(w), pk = pt(k);
     const double ex = dsb(pw.x, pu.x), ey = dsb(pw.y, pu.y), len2 = dad(dml(ex, ex), dml(ey, ey));
@@ -1275,26 +1343,12 @@ SBMT_DEV bool r3_at_corner36(double t, i64* idx) {
   return fr == HALF && !inexact;
 }
 
-// the label of the pixel holding ((x1 + x2) + x3) / 3, from the fixed-point
-// values: floor((X1 + X2 + X3) / 3 + 1/2) is the double formula's unless the
-// sum is within a bound of a pixel line (three floors, 3 2^-36 below the exact
-// sum at most; the double formula's roundings, below 2^-26 px at 2^24)
 template <int G>
-SBMT_DEV unsigned short r3_label36(const R3Args& a, const R3State<G>& s, int p, int q, int r) {
-  constexpr i64 ONE3 = 3ll << 36, BAND = 1ll << 14;  // 3 px; 2^-22 px
-  i64 at[2];
-  bool near = false;
-#pragma unroll
-  for (int d = 0; d < 2; ++d) {
-    const i64 sum = (d ? s.Y[p] + s.Y[q] + s.Y[r] : s.X[p] + s.X[q] + s.X[r]) + (ONE3 >> 1);
-    const i64 f = (sum >= 0 ? sum : sum - (ONE3 - 1)) / ONE3, rem = sum - f * ONE3;
-    at[d] = f;
-    near |= rem < BAND || rem > ONE3 - BAND;
-  }
-  if (near)
-    return r3_label(a, make_double2(s.vx[p], s.vy[p]), make_double2(s.vx[q], s.vy[q]), make_double2(s.vx[r], s.vy[r]));
-  const int l = r3_px(a, at[0], at[1]);
-  return l == R3_OUTSIDE ? (unsigned short)0xFFFF : (unsigned short)l;
+__device__ __noinline__ unsigned short r3_node_label(const R3Args& a, const R3State<G>& s, int p, int q, int r) {
+  const int l = r3_label36(a, s.X[p] + s.X[q] + s.X[r], s.Y[p] + s.Y[q] + s.Y[r]);
+  return l >= 0 ? (unsigned short)l
+                : r3_label(a, make_double2(s.vx[p], s.vy[p]), make_double2(s.vx[q], s.vy[q]),
+                           make_double2(s.vx[r], s.vy[r]));
 }
 
 // Tier-T: the key and rotation of the cell in the table's regime, or key 0
@@ -1463,6 +1517,8 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
     }
     __syncwarp();
     // rank on the edge by (s, kind, k, m); node order runs counter-clockwise
+    int node = -1;
+    u32 gid = 0;
     if (isev) {
       int r = 0;
       for (int t = 0; t < ne; ++t) {
@@ -1485,17 +1541,17 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
         if (j2 < 0) err |= R3_GEOMETRY;
         base = r3_edge_base(a, (u32)other, max(j2, 0)) + (u32)r;
       }
-      put(v, ex, ey, base, 1 << ej);
-      s.mk[v] = emk, s.kind[v] = (unsigned char)ekind;
+      node = v, gid = base;
     }
     // inside vertices
     if (live && me.l >= ne && me.l < ne + ni) {
-      const u32 id = i0v + (u32)(me.l - ne);
-      const int v = 3 + me.l;
-      const double2 p = make_double2((double)emk.x - 0.5, (double)emk.y - 0.5);
-      reinterpret_cast<double2*>(a.xy)[id] = p;
-      put(v, p.x, p.y, id, 0);
-      s.mk[v] = emk, s.kind[v] = 3;
+      ex = (double)emk.x - 0.5, ey = (double)emk.y - 0.5;
+      node = 3 + me.l, gid = i0v + (u32)(me.l - ne);
+      reinterpret_cast<double2*>(a.xy)[gid] = make_double2(ex, ey);
+    }
+    if (node >= 0) {
+      put(node, ex, ey, gid, isev ? 1 << ej : 0);
+      s.mk[node] = emk, s.kind[node] = (unsigned char)ekind;
     }
     if (me.ballot(err != 0)) {
       if (err) atomicOr(a.err, err);
@@ -1509,8 +1565,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
     // the filter's frame
     float M = 0.0f;
     if (live && me.l < n) {
-      const float fx = __fmul_rn((float)(s.X[me.l] - s.X[0]), 1.4551915228366852e-11f);
-      const float fy = __fmul_rn((float)(s.Y[me.l] - s.Y[0]), 1.4551915228366852e-11f);
+      const float fx = i64_float(s.X[me.l] - s.X[0], -36), fy = i64_float(s.Y[me.l] - s.Y[0], -36);
       s.c.f[me.l] = make_float2(fx, fy);
       M = fmaxf(fabsf(fx), fabsf(fy));
     }
@@ -1578,41 +1633,43 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
           const bool before = pos(v) < pos(__ffs(ins) - 1);
           lo = before ? v : -1, hi = before ? -1 : v;
         }
-        auto walk = [&](int at) {
+        // counted, then written after the earlier lanes' pieces
+        int at = 0, sum = 0;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
           int prev = lo, k = 0;
           u32 rest = ins;
-          while (on) {
+          bool end = on && hi >= 0;
+          while (rest || end) {
             int cur;
             if (rest) cur = __ffs(rest) - 1, rest &= rest - 1;
-            else if (hi >= 0) cur = hi, hi = -2;
-            else break;
+            else cur = hi, end = false;
             if (prev >= 0) {
               i64 j;
               r3_at_corner36(dml(dad(pos(prev), pos(cur)), 0.5), &j);  // at a corner: the pixel edge starting there
-              int l0, l1;
-              if (!vert) l0 = r3_px(a, j, line - 1), l1 = r3_px(a, j, line);
-              else l0 = r3_px(a, line - 1, j), l1 = r3_px(a, line, j);
+              // the pixels below or left of the line, and above or right of it
+              const int l0 = r3_pixel(a, vert ? line - 1 : (int)j, vert ? (int)j : line - 1);
+              const int l1 = r3_pixel(a, vert ? line : (int)j, vert ? (int)j : line);
               if (l0 != l1) {
                 const bool f = vert ? l0 < l1 : l1 < l0;  // going +x the left side is above, going +y it is -x
-                if (at >= 0 && at + k < 3 * G)
+                if (pass && at + k < 3 * G)
                   s.pa[at + k] = (unsigned char)(f ? prev : cur), s.pb[at + k] = (unsigned char)(f ? cur : prev);
                 ++k;
               }
             }
             prev = cur;
           }
-          if (hi == -2) hi = prev;
-          return k;
-        };
-        const int k = walk(-1);
-        int before = k;
+          if (pass == 0) {
+            int before = k;
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, before, o, G);
-          if (me.l >= o) before += t;
+            for (int o = 1; o < G; o <<= 1) {
+              const int t = __shfl_up_sync(0xffffffffu, before, o, G);
+              if (me.l >= o) before += t;
+            }
+            sum = __shfl_sync(0xffffffffu, before, G - 1, G);
+            at = np + before - k;
+          }
         }
-        const int sum = __shfl_sync(0xffffffffu, before, G - 1, G);
-        if (k) walk(np + before - k);
         np += sum;
       }
     }
@@ -1636,25 +1693,24 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
         if (t == 1) pc1 = __popc(b);
       }
       klass = np == 1 ? thm32_class(0, pc0) : np == 2 ? thm32_class(pc0, pc1) : 0;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const int w = j == 2 ? 0 : j + 1;
-#pragma unroll
-        for (int vert = 0; vert < 2; ++vert) {
-          // the edge on the pixel line `line`: the pixel edges (g - 1/2, g + 1/2)
-          // it has a stretch of
-          const R3Corner ca = vert ? Sx[j] : Sy[j], cb = vert ? Sx[w] : Sy[w];
-          constexpr i64 HALF = 1ll << 35, ONE = 1ll << 36;
-          if (ca.inexact || cb.inexact || ca.fx != cb.fx || (ca.fx & (ONE - 1)) != HALF) continue;
-          const i64 line = (ca.fx >> 36) + 1;
-          const R3Corner ta = vert ? Sy[j] : Sx[j], tb = vert ? Sy[w] : Sx[w];
-          const bool sw = tb.fx < ta.fx;
-          const i64 e0 = sw ? tb.fx : ta.fx, e1 = sw ? ta.fx : tb.fx;
-          const bool x1 = sw ? ta.inexact : tb.inexact;
-          // g + 1/2 > e0 and g - 1/2 < e1
-          for (i64 g = (e0 + HALF) >> 36; (g << 36) - HALF < e1 + (x1 ? 1 : 0); ++g)
-            if (vert ? r3_vb(a, line, g) : r3_hb(a, g, line)) mask |= 2 << j;
-        }
+#pragma unroll 1
+      for (int e = 0; e < 6; ++e) {
+        // edge j on the vertical or horizontal pixel line `line`: the pixel
+        // edges (g - 1/2, g + 1/2) it has a stretch of
+        const int j = e >> 1, vert = e & 1, w = j == 2 ? 0 : j + 1;
+        const i64 *ac = vert ? s.X : s.Y, *al = vert ? s.Y : s.X;  // across the line, along it
+        constexpr i64 HALF = 1ll << 35, ONE = 1ll << 36;
+        if (((s.ix[j] | s.ix[w]) >> (vert ? 0 : 1)) & 1) continue;
+        const i64 ca = ac[j];
+        if (ca != ac[w] || (ca & (ONE - 1)) != HALF) continue;
+        const int line = (int)(ca >> 36) + 1;
+        const bool sw = al[w] < al[j];
+        const i64 e0 = al[sw ? w : j], e1 = al[sw ? j : w];
+        const int x1 = (s.ix[sw ? j : w] >> (vert ? 1 : 0)) & 1;
+        // g + 1/2 > e0 and g - 1/2 < e1
+        for (int g = (int)((e0 + HALF) >> 36); ((i64)g << 36) - HALF < e1 + x1; ++g)
+          if (r3_pixel(a, vert ? line - 1 : g, vert ? g : line - 1) != r3_pixel(a, vert ? line : g, vert ? g : line))
+            mask |= 2 << j;
       }
       key = r3_tier_t<G>(s, ni, ne, np, cnt[0], cnt[1], cnt[2], &sigma);
       if (key < 0) {
@@ -1674,7 +1730,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
           q3[u] = l == 7 ? 3 + ne : l;
         }
         tri[t0 + k] = make_int3((int)s.gid[q3[0]], (int)s.gid[q3[1]], (int)s.gid[q3[2]]);
-        a.label[t0 + k] = r3_label36<G>(a, s, q3[0], q3[1], q3[2]);
+        a.label[t0 + k] = r3_node_label<G>(a, s, q3[0], q3[1], q3[2]);
         a.code[t0 + k] = code;
       }
     }
@@ -1733,7 +1789,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
           for (int j = 0; j < nf; ++j) r += s.c.face[j] < f ? 1u : 0u;
           const int p = (int)(f >> 16), u = (int)((f >> 8) & 255u), w = (int)(f & 255u);
           tri[t0 + r] = make_int3((int)s.gid[p], (int)s.gid[u], (int)s.gid[w]);
-          a.label[t0 + r] = r3_label36<G>(a, s, p, u, w);
+          a.label[t0 + r] = r3_node_label<G>(a, s, p, u, w);
           a.code[t0 + r] = code;
         }
       }

@@ -560,13 +560,13 @@ struct TState {
 // of the image, the sum is below 2^31.
 SBMT_DEV float zq_float(int a, int b) {
   const u64 v = ((u64)(i64)a << 32) + (u64)(i64)b * 7439101573ull + (u64)(((i64)b * 2227873595ll) >> 32);
-  return __fmul_rn((float)(i64)v, 2.3283064365386963e-10f);
+  return i64_float((i64)v, -32);
 }
 
 // zsign with a single-precision estimate in front: its error is below 2.4e-7
 // (|a| + |b| sqrt3) (three roundings of 2^-24 a term and one of the sum)
 SBMT_DEV int zsign_fast(Zq v) {
-  const float fa = (float)v.a, fb = (float)v.b * 1.7320508f, t = fa + fb;
+  const float fa = i64_float(v.a), fb = i64_float(v.b) * 1.7320508f, t = fa + fb;
   if (fabsf(t) > 4e-7f * (fabsf(fa) + fabsf(fb))) return t > 0.0f ? 1 : -1;
   return zsign(v);
 }
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(64, TG_OCC) k_tierg_group_b(const __grid_const
     const int n = tg_gather<G>(g, cg, rec, live, J.raw + rec.pair_lo, J.segs, J.ev, s, me, &A);
     if (live && n < 0 && me.l == 0) tierg_over(J, rec.cell);
     // every point of a cell lies within M = 6p scaled units of its corner A
-    const float M = (float)(6 * g.p);
+    const float M = (float)(6 * (int)g.p);
     const LatGeo<G> geo{&s, M * M};
     g_greedy<G, false>(s.c, geo, max(n, 0));
     if (n > 0) {
@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(32 * WWARPS) k_tierg_warp_b(const __grid_const
       continue;
     }
     // cell-local coordinates are bounded by the cell extent M = 6p scaled units
-    const float M = (float)(6 * g.p);
+    const float M = (float)(6 * (int)g.p);
     greedy_faces<N>(s, lane, boundary_count(rec), OriFiltered<N>{&s, 8e-6f * M * M}, 1e-4f * M * M);
     write_patch<N>(g, J.img, J.pitch, J.dtype, cg, rec, s, lane, J.tri, J.label, J.code, J.xy, J.cp.xy0,
                    jc(J, JC_ERR));

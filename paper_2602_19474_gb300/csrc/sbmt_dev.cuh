@@ -84,6 +84,15 @@ SBMT_HD float i2f(i64 v) {
   return (float)v;
 #endif
 }
+// the float of any 64-bit integer, times 2^e: its upper 32 bits converted on
+// the 32-bit path (a conversion from 64 bits runs on the FP64 pipe, 19 clocks
+// a warp); within 2^-24 + 2^-31 of it
+SBMT_DEV float i64_float(i64 v, int e = 0) {
+  const u64 u = v < 0 ? 0ull - (u64)v : (u64)v;
+  const int s = max(0, 32 - __clzll((long long)u));
+  const float f = (float)(u32)(u >> s) * __int_as_float((127 + s + e) << 23);
+  return v < 0 ? -f : f;
+}
 SBMT_HD i64 floor_i64(float x) {
 #ifdef __CUDA_ARCH__
   if (fabsf(x) < 2.0e9f) return (i64)(int)floorf(x);
@@ -250,7 +259,7 @@ SBMT_DEV Pq corner_pt(const GridP& g, i64 cx, i64 cy) {
 // strip row holding a point of height y (never on a grid line)
 SBMT_HD i64 strip_of(const GridP& g, Zq y) {
   // y_j = oy + 3 p j sqrt3
-  i64 j = floor_i64((i2f(y.a - g.oy) + i2f(y.b) * 1.7320508f) / (3.0f * (float)g.p * 1.7320508f));
+  i64 j = floor_i64((i2f(y.a - g.oy) + i2f(y.b) * 1.7320508f) / (3.0f * i2f(g.p) * 1.7320508f));
   while (zcmp(zq(g.oy, 3 * g.p * j), y) > 0) --j;
   while (zcmp(zq(g.oy, 3 * g.p * (j + 1)), y) <= 0) ++j;
   return j;
