@@ -1299,7 +1299,7 @@ struct R3State {
 
 // The kernel is long: what it needs rarely or in several places is kept out of
 // line, and short loops stay loops (inlined and unrolled it waited for
-// instructions in 18 of 27 cycles per issue: 595 us against 527).
+// instructions in 18 of 27 cycles per issue: 595 us against 527, before the barriers below).
 __device__ __noinline__ int r3_late(const double* x, const double* y, int u, int v, int w) {
   return r3_sgn(r3_orient(make_double2(x[u], y[u]), make_double2(x[v], y[v]), make_double2(x[w], y[w])));
 }
@@ -1406,10 +1406,17 @@ SBMT_DEV int r3_tier_t(const R3State<G>& s, int ni, int ne, int np, int n0, int 
   return -1;
 }
 
-// LIST: which list; REC: whether its cells come with the count pass's records
-template <int G, int LIST, bool REC>
-__global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
-  constexpr int C_ = 64 / G;
+// LIST: which list; REC: whether its cells come with the count pass's records.
+// The block barriers order nothing (a group's data is its own warp's): they keep the
+// warps of a block in the same part of this long kernel, so that they share what
+// the instruction caches hold.  With blocks of two warps, each warp at a place of
+// its own, 13 of 22 cycles per issue went to waiting for instructions: 527 us for the
+// 1.9e5 cut cells of 4096^2 labels, 454 with four warps to a block, 425 with six, 404 with
+// seven (the most whose groups fit 48 KB of shared memory; four blocks an SM).
+constexpr int CELL_T = 224;
+template <int G, int LIST, bool REC, int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_r3_cells(R3Args a) {
+  constexpr int C_ = T / G;
   __shared__ R3State<G> sm[C_];
   const GLane<G> me;
   R3State<G>& s = sm[threadIdx.x / G];
@@ -1417,7 +1424,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
   u32 ngc = 0, ngt = 0;
   for (u32 q = blockIdx.x * C_ + threadIdx.x / G;; q += gridDim.x * C_) {
     bool live = q < total;
-    if (!__any_sync(0xffffffffu, live)) break;
+    if (!__syncthreads_or(live)) break;
     u32 err = 0, c = 0;
     int cnt[3] = {0, 0, 0}, nb[3] = {-1, -1, -1}, ne, ni;
     u64 entry = 0;  // this lane's event or inside vertex
@@ -1515,7 +1522,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
       es = ddv(alongx ? dsb(ex, P.x) : dsb(ey, P.y), alongx ? dx : dy);
       s.s[me.l] = es;
     }
-    __syncwarp();
+    __syncthreads();
     // rank on the edge by (s, kind, k, m); node order runs counter-clockwise
     int node = -1;
     u32 gid = 0;
@@ -1557,7 +1564,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
       if (err) atomicOr(a.err, err);
       live = false;
     }
-    __syncwarp();
+    __syncthreads();
     R3Corner Sx[3], Sy[3];
 #pragma unroll
     for (int t = 0; t < 3; ++t)
@@ -1678,7 +1685,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
       if (err) atomicOr(a.err, err);
       live = false;
     }
-    __syncwarp();
+    __syncthreads();
     // Alg. 1 mask (a corner on a piece sets both its edges, an event its
     // edge, an edge on a boundary run its own bit, bit 0 an inside vertex)
     // and the (m, n) class of the first two pieces
@@ -1736,7 +1743,7 @@ __global__ void __launch_bounds__(64, 16) k_r3_cells(R3Args a) {
     }
     // Tier-G
     const bool tg = live && key == 0;
-    __syncwarp();
+    __syncthreads();
     if (!__any_sync(0xffffffffu, tg)) continue;
     // constraints: the pieces and the boundary cycle, each an edge as the
     // rule's list has it (above 12 nodes the smaller node first)
@@ -1999,10 +2006,10 @@ int launch_r3_emit(const R3Args& a, cudaStream_t st) {
   const unsigned g = (unsigned)std::min<u64>((a.nt + 255) / 256, 152 * 16);
   k_r3_emit_uncut<<<std::max(g, 1u), 256, 0, st>>>(a);
   k_r3_tierg<<<152 * 8, 32 * R3G_WARPS, 0, st>>>(a);
-  k_r3_cells<32, 4, false><<<152 * 5, 64, 0, st>>>(a);
-  k_r3_cells<32, 2, true><<<152 * 5, 64, 0, st>>>(a);
-  k_r3_cells<16, 1, true><<<152 * 10, 64, 0, st>>>(a);
-  k_r3_cells<8, 0, true><<<152 * 16, 64, 0, st>>>(a);
+  k_r3_cells<32, 4, false, 64><<<152 * 5, 64, 0, st>>>(a);
+  k_r3_cells<32, 2, true, 64><<<152 * 5, 64, 0, st>>>(a);
+  k_r3_cells<16, 1, true, 64><<<152 * 10, 64, 0, st>>>(a);
+  k_r3_cells<8, 0, true, CELL_T><<<152 * (1024 / CELL_T), CELL_T, 0, st>>>(a);
   return 6;
 }
 
