@@ -47,7 +47,7 @@
 // One thread per cut cell rebuilt the cell's graph in double formulas, twice
 // for a Tier-G cell, with 3 of 32 lanes active: 1.20 + 0.71 ms for the 1.9e5 cut
 // cells of a 4096^2 label image at h = 2.  With the records, and one event,
-// line, candidate or triangle per lane, 0.59 ms (0.54 -> 0.62 ms for the count
+// line, candidate or triangle per lane, 0.40 ms (0.38 ms for the count
 // that writes them).
 #include "sbmt_cell.cuh"
 #include "sbmt_greedy.cuh"
@@ -269,69 +269,11 @@ SBMT_DEV u64 r3_entry(int edge, int kind, int m, int k) {
   return (u64)(u32)m | (u64)(u32)k << 16 | (u64)(edge << 2 | kind) << 32;
 }
 
-// the number of events of the edge from P (its lower-id end) to Q, or -1
-// past R3_MAXE, through the filters (the count pass's form: positions are
-// not needed there); ev receives the events (r3_entry), for the record and for
-// the corner found on both line families to count once
-SBMT_DEV int r3_edge_count(const R3Args& a, double2 P, double2 Q, int edge, u64* ev) {
-  int n = 0;
-  const bool hz = P.y == Q.y, vt = P.x == Q.x;
-  const R3Split px = r3_split(P.x), py = r3_split(P.y), qx = r3_split(Q.x), qy = r3_split(Q.y);
-  const float dxf = r3_fdiff(qx, px), dyf = r3_fdiff(qy, py);
-  const float D = fmaxf(fabsf(dxf), fabsf(dyf));
-  const bool grid = r3_corner_ends(px, py, qx, qy, D);
-  if (!hz) {
-    // horizontal lines y = k - 1/2 strictly between P.y and Q.y
-    const float sl = __fdiv_rn(dxf, dyf);
-    int k0;
-    const int nk = r3_lines(py, qy, a.H, &k0);
-    for (int k = k0; k < k0 + nk; ++k) {
-      const float hp = r3_i2f((int)(k - py.i)) - 0.5f;
-      const float w = __fadd_rn(px.f, __fmul_rn(__fsub_rn(hp, py.f), sl));
-      const float z = __fadd_rn(w, 0.5f);
-      const int zi = r3_ffloor(z);
-      const float fr = __fsub_rn(z, r3_i2f(zi)), T = r3_cross_tol(D, sl, w);
-      i64 j;
-      bool corner = false;
-      if (fr > T && fr < 1.0f - T) j = px.i + zi;
-      else if (grid) r3_cross_corners(py, px, qy, qx, k, &j, &corner);
-      else r3_cross_exact(P, Q, (double)k - 0.5, false, &j, &corner);
-      if (corner ? r3_corner_event(a, j, k, hz, vt) : r3_hb(a, j, k)) {
-        if (n == R3_MAXE) return -1;
-        ev[n++] = r3_entry(edge, corner ? 2 : 0, (int)j, (int)k);
-      }
-    }
-  }
-  if (!vt) {
-    // vertical lines x = m - 1/2 strictly between P.x and Q.x
-    const float sl = __fdiv_rn(dyf, dxf);
-    int m0;
-    const int nm = r3_lines(px, qx, a.W, &m0);
-    for (int m = m0; m < m0 + nm; ++m) {
-      const float hp = r3_i2f((int)(m - px.i)) - 0.5f;
-      const float w = __fadd_rn(py.f, __fmul_rn(__fsub_rn(hp, px.f), sl));
-      const float z = __fadd_rn(w, 0.5f);
-      const int zi = r3_ffloor(z);
-      const float fr = __fsub_rn(z, r3_i2f(zi)), T = r3_cross_tol(D, sl, w);
-      i64 j;
-      bool corner = false;
-      if (fr > T && fr < 1.0f - T) j = py.i + zi;
-      else if (grid) r3_cross_corners(px, py, qx, qy, m, &j, &corner);
-      else r3_cross_exact(P, Q, (double)m - 0.5, true, &j, &corner);
-      if (corner) {
-        bool dup = false;
-        for (int t = 0; t < n; ++t)
-          if (ev[t] == r3_entry(edge, 2, (int)m, (int)j)) dup = true;
-        if (dup || !r3_corner_event(a, m, j, hz, vt)) continue;
-      } else if (!r3_vb(a, m, j)) {
-        continue;
-      }
-      if (n == R3_MAXE) return -1;
-      ev[n++] = r3_entry(edge, corner ? 2 : 1, (int)m, (int)j);
-    }
-  }
-  return n;
+SBMT_DEV bool r3_same(double a, double b) {  // a == b without an FP64 compare (finite numbers)
+  const i64 p = __double_as_longlong(a), q = __double_as_longlong(b);
+  return p == q || ((p | q) << 1) == 0;
 }
+
 
 // the cell's two chord ends on a pixel line (vert: the vertical line x = c0,
 // else the horizontal y = c0): (position along the line, source = corner 0..2
@@ -561,10 +503,6 @@ struct R3Found {
 struct R3Geo2 {  // the cell in the filters' numbers
   R3Split x[3], y[3];
 };
-SBMT_DEV bool r3_same(double a, double b) {  // a == b without an FP64 compare (finite numbers)
-  const i64 p = __double_as_longlong(a), q = __double_as_longlong(b);
-  return p == q || ((p | q) << 1) == 0;
-}
 
 // the cell's events into F (up to R3_LIST of them) and their number per edge,
 // the same in every lane; each through the float filter of r3_cross_tol, with
@@ -903,25 +841,102 @@ SBMT_DEV u32* r3_list(const R3Args& a, int q, u32 i) {
 // a cell for which it is used up is listed without a record.
 constexpr int R3_HEAD = 3;
 
+// the events on the cell's edges, through the filters (the count pass's form:
+// positions are not needed there): their number, or -1 past R3_MAXE on an edge; ev
+// receives them (r3_entry), cnt their number per edge.  One loop over the lines
+// of all three edges: with a loop an edge and direction, a warp ran the longest of
+// each (437 us for the candidates of 4096^2 labels, 397 this way, 382 with registers
+// for six blocks an SM instead of four).
+SBMT_DEV int r3_events_t(const R3Args& a, const R3Cell& C, u64* ev, int (&cnt)[3]) {
+  R3Split sx[3], sy[3];
+#pragma unroll
+  for (int t = 0; t < 3; ++t) sx[t] = r3_split(C.K[t].x), sy[t] = r3_split(C.K[t].y);
+  // per edge: its lower-id end first, the differences, whether between two pixel corners
+  float dx[3], dy[3], D[3];
+  bool fwd[3], grid[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const int w = j == 2 ? 0 : j + 1;
+    fwd[j] = C.id[j] < C.id[w];
+    dx[j] = r3_fdiff(sx[w], sx[j]), dy[j] = r3_fdiff(sy[w], sy[j]);
+    D[j] = fmaxf(fabsf(dx[j]), fabsf(dy[j])), grid[j] = r3_corner_ends(sx[j], sy[j], sx[w], sy[w], D[j]);
+  }
+  int ne = 0;
+  cnt[0] = cnt[1] = cnt[2] = 0;
+#pragma unroll 1
+  for (int vert = 0; vert < 2; ++vert) {
+    int first[3], num[3];
+    float slope[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int w = j == 2 ? 0 : j + 1;
+      num[j] = vert ? r3_lines(sx[j], sx[w], a.W, &first[j]) : r3_lines(sy[j], sy[w], a.H, &first[j]);
+      slope[j] = vert ? __fdiv_rn(dy[j], dx[j]) : __fdiv_rn(dx[j], dy[j]);  // (not used without lines)
+    }
+    const int total = num[0] + num[1] + num[2], ne_h = ne;  // vertical lines: the corners found on the horizontal ones count once
+#pragma unroll 1
+    for (int i = 0; i < total; ++i) {
+      const int j = i < num[0] ? 0 : i < num[0] + num[1] ? 1 : 2;
+      const int line = i - (j > 0 ? num[0] : 0) - (j > 1 ? num[1] : 0) + (j == 0 ? first[0] : j == 1 ? first[1] : first[2]);
+      const bool fw = j == 0 ? fwd[0] : j == 1 ? fwd[1] : fwd[2];
+      const int pi = fw ? j : (j == 2 ? 0 : j + 1), qi = fw ? (j == 2 ? 0 : j + 1) : j;
+      const R3Split px = pi == 0 ? sx[0] : pi == 1 ? sx[1] : sx[2], py = pi == 0 ? sy[0] : pi == 1 ? sy[1] : sy[2];
+      const R3Split& pc = vert ? px : py;  // across the line, and along it
+      const R3Split& pl = vert ? py : px;
+      const float sl = j == 0 ? slope[0] : j == 1 ? slope[1] : slope[2], Dj = j == 0 ? D[0] : j == 1 ? D[1] : D[2];
+      const float hp = r3_i2f((int)(line - pc.i)) - 0.5f;
+      const float w = __fadd_rn(pl.f, __fmul_rn(__fsub_rn(hp, pc.f), sl));
+      const float z = __fadd_rn(w, 0.5f);
+      const int zi = r3_ffloor(z);
+      const float fr = __fsub_rn(z, r3_i2f(zi)), tol = r3_cross_tol(Dj, sl, w);
+      i64 at;
+      bool corner = false;
+      if (fr > tol && fr < 1.0f - tol) {
+        at = pl.i + zi;
+      } else {
+        const R3Split qx = qi == 0 ? sx[0] : qi == 1 ? sx[1] : sx[2], qy = qi == 0 ? sy[0] : qi == 1 ? sy[1] : sy[2];
+        if (j == 0 ? grid[0] : j == 1 ? grid[1] : grid[2]) {
+          r3_cross_corners(pc, pl, vert ? qx : qy, vert ? qy : qx, line, &at, &corner);
+        } else {
+          const double2 P = pi == 0 ? C.K[0] : pi == 1 ? C.K[1] : C.K[2], Q = qi == 0 ? C.K[0] : qi == 1 ? C.K[1] : C.K[2];
+          r3_cross_exact(P, Q, (double)line - 0.5, vert, &at, &corner);
+        }
+      }
+      const i64 m = vert ? line : at, k = vert ? at : line;
+      const u64 entry = r3_entry(j, corner ? 2 : vert, (int)m, (int)k);
+      bool found;
+      if (corner) {
+        const double2 P = pi == 0 ? C.K[0] : pi == 1 ? C.K[1] : C.K[2], Q = qi == 0 ? C.K[0] : qi == 1 ? C.K[1] : C.K[2];
+        bool dup = false;
+        if (vert)
+          for (int t = 0; t < ne_h; ++t) dup |= ev[t] == entry;
+        found = !dup && r3_corner_event(a, m, k, r3_same(P.y, Q.y), r3_same(P.x, Q.x));
+      } else {
+        found = vert ? r3_vb(a, m, k) : r3_hb(a, m, k);
+      }
+      if (!found) continue;
+      if ((j == 0 ? cnt[0] : j == 1 ? cnt[1] : cnt[2]) == R3_MAXE) return -1;
+      ev[ne++] = entry;
+      cnt[0] += j == 0, cnt[1] += j == 1, cnt[2] += j == 2;
+    }
+  }
+  return ne;
+}
+
 // the candidates: events on the edges, inside vertices, the cells beside
 // the edges that carry events.  (Eight lanes a candidate, as in k_r3_cells,
-// took 0.99 ms against 0.54: here the cells are alike, and what every lane
+// took 0.99 ms against 0.44: here the cells are alike, and what every lane
 // needs is computed once.)
-__global__ void __launch_bounds__(128) k_r3_count(R3Args a) {
+__global__ void __launch_bounds__(128, 6) k_r3_count(R3Args a) {
   u64 ev[3 * R3_MAXE + R3_MAXI];
   const u32 n = *a.ncand;
   for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
     const u32 c = a.cand[q];
     const R3Cell C = r3_load_k(a, c);
-    int ne = 0, cnt[3];
-    bool bad = false;
-    for (int j = 0; j < 3; ++j) {
-      const int u = j, w = j == 2 ? 0 : j + 1;
-      const bool fwd = C.id[u] < C.id[w];
-      cnt[j] = r3_edge_count(a, fwd ? C.K[u] : C.K[w], fwd ? C.K[w] : C.K[u], j, ev + ne);
-      if (cnt[j] < 0) bad = true;
-      else ne += cnt[j];
-    }
+    int cnt[3];
+    const int found = r3_events_t(a, C, ev, cnt);
+    const bool bad = found < 0;
+    const int ne = bad ? 0 : found;
     const int ni = bad ? 0 : r3_inside(a, C, ev + ne);
     if (bad || ni == -1 || 3 + ne + ni > R3_MAXN) {
       atomicOr(a.err, R3_CAPACITY);
