@@ -230,7 +230,7 @@ struct Lane {
 // launch parameters of the batched path (chosen per size class by the tuner)
 struct Tune {
   int cut_blocks_per_sm = 8;     // persistent cut-cell kernel, 128 threads a block
-  int tierg_blocks_per_sm = 24;  // persistent Tier-G thread kernel, 64 threads a block
+  int tierg_blocks_per_sm = 24;  // Tier-G by groups of 8 lanes, 64 threads a block
   int fork = 1;                  // Tier-G and the large registry buckets on side streams
   int graph = 0;                 // the emission phase captured into a CUDA graph
 };

@@ -151,3 +151,17 @@ def test_a_device_wait_that_runs_out_is_reported_and_the_context_survives():
     assert e.value.code == sb.SBMT_ETIMEDOUT
     g = _fetch(c, sb.mesh_bitmap(c, img, 2))
     assert_same_mesh(g, oracle.mesh_bitmap(img, 2, 1), 2.0, W=img.shape[1])
+
+
+@pytest.mark.parametrize("count", [3, 6, 9])
+def test_emission_by_one_to_eight_warps_a_bucket(count):
+    """The emission gives a bucket of 1024 cells 8, 4, 2 or 1 warps, fewer with
+    more buckets in the call: 8 for one image of 283 buckets, 4, 2 and 1 for three,
+    six and nine of them.  The meshes have to be the same."""
+    c = ctx()
+    img = synth.voronoi_labels(size=707, nseeds=60)
+    single = _fetch(c, sb.mesh_bitmap(c, img, 2, 1))
+    for m in sb.mesh_batch(c, [img] * count, 2):
+        got = _fetch(c, m)
+        for key in ("tri", "label", "code", "xy"):
+            assert np.array_equal(got[key], single[key]), key

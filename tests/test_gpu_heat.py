@@ -143,3 +143,26 @@ def test_block_edges_and_long_rows(side, fan):
     uo, po = H.heat(xy, tri, np.full(len(tri), 0xFFFF), 0xFFFF, 3.0, 0.1, 3, 2.0, 1.0, 6.0)
     assert np.abs(u - uo).max() <= 1e-8 * 100.0
     assert np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
+
+
+@pytest.mark.parametrize("side", [831, 832])
+def test_vectors_on_chip_and_beyond(side):
+    """The largest square grid whose vectors fit the blocks' shared memory (152
+    blocks of 4544 rows), and the next one, which keeps them in L2: the first step
+    satisfies the oracle's backward-Euler equation.  The solver stops at a relative
+    residual of 1e-10; the recurrences drift from the true residual by some 1e-14."""
+    import scipy.sparse as sp
+
+    j, i = np.mgrid[0:side, 0:side]
+    xy = np.stack([i.ravel(), j.ravel() * 0.9], 1).astype(float)
+    a = (j[:-1, :-1] * side + i[:-1, :-1]).ravel()
+    tri = np.concatenate([np.stack([a, a + 1, a + side + 1], 1), np.stack([a, a + side + 1, a + side], 1)]).astype(np.int32)
+    m = sb.mesh_import(ctx(), xy, tri)
+    alpha, dt = 500.0, 0.01
+    u, peaks, its = run_gpu(m, 0xFFFF, alpha, dt, 1, 400.0, 380.0, 60.0, tol=1e-10)
+    sb.mesh_release(ctx(), m)
+    K, M = H.stiffness(xy, tri, len(xy)), H.lumped_mass(xy, tri, len(xy))
+    rhs = M * H.pulse(xy, 400.0, 380.0, 60.0, 100.0)
+    res = sp.diags(M) @ u + alpha * dt * (K @ u) - rhs
+    assert np.linalg.norm(res) <= 2e-10 * np.linalg.norm(rhs), np.linalg.norm(res) / np.linalg.norm(rhs)
+    assert 0 < peaks[0] <= 100.0
