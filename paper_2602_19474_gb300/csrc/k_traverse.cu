@@ -222,7 +222,9 @@ SBMT_DEV double int_double(int v) {
 SBMT_DEV double2 event_xy(const GridP& g, const Event& e) {
   const bool hx = e.xb != 0;  // x is the irrational one (or both are rational)
   const int a1 = hx ? e.xa : e.ya, b1 = hx ? e.xb : e.yb, a0 = hx ? e.ya : e.xa, b0 = hx ? e.yb : e.xb;
-  const double irr = (int_double(a1) + int_double(b1) * 1.7320508075688772935) * g.invS;
+  // (one rounding, stated: left to the compiler, the product was rounded too, which
+  // near x = 0 loses dozens of units in the last place)
+  const double irr = __fma_rn(int_double(b1), 1.7320508075688772935, int_double(a1)) * g.invS;
   const double rat = (b0 == 0 ? int_double(a0) : zdouble(zq(a0, b0))) * g.invS;
   return hx ? make_double2(irr, rat) : make_double2(rat, irr);
 }

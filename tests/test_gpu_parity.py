@@ -133,3 +133,34 @@ def test_tier_g_cells_of_every_group_size(seed, h, sigma, sizes):
     cut = o["cut"][o["cut"][:, 4] == 1]
     have = set((cut[:, 2] + 2 - cut[:, 3]).tolist())
     assert have.issuperset(sizes), sorted(have)
+
+
+@pytest.mark.parametrize("hn,hd", [(2, 1), (4, 1), (2, 3)])
+def test_irrational_event_coordinates_to_the_bit(hn, hd):
+    """An event's irrational coordinate is (a + b sqrt3) / S with whole a, b and S
+    = 6 h_den: one rounding for the sum (with the double next to sqrt3), one for the
+    product with 1 / S."""
+    from fractions import Fraction
+
+    import paper_2602_19474_gb300 as sb
+    from gpu_util import ctx
+
+    img = synth.voronoi_labels(size=48, nseeds=9)
+    c = ctx()
+    m = sb.mesh_bitmap(c, img, hn, hd)
+    xy = sb.view_numpy(sb.mesh_query(c, m, -1))["xy"].copy()
+    sb.mesh_release(c, m)
+    S, r3 = 6 * hd, 1.7320508075688772935
+    b = np.arange(-200 * hd, 200 * hd + 1)
+    b = b[b != 0]
+    seen = 0
+    for x in xy[:, 0]:
+        if abs(x * S - round(x * S)) < 1e-6:
+            continue
+        a = np.rint(x * S - b * r3)
+        d = np.abs(a + b * r3 - x * S)
+        k = int(d.argmin())
+        assert d[k] < 1e-9
+        assert float(Fraction(int(a[k])) + Fraction(int(b[k])) * Fraction(r3)) * (1.0 / S) == x
+        seen += 1
+    assert seen > 100
