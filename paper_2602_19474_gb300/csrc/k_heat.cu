@@ -180,31 +180,51 @@ __global__ void __launch_bounds__(HB) k_heat_fill(const HeatTri* rec, u32 n, dou
 }
 
 // each row's entries of one column summed, in place at the row's start;
-// mcnt: the merged counts
-__global__ void __launch_bounds__(HB) k_heat_merge(u32 n, const u32* rowptr, u32* col, double* val, u32* mcnt) {
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const u32 e0 = rowptr[i], e1 = rowptr[i + 1];
-    u32 m = 0;
-    for (u32 e = e0; e < e1; ++e) {
-      const u32 c = col[e];
-      const double v = val[e];
-      u32 k = 0;
-      while (k < m && col[e0 + k] != c) ++k;
-      if (k < m) {
-        val[e0 + k] += v;
-      } else {
-        col[e0 + m] = c, val[e0 + m] = v;
-        ++m;
-      }
+// mcnt: the merged counts.  A row of at most MR entries (two per neighbour) is
+// merged and ordered in a column of shared memory of its thread's own: in
+// place, each step waited for the one before through the cache (128 us for
+// 0.38e6 rows, 47 this way).
+constexpr int MR = 16, MT = 192;
+SBMT_DEV u32 merge_row(u32 n, u32* col, double* val, u32 step) {
+  u32 m = 0;
+  for (u32 e = 0; e < n; ++e) {
+    const u32 c = col[e * step];
+    const double v = val[e * step];
+    u32 k = 0;
+    while (k < m && col[k * step] != c) ++k;
+    if (k < m) {
+      val[k * step] += v;
+    } else {
+      col[m * step] = c, val[m * step] = v;
+      ++m;
     }
-    // the row's entries by column, so that each product sums them in one order
-    for (u32 a = 1; a < m; ++a)
-      for (u32 b = a; b > 0 && col[e0 + b] < col[e0 + b - 1]; --b) {
-        const u32 tc = col[e0 + b];
-        col[e0 + b] = col[e0 + b - 1], col[e0 + b - 1] = tc;
-        const double tv = val[e0 + b];
-        val[e0 + b] = val[e0 + b - 1], val[e0 + b - 1] = tv;
-      }
+  }
+  // the row's entries by column, so that each product sums them in one order
+  for (u32 a = 1; a < m; ++a) {
+    const u32 c = col[a * step];
+    const double v = val[a * step];
+    u32 b = a;
+    for (; b > 0 && c < col[(b - 1) * step]; --b)
+      col[b * step] = col[(b - 1) * step], val[b * step] = val[(b - 1) * step];
+    col[b * step] = c, val[b * step] = v;
+  }
+  return m;
+}
+__global__ void __launch_bounds__(MT) k_heat_merge(u32 n, const u32* rowptr, u32* col, double* val, u32* mcnt) {
+  __shared__ double s_val[MR][MT];
+  __shared__ u32 s_col[MR][MT];
+  u32* sc = &s_col[0][threadIdx.x];
+  double* sv = &s_val[0][threadIdx.x];
+  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const u32 e0 = rowptr[i], cnt = rowptr[i + 1] - e0;
+    if (cnt > MR) {
+      mcnt[i] = merge_row(cnt, col + e0, val + e0, 1);
+      continue;
+    }
+#pragma unroll 4
+    for (u32 e = 0; e < cnt; ++e) sc[e * MT] = col[e0 + e], sv[e * MT] = val[e0 + e];
+    const u32 m = merge_row(cnt, sc, sv, MT);
+    for (u32 e = 0; e < m; ++e) col[e0 + e] = sc[e * MT], val[e0 + e] = sv[e * MT];
     mcnt[i] = m;
   }
 }
@@ -660,7 +680,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     launches += 1 + launch_scan(flag, rowptr, n, sscr, st);
     if (cudaMemcpyAsync(flag, rowptr, 4 * (size_t)n, cudaMemcpyDeviceToDevice, st)) return -1;
     k_heat_fill<<<gr, HB, 0, st>>>(rec, nr, tau, flag, col, val);
-    k_heat_merge<<<gv, HB, 0, st>>>(n, rowptr, col, val, mcnt);
+    k_heat_merge<<<(unsigned)std::min<u64>((n + MT - 1) / MT, 152 * 6), MT, 0, st>>>(n, rowptr, col, val, mcnt);
     launches += 2;
   }
   bool converged = true;
