@@ -890,8 +890,10 @@ int launch_tierg(const Job& oj, const Job* jobs, const u32* bpre, int njobs, u32
   k_gorder_b<ONE><<<nblocks, 32 * GORDER_W, 0, st>>>(oj, jobs, bpre, njobs, bp.bd, bp.olist, bp.slist, bp.wlist,
                                                      bp.wlast);
   k_tierg_group_b<ONE, 8><<<152 * blocks_per_sm, 64, 0, st>>>(oj, jobs, &bp.bd->nolist, bp.olist);
-  // the larger cells on their own stream when given one, beside the 8-lane
-  // groups, the largest first
+  // the larger cells on their own stream when given one, after the 8-lane
+  // groups and beside the emission, the largest first.  (Beside the groups too, from the
+  // order alone: 1 to 2% faster with few cells, but 2.06 against 2.04 ms on
+  // 8192^2 labels, where they take room from both.)
   if (st2) {
     if (cudaEventRecord(ev_order, st) != cudaSuccess || cudaStreamWaitEvent(st2, ev_order, 0) != cudaSuccess) return -1;
   }
