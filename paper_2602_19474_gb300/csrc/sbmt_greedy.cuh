@@ -121,10 +121,14 @@ SBMT_DEV void g_greedy(GCell<G>& s, const Geo& geo, int n) {
   const int half = n >> 1;
   const float tol = geo.tol();
   const int nmax = warp_max(n), hmax = nmax >> 1;
-  // sets of the pairs (u, u + d), d up to n / 2 (the middle one twice when n
-  // is even: the same values)
+  // sets of the pairs (u, u + d), d up to n / 2; when n is even, the pairs half the
+  // cycle apart by their lower vertex's lane alone.  A pair's L and Z must come
+  // from one lane: the float determinants taken from its two ends round
+  // differently, and at the edge of the band one decides a vertex that the other
+  // leaves undecided.
+  auto mine = [&](int d) { return u < n && d <= half && !(2 * d == n && u >= d); };
   for (int d = 1; d <= hmax; ++d) {
-    if (u < n && d <= half) {
+    if (mine(d)) {
       int v = u + d;
       if (v >= n) v -= n;
       const float2 pu = s.f[u], pv = s.f[v];
@@ -162,7 +166,7 @@ SBMT_DEV void g_greedy(GCell<G>& s, const Geo& geo, int n) {
   const u32 eu = u < n ? s.em[u] : 0u;
   const int nce = n ? s.nce : 0;
   for (int d = 1; d <= hmax; ++d) {
-    bool ok = u < n && d <= half && !(2 * d == n && u >= d);
+    bool ok = mine(d);
     int p = 0, q = 0;
     if (ok) {
       int v = u + d;
