@@ -164,7 +164,10 @@ SBMT_DEV i64 r3_fix36(double v, bool* inexact) {
   *inexact = lost;
   return neg ? -f : f;
 }
-// the float of an integer |n| < 2^22, exactly: n in the mantissa of 1.5 2^23 + n
+// the float of an integer |n| < 2^22, exactly: n in the mantissa of 1.5 2^23 + n.
+// (Of larger ones it is wrong by up to millions: used only where the pixel index
+// has that range, or an edge long enough to give a larger n has a crossing
+// tolerance above 1/2, which leaves the crossing to the double formula.)
 SBMT_DEV float r3_i2f(int n) { return __fsub_rn(__int_as_float(0x4B400000 + n), 12582912.0f); }
 // the nearest integer to a float |z| < 2^22, and the floor
 SBMT_DEV int r3_fint(float z) { return __float_as_int(__fadd_rn(z, 12582912.0f)) - 0x4B400000; }
@@ -219,8 +222,12 @@ SBMT_DEV float r3_fdiff(const R3Split& q, const R3Split& p) {
 // 2^-24 (8 + 8|s| + 7 D + |w|) of the real w of the double inputs (D: the
 // edge's larger extent; |A| is below the extent across the line, |A s|
 // below the extent along it), and the double formula within
-// 2^-53 (|position| + 3 D) of that real value; T (below) is above their
-// sum at every coordinate up to 2^24.
+// 2^-53 (|position| + 3 D) of that real value.  Where the line, or a pixel
+// corner compared with w, is 2^23 or more from P (cells reaching millions of
+// pixels outside the image), its distance in float (r3_half) is within 2^-23 of
+// it: 2 more of D and of |w|.  T (below) is above the sum at every coordinate up
+// to 2^24.
+SBMT_DEV float r3_half(i64 n) { return __fsub_rn((float)(int)n, 0.5f); }  // n - 1/2, |n| <= 2^24 + 2^15
 SBMT_DEV float r3_cross_tol(float D, float s, float w) {
   return 6.0e-7f * (D + fabsf(s) + 2.0f * fabsf(w) + 3.0f) + 1.5e-8f;
 }
@@ -421,14 +428,14 @@ __device__ __noinline__ int r3_end_cmp_exact(const R3Cell& C, int src, i64 cx, i
 // formula
 SBMT_DEV bool r3_end_below(const R3Cell& C, const R3Split* sx, const R3End& e, i64 cx, int cy) {
   if (e.src < 3) return r3_lt(sx[e.src], cx);
-  const float h = r3_i2f((int)(cx - e.b)) - 0.5f;
+  const float h = r3_half(cx - e.b);
   if (__fsub_rn(h, e.w) > e.T) return true;
   if (__fsub_rn(e.w, h) > e.T) return false;
   return r3_end_cmp_exact(C, e.src, cx, cy) < 0;
 }
 SBMT_DEV bool r3_end_above(const R3Cell& C, const R3Split* sx, const R3End& e, i64 cx, int cy) {
   if (e.src < 3) return r3_gt(sx[e.src], cx);
-  const float h = r3_i2f((int)(cx - e.b)) - 0.5f;
+  const float h = r3_half(cx - e.b);
   if (__fsub_rn(e.w, h) > e.T) return true;
   if (__fsub_rn(h, e.w) > e.T) return false;
   return r3_end_cmp_exact(C, e.src, cx, cy) > 0;
@@ -469,7 +476,7 @@ SBMT_DEV int r3_inside(const R3Args& a, const R3Cell& C, u64* out) {
       if (!((lt[u] && gt[v]) || (lt[v] && gt[u]))) continue;
       if (ne == 2) return -2;
       const int P = C.id[u] < C.id[v] ? u : v;
-      const float hP = r3_i2f((int)(cy - sy[P].i)) - 0.5f;
+      const float hP = r3_half(cy - sy[P].i);
       const float w = __fadd_rn(sx[P].f, __fmul_rn(__fsub_rn(hP, sy[P].f), sl[j]));
       e[ne++] = R3End{sx[P].i, w, r3_cross_tol(D[j], sl[j], w), 3 + j};
     }
@@ -629,9 +636,9 @@ SBMT_DEV int r3_inside_g(const R3Args& a, const R3Cell& C, const R3Geo2& S, bool
           const R3Split &px = fwd ? S.x[u] : S.x[v], &py = fwd ? S.y[u] : S.y[v];
           const R3Split &qx = fwd ? S.x[v] : S.x[u], &qy = fwd ? S.y[v] : S.y[u];
           const float dxf = r3_fdiff(qx, px), dyf = r3_fdiff(qy, py), sl = __fdiv_rn(dxf, dyf);
-          const float hP = r3_i2f((int)(cy - py.i)) - 0.5f;
+          const float hP = r3_half(cy - py.i);
           const float w = __fadd_rn(px.f, __fmul_rn(__fsub_rn(hP, py.f), sl));
-          const float T = r3_cross_tol(fmaxf(fabsf(dxf), fabsf(dyf)), sl, w), h = r3_i2f((int)(cx - px.i)) - 0.5f;
+          const float T = r3_cross_tol(fmaxf(fabsf(dxf), fabsf(dyf)), sl, w), h = r3_half(cx - px.i);
           if (__fsub_rn(h, w) > T) some_below = true;
           else if (__fsub_rn(w, h) > T) some_above = true;
           else {

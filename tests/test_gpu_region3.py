@@ -361,3 +361,37 @@ def test_cells_of_every_group_size(hn, sigma, w, h):
     g = gpu_full(img, hn, 1)
     T, o = oracle_full(img, hn, 1)
     assert_same(g, o)
+
+
+FAR = [(-6.0e6, -3.0e6), (-3.0e6, -6.0e6), (-1.6e7, -0.8e7), (-4194200.0, -2.1e6), (-4194400.0, -2.1e6)]
+
+
+@pytest.mark.parametrize("fill", [0, 40])
+@pytest.mark.parametrize("mirror", [False, True])
+@pytest.mark.parametrize("far", FAR)
+def test_cells_reaching_far_outside_the_image(far, mirror, fill):
+    """An imported cell with a corner millions of pixels outside a small image
+    (2^22 px and more from the pixel corners compared with), whose long edge
+    passes a PSLG vertex at a few pixels: the inside vertices are the double
+    formula's.  With and without the count pass's record (room for one word a
+    cell: cells apart from the image make more)."""
+    img = np.zeros((24, 64), np.uint8)
+    a, b = np.array(far), np.array([60.25, 15.0])
+    d = (a - b) / np.hypot(*(a - b))
+    for s in (7.0, 13.0):  # two pixels beside the long edge, between it and the third corner's
+        px, py = np.rint(b + s * d + np.array([-2.4, 1.3])).astype(int)
+        img[py, px] = 1
+    c = b + 90.0 * d + np.array([-22.0, 12.0])
+    xy = np.stack([a, b, c])
+    if mirror:
+        xy[:, 0], img = 63.0 - xy[:, 0], np.ascontiguousarray(img[:, ::-1])
+    o = (xy[1, 0] - xy[0, 0]) * (xy[2, 1] - xy[0, 1]) - (xy[1, 1] - xy[0, 1]) * (xy[2, 0] - xy[0, 0])
+    tri = [[0, 1, 2] if o > 0 else [0, 2, 1]]
+    for k in range(fill):
+        n = len(xy)
+        xy = np.concatenate([xy, np.array([[0.0, 0.0], [1.0, 0.0], [0.0, 1.0]]) + [200.0 + 2 * k, 100.0]])
+        tri.append([n, n + 1, n + 2])
+    tri = np.array(tri, np.int32)
+    want = oracle.region3(img, xy, tri)
+    assert want["n_inside"] >= 4
+    assert_same(_imported(img, xy, tri), want)
