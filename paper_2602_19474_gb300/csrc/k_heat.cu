@@ -573,14 +573,14 @@ __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatC
         if (look) rr = s_sum[1];
       }
     }
-    // the step's peak (positive doubles order as their bits), and x for the
-    // next step's product
+    // the step's peak (positive doubles order as their bits, infinity above all;
+    // NaNs are left out, as fmax leaves them), and x for the next step's product
     unsigned long long top = 0;
     for (u32 l = tid; l < rows; l += CT) {
       const double xv = x[l];
       if (ONCHIP) h.x[row0 + l] = xv;
       const long long bits = __double_as_longlong(xv);
-      if (bits > 0) top = max(top, (unsigned long long)bits);
+      if (bits > 0 && bits <= 0x7FF0000000000000ll) top = max(top, (unsigned long long)bits);
     }
     for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
     if ((threadIdx.x & 31) == 0 && top) atomicMax(h.peak + step, top);

@@ -166,3 +166,15 @@ def test_vectors_on_chip_and_beyond(side):
     res = sp.diags(M) @ u + alpha * dt * (K @ u) - rhs
     assert np.linalg.norm(res) <= 2e-10 * np.linalg.norm(rhs), np.linalg.norm(res) / np.linalg.norm(rhs)
     assert 0 < peaks[0] <= 100.0
+
+
+@pytest.mark.parametrize("amplitude,peak", [(np.nan, 0.0), (np.inf, np.inf), (-np.inf, 0.0)])
+def test_peaks_leave_nans_out(amplitude, peak):
+    """The peak is the maximum of 0 and the values that are numbers: with an
+    amplitude that is none, or where an infinite one meets an exponential that is
+    0 (NaN far from the centre), no step iterates and the peak holds no NaN."""
+    m = sb.mesh_bitmap(ctx(), synth.disk(), 2, 1)
+    u, peaks, its = run_gpu(m, 1, 100.0, 0.05, 2, 31.5, 31.5, 0.5, amp=amplitude)
+    sb.mesh_release(ctx(), m)
+    assert peaks.tolist() == [peak, peak]
+    assert its == [0, 0] and np.isnan(u).any()
