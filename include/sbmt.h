@@ -442,6 +442,12 @@ typedef struct {
 int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* params, double* u, double* peaks,
               int32_t* iterations);
 
+/* Settings of this context's mesh_heat for tests (0: none).
+ * SBMT_HEAT_BLOCKS: the solver's launch takes at most `value` blocks, as
+ * where fewer SMs are to be had (it takes one block per SM otherwise). */
+enum { SBMT_HEAT_BLOCKS = 0 };
+int mesh_heat_debug(sbmt_ctx* ctx, int what, int value);
+
 /* Per-kernel device time, for tracing and roofline accounting (no
  * counterpart in the paper, which reports no timings).  With enable != 0
  * every kernel launch of the context is bracketed by two CUDA events on the

@@ -36,10 +36,11 @@ SBMT_PLAIN, SBMT_PREPROCESS = 0, 1
 SBMT_EXPLICIT, SBMT_COMPACT = 0, 1
 SBMT_KEEP_STAGES = 1
 SBMT_DEBUG_STALL_SCAN = 2
+SBMT_HEAT_BLOCKS = 0
 
 EXPORTS = ("mesh_create", "mesh_bitmap", "mesh_batch", "mesh_autotune", "mesh_tuning", "mesh_set_tuning",
            "mesh_query", "mesh_release", "mesh_destroy", "mesh_stage", "mesh_profile", "mesh_profile_read", "mesh_quality", "mesh_project",
-           "mesh_preprocess", "mesh_preprocess_info", "mesh_retriangulate", "mesh_import", "mesh_heat", "mesh_check", "mesh_footprint", "mesh_bound", "server_create",
+           "mesh_preprocess", "mesh_preprocess_info", "mesh_retriangulate", "mesh_import", "mesh_heat", "mesh_heat_debug", "mesh_check", "mesh_footprint", "mesh_bound", "server_create",
            "server_submit", "server_wait", "server_cancel", "server_release", "server_stats", "server_destroy",
            "sbmt_last_error", "sbmt_server_last_error")
 
@@ -156,6 +157,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
     lib.mesh_retriangulate.argtypes = [vp, ctypes.POINTER(sbmt_image), ctypes.c_uint64, ctypes.POINTER(ctypes.c_uint64)]
     lib.mesh_import.argtypes = [vp, vp, ctypes.c_int64, vp, ctypes.c_int64, ctypes.POINTER(ctypes.c_uint64)]
     lib.mesh_heat.argtypes = [vp, ctypes.c_uint64, ctypes.POINTER(sbmt_heat_params), vp, vp, vp]
+    lib.mesh_heat_debug.argtypes = [vp, ctypes.c_int, ctypes.c_int]
     lib.mesh_check.argtypes = [ctypes.POINTER(sbmt_image), ctypes.POINTER(sbmt_params)]
     lib.mesh_footprint.argtypes = [vp, ctypes.c_uint64, ctypes.POINTER(ctypes.c_size_t)]
     lib.mesh_bound.argtypes = [ctypes.POINTER(sbmt_image), ctypes.POINTER(sbmt_params), ctypes.POINTER(ctypes.c_size_t)]
@@ -176,7 +178,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
     for f in ("mesh_create", "mesh_bitmap", "mesh_batch", "mesh_autotune", "mesh_tuning", "mesh_set_tuning",
               "mesh_query", "mesh_release", "mesh_destroy",
               "mesh_stage", "mesh_profile", "mesh_profile_read", "mesh_quality", "mesh_project", "mesh_preprocess",
-              "mesh_preprocess_info", "mesh_heat"):
+              "mesh_preprocess_info", "mesh_heat", "mesh_heat_debug"):
         getattr(lib, f).restype = ctypes.c_int
     del i32
     _lib = lib
@@ -434,6 +436,11 @@ def mesh_heat(ctx: int, mesh: int, label: int, alpha: float, dt: float, steps: i
     its = (ctypes.c_int32 * max(steps, 1))()
     _check(load().mesh_heat(ctx, mesh, ctypes.byref(pr), ctypes.c_void_p(u.data_ptr()), peaks, its))
     return u, [peaks[k] for k in range(steps)], [its[k] for k in range(steps)]
+
+
+def mesh_heat_debug(ctx: int, what: int, value: int) -> None:
+    """A setting of this context's mesh_heat for tests (SBMT_HEAT_*)."""
+    _check(load().mesh_heat_debug(ctx, what, value))
 
 
 def mesh_profile(ctx: int, enable: bool) -> None:

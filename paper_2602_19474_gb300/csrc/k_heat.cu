@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(HB) k_heat_put(u32 n, const u32* list, const d
 // for block 0 gained nothing.
 // ---------------------------------------------------------------------------
 constexpr int CT = 512;         // threads per block
-constexpr int CG_BLOCKS = 152;  // at most one block per SM
+constexpr int CG_BLOCKS = 152;  // the most blocks: one per SM of this GPU
 constexpr int CG_SUMS = 3;      // the most sums a barrier carries
 constexpr int SLOT_WORDS = 4 * CG_SUMS * CG_BLOCKS + 16 * CG_BLOCKS;
 struct HeatCg {
@@ -605,7 +605,7 @@ size_t heat_scratch_bytes(u64 T, u64 V, int nsteps) {
 
 int heat_solve(const double* xy, const int* tri, const unsigned short* label, u64 T, u64 V, int L, double alpha,
                double dt, int nsteps, double x0, double y0, double sigma, double amp, double tol, int maxit,
-               double* u, double* peaks, int* iters, void* scratch, cudaStream_t st) {
+               double* u, double* peaks, int* iters, int max_blocks, void* scratch, cudaStream_t st) {
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   char* s = (char*)scratch;
   size_t off = 0;
@@ -707,15 +707,25 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     h.mass = mass, h.dg = dg, h.dinv = dinv, h.x = x, h.r = r, h.z = z, h.p = p, h.q = q;
     h.slot = slot, h.fail = (u32*)res, h.peak = peak, h.iters = its, h.done = (int*)res + 2;
     void* args[] = {&h};
-    const unsigned grid = (unsigned)std::min<u64>(CG_BLOCKS, (n + CT - 1) / CT);
-    h.block_rows = 32 * (((n + 31) / 32 + grid - 1) / grid);
-    const size_t vec_bytes = (size_t)CG_VECS * 8 * h.block_rows;
-    const bool onchip = vec_bytes <= CG_SMEM;
-    const void* cg = onchip ? (const void*)k_heat_cg<true> : (const void*)k_heat_cg<false>;
-    if (onchip && cudaFuncSetAttribute(cg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM) != cudaSuccess)
-      return -1;
-    if (cudaLaunchCooperativeKernel(cg, dim3(grid), dim3(CT), args, onchip ? vec_bytes : 0, st) != cudaSuccess)
-      return -1;
+    // One block per SM, as many as the process may use at once: a launch whose
+    // blocks cannot all be resident is refused, and is tried with half of them.
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) return -1;
+    unsigned grid = (unsigned)std::min<u64>(std::min(CG_BLOCKS, std::max(sms, 1)), (n + CT - 1) / CT);
+    if (max_blocks > 0) grid = std::min(grid, (unsigned)max_blocks);
+    while (true) {
+      h.block_rows = 32 * (((n + 31) / 32 + grid - 1) / grid);
+      const size_t vec_bytes = (size_t)CG_VECS * 8 * h.block_rows;
+      const bool onchip = vec_bytes <= CG_SMEM;
+      const void* cg = onchip ? (const void*)k_heat_cg<true> : (const void*)k_heat_cg<false>;
+      if (onchip && cudaFuncSetAttribute(cg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM) != cudaSuccess)
+        return -1;
+      const cudaError_t e = cudaLaunchCooperativeKernel(cg, dim3(grid), dim3(CT), args, onchip ? vec_bytes : 0, st);
+      if (e == cudaSuccess) break;
+      if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) return -1;
+      cudaGetLastError();
+      grid /= 2;
+    }
     ++launches;
     std::vector<char> hres(res_bytes);
     if (cudaMemcpyAsync(hres.data(), res, res_bytes, cudaMemcpyDeviceToHost, st) || cudaStreamSynchronize(st))

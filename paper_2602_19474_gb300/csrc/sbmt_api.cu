@@ -265,6 +265,7 @@ struct sbmt_ctx {
   Tune tune;
   std::map<std::string, Tune> tuned;
   bool tuned_loaded = false;
+  int heat_blocks = 0;  // mesh_heat_debug
 };
 
 namespace {
@@ -2037,12 +2038,19 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* hp, double*
   int n = 0;
   TRACE(KN_HEAT, n = heat_solve(m->xy, m->tri, m->label, (u64)m->nt, (u64)m->nv, hp->label, hp->alpha, hp->dt,
                                 hp->steps, hp->x0, hp->y0, hp->sigma, hp->amplitude, hp->tol, hp->max_iterations, u,
-                                peaks, iterations, scratch, st));
+                                peaks, iterations, ctx->heat_blocks, scratch, st));
   arena_end(lane);
   if (n == -2) return fail(SBMT_ETIMEDOUT, "a step did not reach the residual within %d iterations", hp->max_iterations);
   if (n == -3) return fail(SBMT_ETIMEDOUT, "a device wait ran out in the heat solver");
   if (n < 0) return fail(SBMT_ECUDA, "heat solve: %s", cudaGetErrorString(cudaGetLastError()));
   CK(cudaGetLastError());
+  return SBMT_OK;
+}
+
+int mesh_heat_debug(sbmt_ctx* ctx, int what, int value) {
+  if (!ctx || what != SBMT_HEAT_BLOCKS || value < 0) return fail(SBMT_EINVAL, "heat debug setting");
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  ctx->heat_blocks = value;
   return SBMT_OK;
 }
 

@@ -178,3 +178,24 @@ def test_peaks_leave_nans_out(amplitude, peak):
     sb.mesh_release(ctx(), m)
     assert peaks.tolist() == [peak, peak]
     assert its == [0, 0] and np.isnan(u).any()
+
+
+@pytest.mark.parametrize("blocks", [1, 2, 7, 151])
+def test_fewer_sms(blocks):
+    """The solver with as few blocks as a part with fewer SMs has, vectors on
+    chip and (one block of 88^2 rows) beyond: the oracle's solution."""
+    side = 88
+    j, i = np.mgrid[0:side, 0:side]
+    xy = np.stack([i.ravel(), j.ravel() * 0.9], 1).astype(float)
+    a = (j[:-1, :-1] * side + i[:-1, :-1]).ravel()
+    tri = np.concatenate([np.stack([a, a + 1, a + side + 1], 1), np.stack([a, a + side + 1, a + side], 1)]).astype(np.int32)
+    m = sb.mesh_import(ctx(), xy, tri)
+    sb.mesh_heat_debug(ctx(), sb.SBMT_HEAT_BLOCKS, blocks)
+    try:
+        u, peaks, its = run_gpu(m, 0xFFFF, 3.0, 0.1, 3, 40.0, 38.0, 9.0)
+    finally:
+        sb.mesh_heat_debug(ctx(), sb.SBMT_HEAT_BLOCKS, 0)
+        sb.mesh_release(ctx(), m)
+    uo, po = H.heat(xy, tri, np.full(len(tri), 0xFFFF), 0xFFFF, 3.0, 0.1, 3, 40.0, 38.0, 9.0)
+    assert np.abs(u - uo).max() <= 1e-8 * 100.0
+    assert np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
