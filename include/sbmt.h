@@ -42,7 +42,7 @@ extern "C" {
 #define SBMT_EINVAL (-1)    /* bad argument: dims, dtype, pitch, h, origin, mode */
 #define SBMT_ENOMEM (-2)    /* device allocation failed */
 #define SBMT_EPENDING (-3)  /* mesh_query poll: work not finished yet */
-#define SBMT_ETIMEDOUT (-4) /* mesh_query: wait limit reached */
+#define SBMT_ETIMEDOUT (-4) /* a wait limit reached (mesh_query's, or a bounded device wait), or no convergence */
 #define SBMT_ECAPACITY (-5) /* a cell holds more boundary vertices than the per-cell limit (mesh_stage 4 lists them) */
 #define SBMT_EPROTO (-6)    /* requested mode is not available (SBMT_PREPROCESS in mesh_bitmap) */
 #define SBMT_ECUDA (-7)     /* a CUDA call failed (message in sbmt_last_error) */
@@ -429,8 +429,11 @@ int mesh_project(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_image* field, float* 
  *              step;
  *  iterations  host, `steps` int32, or NULL: the CG iterations of each step.
  * Explicit meshes only (SBMT_EINVAL otherwise, or for bad parameters).
- * SBMT_ETIMEDOUT if a step does not converge within max_iterations.  Runs on
- * the context's stream after the mesh and returns when done. */
+ * SBMT_ETIMEDOUT if a step does not converge within max_iterations (u, peaks
+ * and iterations then hold that step's state), or if a bounded device wait ran
+ * out (see SBMT_HEAT_STALL; u, peaks and iterations are then unwritten;
+ * sbmt_last_error tells the two apart).  Runs on the context's stream after the
+ * mesh and returns when done. */
 typedef struct {
   int32_t label;
   double alpha, dt;
@@ -444,8 +447,13 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* params, dou
 
 /* Settings of this context's mesh_heat for tests (0: none).
  * SBMT_HEAT_BLOCKS: the solver's launch takes at most `value` blocks, as
- * where fewer SMs are to be had (it takes one block per SM otherwise). */
-enum { SBMT_HEAT_BLOCKS = 0 };
+ * where fewer SMs are to be had (it takes one block per SM otherwise).
+ * SBMT_HEAT_STALL is a test of the bound on device waits: at the launch's
+ * barrier number `value` (1, 2, ...) its last block withholds its sums, so that
+ * the waits for them run out (two seconds) and the call returns SBMT_ETIMEDOUT,
+ * leaving the context usable (for a region of two blocks, 513 free vertices, or
+ * more). */
+enum { SBMT_HEAT_BLOCKS = 0, SBMT_HEAT_STALL = 1 };
 int mesh_heat_debug(sbmt_ctx* ctx, int what, int value);
 
 /* Per-kernel device time, for tracing and roofline accounting (no

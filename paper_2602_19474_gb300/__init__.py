@@ -36,7 +36,7 @@ SBMT_PLAIN, SBMT_PREPROCESS = 0, 1
 SBMT_EXPLICIT, SBMT_COMPACT = 0, 1
 SBMT_KEEP_STAGES = 1
 SBMT_DEBUG_STALL_SCAN = 2
-SBMT_HEAT_BLOCKS = 0
+SBMT_HEAT_BLOCKS, SBMT_HEAT_STALL = 0, 1
 
 EXPORTS = ("mesh_create", "mesh_bitmap", "mesh_batch", "mesh_autotune", "mesh_tuning", "mesh_set_tuning",
            "mesh_query", "mesh_release", "mesh_destroy", "mesh_stage", "mesh_profile", "mesh_profile_read", "mesh_quality", "mesh_project",

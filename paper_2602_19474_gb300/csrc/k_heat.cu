@@ -287,6 +287,7 @@ struct HeatCg {
   u32 n, nsteps;
   u32 block_rows;  // the most rows a block has, in whole slices
   int maxit, sliced;
+  u32 stall;  // test of the wait's bound: the last block publishes nothing at this barrier (1, 2, ...)
   double tol;
   const u32* rowptr;
   const u32* mcnt;
@@ -394,9 +395,11 @@ SBMT_DEV bool grid_sums(const HeatCg& h, const double (&v)[K], u32& gen, double 
       for (int k = 0; k < CG_SUMS; ++k)
         st_relaxed(in2 + k * CG_BLOCKS + blockIdx.x, CG_EMPTY), st_relaxed(out2 + 4 * blockIdx.x + k, CG_EMPTY);
       fence_gpu();
+      if (gen + 1 != h.stall || blockIdx.x != gridDim.x - 1) {
 #pragma unroll
-      for (int k = 0; k < K; ++k)
-        st_relaxed(in + k * CG_BLOCKS + blockIdx.x, (unsigned long long)__double_as_longlong(t[k]));
+        for (int k = 0; k < K; ++k)
+          st_relaxed(in + k * CG_BLOCKS + blockIdx.x, (unsigned long long)__double_as_longlong(t[k]));
+      }
     }
     mid();
     if (blockIdx.x == 0) {
@@ -605,7 +608,7 @@ size_t heat_scratch_bytes(u64 T, u64 V, int nsteps) {
 
 int heat_solve(const double* xy, const int* tri, const unsigned short* label, u64 T, u64 V, int L, double alpha,
                double dt, int nsteps, double x0, double y0, double sigma, double amp, double tol, int maxit,
-               double* u, double* peaks, int* iters, int max_blocks, void* scratch, cudaStream_t st) {
+               double* u, double* peaks, int* iters, int max_blocks, int stall, void* scratch, cudaStream_t st) {
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   char* s = (char*)scratch;
   size_t off = 0;
@@ -703,6 +706,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     int* its = (int*)(peak + nsteps);
     HeatCg h{};
     h.n = n, h.nsteps = (u32)nsteps, h.maxit = maxit, h.sliced = sliced ? 1 : 0, h.tol = tol;
+    h.stall = (u32)stall;
     h.rowptr = rowptr, h.mcnt = mcnt, h.col = col, h.val = val, h.scol = scol, h.sval = sval;
     h.mass = mass, h.dg = dg, h.dinv = dinv, h.x = x, h.r = r, h.z = z, h.p = p, h.q = q;
     h.slot = slot, h.fail = (u32*)res, h.peak = peak, h.iters = its, h.done = (int*)res + 2;

@@ -265,7 +265,7 @@ struct sbmt_ctx {
   Tune tune;
   std::map<std::string, Tune> tuned;
   bool tuned_loaded = false;
-  int heat_blocks = 0;  // mesh_heat_debug
+  int heat_debug[2] = {0, 0};  // mesh_heat_debug
 };
 
 namespace {
@@ -2038,7 +2038,8 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* hp, double*
   int n = 0;
   TRACE(KN_HEAT, n = heat_solve(m->xy, m->tri, m->label, (u64)m->nt, (u64)m->nv, hp->label, hp->alpha, hp->dt,
                                 hp->steps, hp->x0, hp->y0, hp->sigma, hp->amplitude, hp->tol, hp->max_iterations, u,
-                                peaks, iterations, ctx->heat_blocks, scratch, st));
+                                peaks, iterations, ctx->heat_debug[SBMT_HEAT_BLOCKS],
+                                ctx->heat_debug[SBMT_HEAT_STALL], scratch, st));
   arena_end(lane);
   if (n == -2) return fail(SBMT_ETIMEDOUT, "a step did not reach the residual within %d iterations", hp->max_iterations);
   if (n == -3) return fail(SBMT_ETIMEDOUT, "a device wait ran out in the heat solver");
@@ -2048,9 +2049,9 @@ int mesh_heat(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_heat_params* hp, double*
 }
 
 int mesh_heat_debug(sbmt_ctx* ctx, int what, int value) {
-  if (!ctx || what != SBMT_HEAT_BLOCKS || value < 0) return fail(SBMT_EINVAL, "heat debug setting");
+  if (!ctx || what < 0 || what > SBMT_HEAT_STALL || value < 0) return fail(SBMT_EINVAL, "heat debug setting");
   std::lock_guard<std::mutex> lk(ctx->mu);
-  ctx->heat_blocks = value;
+  ctx->heat_debug[what] = value;
   return SBMT_OK;
 }
 

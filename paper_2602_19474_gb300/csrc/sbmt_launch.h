@@ -330,13 +330,15 @@ int launch_r3_emit(const R3Args& a, cudaStream_t st);
 // residual tol, at most maxit iterations per step): u (device, V doubles)
 // receives the solution; peaks / iters (host, nsteps each, or null) the
 // maximum of u and the iterations after each step.  max_blocks > 0: no more
-// blocks than that in the solver's launch.  scratch holds
+// blocks than that in the solver's launch; stall > 0: its last block withholds
+// its sums at that barrier.  scratch holds
 // heat_scratch_bytes(T, V, nsteps) bytes (256-byte aligned).  Synchronises
 // with the device twice; returns the kernels launched, -1 if a CUDA call
-// failed, -2 if a step did not converge, -3 if a wait across the grid ran out.
+// failed, -2 if a step did not converge, -3 if a wait across the grid ran out
+// (u, peaks and iters are then unwritten).
 size_t heat_scratch_bytes(u64 T, u64 V, int nsteps);
 int heat_solve(const double* xy, const int* tri, const unsigned short* label, u64 T, u64 V, int L, double alpha,
                double dt, int nsteps, double x0, double y0, double sigma, double amp, double tol, int maxit,
-               double* u, double* peaks, int* iters, int max_blocks, void* scratch, cudaStream_t st);
+               double* u, double* peaks, int* iters, int max_blocks, int stall, void* scratch, cudaStream_t st);
 
 }  // namespace sbmt

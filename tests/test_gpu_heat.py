@@ -199,3 +199,29 @@ def test_fewer_sms(blocks):
     uo, po = H.heat(xy, tri, np.full(len(tri), 0xFFFF), 0xFFFF, 3.0, 0.1, 3, 40.0, 38.0, 9.0)
     assert np.abs(u - uo).max() <= 1e-8 * 100.0
     assert np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
+
+
+@pytest.mark.parametrize("barrier", [1, 2, 5])
+def test_a_wait_that_runs_out(barrier):
+    """One block withholds its sums at a barrier: the call ends with the bounded
+    wait's error, u, peaks and iterations unwritten, and the next call on the
+    context is right."""
+    import torch
+
+    m = sb.mesh_bitmap(ctx(), np.pad(np.ones((70, 80), np.uint8), 4), 2, 1)
+    v = sb.mesh_query(ctx(), m, -1)
+    args = (1, 50.0, 0.05, 2, 40.0, 38.0, 12.0)
+    u = torch.full((v.n_vertices,), 7.0, dtype=torch.float64, device="cuda")
+    sb.mesh_heat_debug(ctx(), sb.SBMT_HEAT_STALL, barrier)
+    try:
+        with pytest.raises(sb.SbmtError) as e:
+            sb.mesh_heat(ctx(), m, *args, 100.0, 1e-12, u=u)
+    finally:
+        sb.mesh_heat_debug(ctx(), sb.SBMT_HEAT_STALL, 0)
+    assert e.value.code == sb.SBMT_ETIMEDOUT and "device wait" in str(e.value)
+    assert bool((u == 7.0).all())
+    got, peaks, its = run_gpu(m, *args)
+    g = sb.view_numpy(v)
+    sb.mesh_release(ctx(), m)
+    uo, po = H.heat(g["xy"], g["tri"], g["label"], *args)
+    assert np.abs(got - uo).max() <= 1e-8 * 100.0 and np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
