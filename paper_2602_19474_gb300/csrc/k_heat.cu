@@ -298,7 +298,7 @@ struct HeatCg {
   const double* mass;
   const double* dg;
   const double* dinv;
-  double *x, *r, *z, *p, *q;
+  double *x, *r, *z, *p, *q, *b;
   unsigned long long* slot;  // SLOT_WORDS published sums, all bits set at first
   u32* fail;                 // a wait ran out
   unsigned long long* peak;  // per step: the maximum of x (double bits), 0 at least
@@ -489,6 +489,17 @@ constexpr size_t CG_SMEM = 227 * 1024 - 13 * 1024;  // what a block has for them
 // Two barriers an iteration: the product is taken of z, which is final
 // before beta is known, and q = A z + beta q, p = z + beta p follow from it, so that
 // the new p needs no barrier of its own before the next product.
+//
+// These recurrences drift from the true residual b - A x sooner than a product
+// taken of p itself: over regions of 5e3 to 5e4 vertices of a label image the
+// residual a step can reach was the same at alpha dt = 5 (a step of some 50
+// iterations), and at 5e4 and 5e6 (300 to 800 iterations) 1.3 to 1.6 times as
+// large.  So a long step takes r = b - A x anew after ANEW iterations, 4 ANEW,
+// and so on: what drifted until then is gone, and the reachable residual is
+// 0.3 to 0.6 times the product form's at alpha dt = 500 and below 0.1 times at 5e4
+// and above.  It costs a product and two barriers each time, none in a step of
+// fewer iterations.
+constexpr int ANEW = 96;  // a multiple of 8: where the residual is looked at
 template <bool ONCHIP>
 __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatCg h) {
   extern __shared__ double s_vec[];
@@ -517,14 +528,14 @@ __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatC
       const double xi = x[l], bi = h.mass[i] * xi, dd = h.dg[i] * xi;
       const double qi = row_times(h, i, h.x, dd);
       const double di = dinv_at(l), rv = di != 0.0 ? bi - qi : 0.0, zv = rv * di;
-      r[l] = rv, z[l] = zv, p[l] = 0.0, q[l] = 0.0;
+      r[l] = rv, z[l] = zv, p[l] = 0.0, q[l] = 0.0, h.b[i] = bi;
       if (ONCHIP) h.z[i] = zv;
       a3[0] += rv * zv, a3[1] += rv * rv, a3[2] += bi * bi;
     }
     if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
     double rz = s_sum[0], rr = s_sum[1], be = 0.0;
     const double stop = h.tol * h.tol * s_sum[2];
-    int it = 0;
+    int it = 0, anew = ANEW;
     while (rr > stop && it < h.maxit) {
       bool look = false;
       while (!look) {
@@ -575,6 +586,27 @@ __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatC
         rz = s_sum[0], be = s_k;
         if (look) rr = s_sum[1];
       }
+      if (it == anew && rr > stop) {
+        // r = b - A x again, in the place of the recurrence's (x of all blocks
+        // is there after the barrier); the direction goes on
+        anew *= 4;
+        if (ONCHIP)
+          for (u32 l = tid; l < rows; l += CT) h.x[row0 + l] = x[l];
+        const double none[1] = {0.0};
+        if (!grid_sums<1, false>(h, none, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
+        double a2[2] = {0.0, 0.0};
+        for (u32 l = tid; l < rows; l += CT) {
+          const u32 i = row0 + l;
+          const double di = dinv_at(l), rv = di != 0.0 ? h.b[i] - row_times(h, i, h.x, h.dg[i] * x[l]) : 0.0, zv = rv * di;
+          r[l] = rv, z[l] = zv;
+          if (ONCHIP) h.z[i] = zv;
+          a2[0] += rv * zv, a2[1] += rv * rv;
+        }
+        if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail, [] {},
+                                [&](const double* t) { s_k = rz != 0.0 ? be * (t[0] / rz) : 0.0; }))
+          return;
+        rz = s_sum[0], rr = s_sum[1], be = s_k;
+      }
     }
     // the step's peak (positive doubles order as their bits, infinity above all;
     // NaNs are left out, as fmax leaves them), and x for the next step's product
@@ -601,7 +633,7 @@ unsigned grid_v(u64 n) { return (unsigned)std::max<u64>(1, std::min<u64>((n + HB
 }  // namespace
 
 size_t heat_scratch_bytes(u64 T, u64 V, int nsteps) {
-  return 256 * 32 + T * (sizeof(HeatTri) + 6 * (4 + 8) + 4 + 4 + 12) + V * (4 + 4 + 4 + 4 + 4 + 4 + 4 + 8 * 9) +
+  return 256 * 32 + T * (sizeof(HeatTri) + 6 * (4 + 8) + 4 + 4 + 12) + V * (4 + 4 + 4 + 4 + 4 + 4 + 4 + 8 * 10) +
          8 * SLOT_WORDS + 12 * (size_t)std::max(nsteps, 1) + 64 +
          4 * scan_scratch_words((u32)std::min<u64>(std::max(T, V), 0xFFFFFFFFu));
 }
@@ -639,6 +671,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
   double* r = (double*)take(8 * V);
   double* z = (double*)take(8 * V);
   double* p = (double*)take(8 * V);
+  double* b = (double*)take(8 * V);
   unsigned long long* slot = (unsigned long long*)take(8 * SLOT_WORDS);
   // the solver's results: a failed wait, 0, steps done, convergence, then per
   // step the peak and the iterations
@@ -708,7 +741,7 @@ int heat_solve(const double* xy, const int* tri, const unsigned short* label, u6
     h.n = n, h.nsteps = (u32)nsteps, h.maxit = maxit, h.sliced = sliced ? 1 : 0, h.tol = tol;
     h.stall = (u32)stall;
     h.rowptr = rowptr, h.mcnt = mcnt, h.col = col, h.val = val, h.scol = scol, h.sval = sval;
-    h.mass = mass, h.dg = dg, h.dinv = dinv, h.x = x, h.r = r, h.z = z, h.p = p, h.q = q;
+    h.mass = mass, h.dg = dg, h.dinv = dinv, h.x = x, h.r = r, h.z = z, h.p = p, h.q = q, h.b = b;
     h.slot = slot, h.fail = (u32*)res, h.peak = peak, h.iters = its, h.done = (int*)res + 2;
     void* args[] = {&h};
     // One block per SM, as many as the process may use at once: a launch whose

@@ -225,3 +225,44 @@ def test_a_wait_that_runs_out(barrier):
     sb.mesh_release(ctx(), m)
     uo, po = H.heat(g["xy"], g["tri"], g["label"], *args)
     assert np.abs(got - uo).max() <= 1e-8 * 100.0 and np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)
+
+
+@pytest.mark.parametrize("alpha_dt", [500.0, 5.0e4, 5.0e6])
+def test_reachable_residual_at_long_steps(alpha_dt):
+    """Steps far longer than a cell's diffusion time (hundreds of iterations):
+    the true residual that a step ends at, with a tolerance below what can be
+    reached, is no larger than that of conjugate gradients whose every q is the
+    product A p, as the geometric mean over 16 pulses (one pulse's ratio moves by
+    a few tenths with the rounding)."""
+    import scipy.sparse as sp
+
+    img = synth.voronoi_labels(size=200, nseeds=5)
+    L = int(np.bincount(img.ravel()).argmax())
+    m = sb.mesh_bitmap(ctx(), img, 2, 1)
+    g = sb.view_numpy(sb.mesh_query(ctx(), m, -1))
+    sel, free, _ = H.region(g["tri"], g["label"], L)
+    idx, t = np.nonzero(free)[0], g["tri"][sel]
+    M = H.lumped_mass(g["xy"], t, len(g["xy"]))[idx]
+    A = (H.stiffness(g["xy"], t, len(g["xy"])) * alpha_dt)[idx][:, idx].tocsr() + sp.diags(M).tocsr()
+    P = g["xy"][idx]
+    rng = np.random.default_rng(11)
+    log = []
+    for _ in range(16):
+        c = P.mean(0) + np.ptp(P, axis=0) * rng.uniform(-0.25, 0.25, 2)
+        sigma = rng.uniform(5.0, 20.0)
+        u, _, _ = run_gpu(m, L, alpha_dt, 1.0, 1, c[0], c[1], sigma, tol=1e-13)
+        x = H.pulse(P, c[0], c[1], sigma, 100.0)
+        b, dinv = M * x, 1.0 / A.diagonal()
+        end = np.linalg.norm(b - A @ u[idx])
+        r = b - A @ x
+        z = r * dinv
+        p, rz, it = z.copy(), r @ z, 0
+        while it % 8 or np.linalg.norm(r) > 1e-13 * np.linalg.norm(b):
+            q = A @ p
+            al = rz / (p @ q)
+            x, r = x + al * p, r - al * q
+            z = r * dinv
+            p, rz, it = z + (r @ z) / rz * p, r @ z, it + 1
+        log.append(np.log(end / np.linalg.norm(b - A @ x)))
+    sb.mesh_release(ctx(), m)
+    assert np.mean(log) <= 0.0, np.exp(np.mean(log))
