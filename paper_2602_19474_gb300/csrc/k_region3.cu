@@ -747,9 +747,8 @@ SBMT_DEV int r3_neighbour(const R3Args& a, u32 c, const R3Cell& C, int j) {
   const int u = C.id[j], w = C.id[j == 2 ? 0 : j + 1];
   int found = -1;
   for (u32 e = a.head[u]; e != NONE;) {
-    const uint2 x = a.link[e];
-    const u32 c2 = x.x;
-    e = x.y;
+    const u32 c2 = a.cand[e / 3u];
+    e = a.link[e];
     if (c2 == c) continue;
     const int* t = a.ttri + 3 * (u64)c2;
     if (t[0] == w || t[1] == w || t[2] == w) {
@@ -776,8 +775,9 @@ SBMT_DEV int r3_edge_in(const R3Args& a, u32 c2, int u, int w) {
 // candidates, and only those need listing -- a linked list per vertex, pushed
 // by exchanging its head (the counts, scan and lists over every cell took 0.19
 // ms for 9.8e6 cells, 0.02 ms for the few percent that are
-// candidates).  The order of a list
-// depends on the run; what is looked up in it does not.
+// candidates).  Entry 3 q + k is candidate q's at its corner k, so that an entry is
+// its successor alone.  The order of a list depends on the run; what is looked up
+// in it does not.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_r3_link(R3Args a) {
   const u32 n = *a.ncand;
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(256) k_r3_link(R3Args a) {
         continue;
       }
       const u32 e = 3 * q + (u32)k;
-      a.link[e] = make_uint2(c, atomicExch(a.head + v, e));
+      a.link[e] = atomicExch(a.head + v, e);
     }
   }
 }

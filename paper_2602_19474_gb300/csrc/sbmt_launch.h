@@ -302,7 +302,7 @@ struct R3Args {
   u32 nv;
   u64 nt;
   u32* head;    // per vertex: its list of candidate cells (all bits set: none)
-  uint2* link;  // list entries (cell, next), 3 per candidate
+  u32* link;    // list entries, 3 per candidate (3 q + corner for candidate q): the next one
   // per cut cell (unset elsewhere): triangles, owned events (and per edge),
   // inside vertices; per word of 32 cells: the cut cells, and the sums of their
   // triangles beyond one, owned events and inside vertices with their scans

@@ -395,3 +395,37 @@ def test_cells_reaching_far_outside_the_image(far, mirror, fill):
     want = oracle.region3(img, xy, tri)
     assert want["n_inside"] >= 4
     assert_same(_imported(img, xy, tri), want)
+
+
+def _pool_bytes():
+    """The bytes in use of the device's stream-ordered allocations."""
+    import ctypes
+
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, used = ctypes.c_void_p(), ctypes.c_uint64()
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert cu.cuMemPoolGetAttribute(pool, 7, ctypes.byref(used)) == 0  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+    return used.value
+
+
+def test_scratch_bytes_of_a_retriangulation():
+    """The working memory of mesh_retriangulate stays at 58 bytes a cell (for
+    two cells a vertex), beside the 16 MB that the context adds to what it keeps."""
+    n = 1500
+    j, i = np.mgrid[0:n, 0:n]
+    xy = np.stack([i.ravel(), j.ravel()], 1) * 0.5 + [0.1, 0.2]
+    a = (j[:-1, :-1] * n + i[:-1, :-1]).ravel().astype(np.int32)
+    tri = np.concatenate([np.stack([a, a + 1, a + n + 1], 1), np.stack([a, a + n + 1, a + n], 1)])
+    img = np.zeros((32, 32), np.uint8)
+    ctx()
+    c = sb.mesh_create(0)
+    try:
+        b = sb.mesh_import(c, xy, tri)
+        sb.mesh_query(c, b, -1)
+        before = _pool_bytes()  # the import keeps no scratch
+        m = sb.mesh_retriangulate(c, img, b)
+        sb.mesh_query(c, m, -1)
+        scratch = _pool_bytes() - before - sb.mesh_footprint(c, m)
+    finally:
+        sb.mesh_destroy(c)
+    assert len(tri) * 40 < scratch - (16 << 20) <= len(tri) * 58 + (1 << 20), (scratch - (16 << 20)) / len(tri)
