@@ -391,9 +391,8 @@ __global__ void __launch_bounds__(128) k_pre_region1(PreArgs a) {
   for (u32 e0 = blockIdx.x * blockDim.x; e0 < nq; e0 += gridDim.x * blockDim.x) {
     const u32 e = e0 + threadIdx.x;
     bool reach = false;
-    uint2 qe = make_uint2(0u, 0u);
     if (e < nq) {
-      qe = a.vq[e];
+      const uint2 qe = a.vq[e];
       const int r = (int)qe.y;
       const i64 v = qe.x, j = g.vj0 + r, i = g.vlo[r] + (v - g.vbase[r]), mi = 2 * i + j - a.m0;
       const double x = a.tab[mi], y = a.ytab[r];
@@ -419,7 +418,7 @@ __global__ void __launch_bounds__(128) k_pre_region1(PreArgs a) {
       u32 q0 = 0;
       if (lane == 0) q0 = atomicAdd(a.cnt + 6, (u32)__popc(m));
       q0 = __shfl_sync(0xFFFFFFFFu, q0, 0);
-      if (reach) a.rq[q0 + __popc(m & ((1u << lane) - 1u))] = qe;
+      if (reach) a.rq[q0 + __popc(m & ((1u << lane) - 1u))] = e;
     }
   }
   nsnap = __reduce_add_sync(0xFFFFFFFFu, nsnap);
@@ -435,7 +434,7 @@ __global__ void __launch_bounds__(128) k_pre_repel(PreArgs a) {
   double2* xy = reinterpret_cast<double2*>(a.xy);
   u32 nrep = 0;
   for (u32 e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const uint2 qe = a.rq[e];
+    const uint2 qe = a.vq[a.rq[e]];
     const int r = (int)qe.y;
     const i64 v = qe.x, mi = 2 * (g.vlo[r] + (v - g.vbase[r])) + (g.vj0 + r) - a.m0;
     double2 out;

@@ -268,7 +268,7 @@ struct PreArgs {
   double* ytab;  // y of every vertex row, and its float copy
   float* ytabf;
   uint2* vq;     // Region I queue: (vertex id, vertex row), nverts entries, cnt[7] of them
-  uint2* rq;     // Step 2 queue: (vertex id, vertex row), nverts entries
+  u32* rq;       // Step 2 queue: places in vq, nverts entries
   int* prow;
   float2* xyf;
   u32* plist;

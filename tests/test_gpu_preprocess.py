@@ -212,3 +212,26 @@ def test_full_size_windows():
     del t
     sb.mesh_release(c, m)
     torch.cuda.empty_cache()
+
+
+def test_scratch_bytes():
+    """The working memory of mesh_preprocess on an image without boundary points:
+    per lattice vertex 8 bytes of float coordinates, 12 of queues and 1/2 of split-cell
+    bits and their scan, per pixel 3/8 of two bit-planes and a scan, beside the 16 MB
+    that the context adds to what it keeps."""
+    from test_gpu_region3 import _pool_bytes
+
+    n = 6000
+    img = np.ones((n, n), np.uint8)
+    ctx()
+    c = sb.mesh_create(0)
+    try:
+        before = _pool_bytes()
+        m = sb.mesh_preprocess(c, img, 2, 1)
+        v = sb.mesh_query(c, m, -1)
+        scratch = _pool_bytes() - before - sb.mesh_footprint(c, m) - n * n  # the host image's device copy
+        verts = v.n_lattice_vertices
+    finally:
+        sb.mesh_destroy(c)
+    per = (scratch - (16 << 20) - n * n * 0.375) / verts
+    assert 10.0 < per <= 21.0, per
