@@ -329,7 +329,8 @@ int mesh_footprint(sbmt_ctx* ctx, sbmt_mesh mesh, size_t* bytes);
 
 /* Wait up to wait_ms milliseconds (0 = poll, < 0 = no limit) for a mesh and
  * fill *out.  Returns SBMT_EPENDING / SBMT_ETIMEDOUT while unfinished, or
- * the mesh's status. */
+ * the mesh's status.  A wait without limit polls without a pause for its first
+ * 5 ms, later (and with a limit from the start) every 20 us. */
 int mesh_query(sbmt_ctx* ctx, sbmt_mesh mesh, int wait_ms, sbmt_mesh_view* out);
 
 /* Free the device memory of one mesh (waits for its work first). */

@@ -1775,20 +1775,22 @@ int mesh_query(sbmt_ctx* ctx, sbmt_mesh mesh, int wait_ms, sbmt_mesh_view* out) 
     if (it == ctx->meshes.end()) return fail(SBMT_ENOENT, "unknown mesh %llu", (unsigned long long)mesh);
     m = it->second;
   }
-  if (wait_ms < 0) {
-    // no limit: the driver's own wait, which returns within microseconds of
-    // the event (a sleep between polls overslept by some 50)
-    const cudaError_t q = cudaEventSynchronize(m->done);
-    if (q != cudaSuccess) return fail(SBMT_ECUDA, "mesh work failed: %s", cudaGetErrorString(q));
-  }
+  // A wait without a limit polls without a pause for its first 5 ms (a sleep of
+  // 20 us between polls overslept by some 50, a tenth of a small mesh's call), and
+  // then sleeps between polls like one with a limit, so that a thread in a long
+  // wait leaves its core to others.
   const auto t0 = std::chrono::steady_clock::now();
-  while (wait_ms >= 0) {
+  while (true) {
     const cudaError_t q = cudaEventQuery(m->done);
     if (q == cudaSuccess) break;
     if (q != cudaErrorNotReady) return fail(SBMT_ECUDA, "mesh work failed: %s", cudaGetErrorString(q));
     if (wait_ms == 0) return SBMT_EPENDING;
     const auto waited = std::chrono::steady_clock::now() - t0;
-    if (waited > std::chrono::milliseconds(wait_ms)) return SBMT_ETIMEDOUT;
+    if (wait_ms > 0 && waited > std::chrono::milliseconds(wait_ms)) return SBMT_ETIMEDOUT;
+    if (wait_ms < 0 && waited < std::chrono::milliseconds(5)) {
+      std::this_thread::yield();
+      continue;
+    }
     std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
   int rc = settle(m);

@@ -165,3 +165,32 @@ def test_emission_by_one_to_eight_warps_a_bucket(count):
         got = _fetch(c, m)
         for key in ("tri", "label", "code", "xy"):
             assert np.array_equal(got[key], single[key]), key
+
+
+def test_a_long_wait_leaves_its_core():
+    """mesh_query without a limit on work some 0.4 s away: the waiting thread's
+    own CPU time stays a fraction of the wait."""
+    import time
+
+    import torch
+
+    st = torch.cuda.Stream()
+    c = sb.mesh_create(0, 0, st.cuda_stream)
+    try:
+        img = synth.disk()
+        m = sb.mesh_bitmap(c, img, 2)
+        v = sb.mesh_query(c, m, -1)
+        out = torch.empty(v.n_triangles, dtype=torch.float32, device="cuda")
+        field = torch.ones(img.shape, dtype=torch.float32, device="cuda")
+        with torch.cuda.stream(st):
+            sb.mesh_project(c, m, field, out)  # (a first launch loads the kernels and waits)
+            torch.cuda._sleep(1000)
+            torch.cuda.synchronize()
+            torch.cuda._sleep(800_000_000)
+        sb.mesh_project(c, m, field, out)  # mesh_query waits for it too
+        w0, c0 = time.monotonic(), time.thread_time()
+        sb.mesh_query(c, m, -1)
+        wall, cpu = time.monotonic() - w0, time.thread_time() - c0
+    finally:
+        sb.mesh_destroy(c)
+    assert wall > 0.2 and cpu < 0.4 * wall, (wall, cpu)
