@@ -266,3 +266,20 @@ def test_reachable_residual_at_long_steps(alpha_dt):
         log.append(np.log(end / np.linalg.norm(b - A @ x)))
     sb.mesh_release(ctx(), m)
     assert np.mean(log) <= 0.0, np.exp(np.mean(log))
+
+
+@pytest.mark.parametrize("n", [511, 512, 513, 1024, 1025])
+def test_regions_at_the_edges_of_a_block(n):
+    """Regions of n free vertices, one block's threads, one more and so on (a fan of
+    neighbours around a centre, every vertex free): the oracle's solution."""
+    k = np.arange(n - 1)
+    ang = 2 * np.pi * k / (n - 1)
+    rad = 20.0 + (k % 2)
+    xy = np.concatenate([[[0.0, 0.0]], np.stack([rad * np.cos(ang), rad * np.sin(ang)], 1)])
+    tri = np.stack([np.zeros(n - 1, int), 1 + k, 1 + (k + 1) % (n - 1)], 1).astype(np.int32)
+    m = sb.mesh_import(ctx(), xy, tri)
+    u, peaks, its = run_gpu(m, 0xFFFF, 3.0, 0.1, 3, 2.0, 1.0, 9.0)
+    sb.mesh_release(ctx(), m)
+    uo, po = H.heat(xy, tri, np.full(len(tri), 0xFFFF), 0xFFFF, 3.0, 0.1, 3, 2.0, 1.0, 9.0)
+    assert np.abs(u - uo).max() <= 1e-8 * 100.0
+    assert np.allclose(peaks, po, rtol=0, atol=1e-8 * 100.0)

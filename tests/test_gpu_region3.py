@@ -429,3 +429,36 @@ def test_scratch_bytes_of_a_retriangulation():
     finally:
         sb.mesh_destroy(c)
     assert len(tri) * 40 < scratch - (16 << 20) <= len(tri) * 58 + (1 << 20), (scratch - (16 << 20)) / len(tri)
+
+
+@pytest.mark.parametrize("fill", [0, 6000])
+def test_node_counts_at_the_edges_of_the_groups(fill):
+    """Single cells over a striped image (single pixels flipped), up to four of every
+    node count within the per-cell limits: 8 and 9, 16 and 17, 32 and 33 nodes, where
+    the group of lanes changes, and 48, the limit.  Without and with room for the
+    cells' records (their entries and heads, 64-bit words, against one word a cell;
+    uncut cells apart from the image make the room)."""
+    rng = np.random.default_rng(1)
+    img = (np.arange(64)[None, :] % 2 + 2 * (np.arange(64)[:, None] // 16 % 2)).astype(np.uint8)
+    img[rng.random((64, 64)) < 0.01] ^= 1
+    kept = {}
+    for _ in range(3000):
+        t = rng.uniform(0, 2 * np.pi) + 2 * np.pi * np.arange(3) / 3 + rng.uniform(-0.4, 0.4, 3)
+        xy = rng.uniform(12, 52, 2) + rng.uniform(1.5, 13) * np.stack([np.cos(t), np.sin(t)], 1) * rng.uniform(0.6, 1.2, (3, 1))
+        o = oracle.region3(img, xy, np.array([[0, 1, 2]], np.int32))
+        ne, ni = o["n_events"], o["n_inside"]
+        if ne + ni == 0 or 3 + ne + ni > 48 or ni > 16 or len(kept.get(3 + ne + ni, [])) == 4:
+            continue
+        ev, e = o["xy"][3:3 + ne], np.roll(xy, -1, 0) - xy
+        off = np.abs(e[:, None, 0] * (ev[None, :, 1] - xy[:, None, 1]) - e[:, None, 1] * (ev[None, :, 0] - xy[:, None, 0]))
+        if np.bincount(off.argmin(0), minlength=3).max() <= 16:
+            kept.setdefault(3 + ne + ni, []).append(xy)
+    assert {8, 9, 16, 17, 32, 33, 48} <= set(kept)
+    xy = np.concatenate([x for n in sorted(kept) for x in kept[n]])
+    words = sum(n * len(kept[n]) for n in kept if n <= 32)
+    k = np.arange(fill)
+    far = np.stack([200.0 + k, np.full(fill, 100.0)], 1)[:, None] + [[0.0, 0.0], [0.5, 0.0], [0.0, 0.5]]
+    xy = np.concatenate([xy, far.reshape(-1, 2)])
+    tri = np.arange(len(xy), dtype=np.int32).reshape(-1, 3)
+    assert (words <= len(tri)) == (fill > 0)
+    assert_same(_imported(img, xy, tri), oracle.region3(img, xy, tri))
