@@ -12,14 +12,14 @@ namespace {
 
 constexpr int TILE = 2048;  // elements per tile (256 threads x 8)
 
-// one block of 1024 threads: exclusive scan of n strided values, total at out[n]
-__global__ void __launch_bounds__(1024) k_scan_small(const u32* in, int stride, u32* out, u32 n) {
+// one block of 1024 threads: exclusive scan of n values, total at out[n]
+__global__ void __launch_bounds__(1024) k_scan_small(const u32* in, u32* out, u32 n) {
   __shared__ u32 sh[1024];
   const u32 t = threadIdx.x;
   const u32 chunk = (n + 1023) / 1024;
   const u32 a = min(n, t * chunk), e = min(n, a + chunk);
   u32 s = 0;
-  for (u32 i = a; i < e; ++i) s += in[(u64)i * stride];
+  for (u32 i = a; i < e; ++i) s += in[i];
   sh[t] = s;
   __syncthreads();
   for (u32 o = 1; o < 1024; o <<= 1) {
@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(1024) k_scan_small(const u32* in, int stride, 
   }
   u32 run = sh[t] - s;
   for (u32 i = a; i < e; ++i) {
-    const u32 v = in[(u64)i * stride];
+    const u32 v = in[i];
     out[i] = run;
     run += v;
   }
@@ -39,9 +39,11 @@ __global__ void __launch_bounds__(1024) k_scan_small(const u32* in, int stride, 
 
 // Up to three arrays of one length at once (blockIdx.y: which), as two kernels:
 // the tiles' sums, then the tiles, every block adding the sums before its tile
-// itself.  For up to some thousand tiles that costs less than a launch of one
-// block for their scan (1.9e7 values: 22 us for the three-kernel form's middle
-// kernel and its gap alone); above, the sums are scanned in between.
+// itself.  Up to SELF_TILES tiles that costs less than a launch of one block that
+// scans the sums in between (one array, caches flushed: 1.0e6 values 19 and 23 us,
+// 8.0e6 59 and 64, 1.67e7 -- 8155 tiles -- 109 and 117); above, where the sums
+// read grow with the square of the tiles, they are scanned (equal near 4e7 values;
+// 5.0e7: 322 and 312 us).
 // A value is the word itself or, with BITS, the number of its bits (of a
 // bit-plane with rows of wpr words, those of columns 0 .. W; wpr 0: all).
 struct Scan3 {
@@ -116,7 +118,7 @@ int run_scan(const Scan3& s, int arrays, u32 n, cudaStream_t st) {
     k_tile_scan<BITS, false><<<dim3(tiles, arrays), 256, 0, st>>>(s, n);
     return 2;
   }
-  for (int k = 0; k < arrays; ++k) k_scan_small<<<1, 1024, 0, st>>>(s.part[k], 1, s.part[k], tiles);
+  for (int k = 0; k < arrays; ++k) k_scan_small<<<1, 1024, 0, st>>>(s.part[k], s.part[k], tiles);
   k_tile_scan<BITS, true><<<dim3(tiles, arrays), 256, 0, st>>>(s, n);
   return 2 + arrays;
 }
@@ -222,7 +224,7 @@ size_t scan_scratch_words(u32 n) { return (size_t)n / TILE + 2; }
 
 int launch_scan(const u32* in, u32* out, u32 n, u32* scratch, cudaStream_t st) {
   if (n <= 4096) {
-    k_scan_small<<<1, 1024, 0, st>>>(in, 1, out, n);
+    k_scan_small<<<1, 1024, 0, st>>>(in, out, n);
     return 1;
   }
   Scan3 s{};
