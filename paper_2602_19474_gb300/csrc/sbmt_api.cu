@@ -1798,8 +1798,7 @@ int mesh_query(sbmt_ctx* ctx, sbmt_mesh mesh, int wait_ms, sbmt_mesh_view* out) 
   std::memset(out, 0, sizeof *out);
   out->n_vertices = m->nv, out->n_triangles = m->nt, out->n_cells = m->ncells;
   if (m->r3) {
-    // h_info: error bits, cut cells, Tier-G cells (all queued), Tier-G
-    // triangles, candidates, Tier-G cells done by one thread
+    // h_info: error bits, cut cells, Tier-G cells, Tier-G triangles, candidates
     out->n_cut_cells = m->h_info[1], out->n_tierG_cells = m->h_info[2];
     out->n_tierG_triangles = m->h_info[3];
     out->n_events = m->ne_total, out->n_inside_vertices = m->nc_total, out->n_lattice_vertices = m->nvg;
@@ -2086,9 +2085,9 @@ int mesh_stage(sbmt_ctx* ctx, sbmt_mesh mesh, int stage, void* host_out, int64_t
   auto it = ctx->meshes.find(mesh);
   if (it == ctx->meshes.end()) return fail(SBMT_ENOENT, "unknown mesh");
   MeshRec* m = it->second;
-  if (stage == 4) {  // cells over the Tier-G limit, for every mesh (none in a preprocessed one)
+  if (stage == 4) {  // cells over the Tier-G limit, for every mesh (none in a preprocessed or retriangulated one)
     CK(cudaEventSynchronize(m->done));
-    const u32 cnt = m->pre ? 0u : m->h_info[4], kept = std::min<u32>(cnt, OVER_CAP);
+    const u32 cnt = m->pre || m->r3 ? 0u : m->h_info[4], kept = std::min<u32>(cnt, OVER_CAP);
     std::vector<u32> ids(kept);
     if (kept) CK(cudaMemcpy(ids.data(), m->over_cells, kept * sizeof(u32), cudaMemcpyDeviceToHost));
     std::sort(ids.begin(), ids.end());

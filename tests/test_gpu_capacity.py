@@ -41,3 +41,14 @@ def test_no_cells_over_the_limit_at_h2():
     assert v.status == sb.SBMT_OK
     assert len(sb.mesh_stage(c, m, 4)) == 0
     sb.mesh_release(c, m)
+
+
+def test_meshes_without_the_lattice_path_list_none():
+    c = ctx()
+    img = synth.disk()
+    pre = sb.mesh_preprocess(c, img, 2, 1)
+    own = sb.mesh_import(c, np.array([[0.0, 0.0], [9.0, 0.0], [0.0, 9.0]]), np.array([[0, 1, 2]], np.int32))
+    for m in (pre, sb.mesh_retriangulate(c, img, pre), own):
+        sb.mesh_query(c, m, -1)
+        assert sb.mesh_stage(c, m, 4).shape[0] == 0
+        sb.mesh_release(c, m)
