@@ -120,7 +120,7 @@ def load_serving_pool() -> list:
 STAGE_SOURCES = {
     "k_corner_bits": ["k_extract.cu"], "k_segments": ["k_extract.cu"], "k_seg_count": ["k_extract.cu", "k_traverse.cu"],
     "k_walk": ["k_traverse.cu"], "k_rank": ["k_traverse.cu"], "k_sort": ["k_cells.cu"],
-    "k_cutcells": ["k_cells.cu"], "k_emit": ["k_cells.cu"], "k_tierg": ["k_tierg.cu"],
+    "k_cutcells": ["k_cells.cu"], "k_emit": ["k_cells.cu"], "k_tierg": ["k_tierg.cu", "sbmt_greedy.cuh"],
     "k_lattice_xy": ["k_cells.cu"], "k_scan": ["k_scan.cu"],
 }
 
