@@ -521,92 +521,88 @@ __global__ void __launch_bounds__(CT, 1) k_heat_cg(const __grid_constant__ HeatC
   auto dinv_at = [&](u32 l) { return ONCHIP ? dinv[l] : h.dinv[row0 + l]; };
   u32 gen = 0;
   for (u32 step = 0; step < h.nsteps; ++step) {
-    // b = M x; r = b - A x, z = D^-1 r; r.z, r.r, b.b
-    double a3[3] = {0.0, 0.0, 0.0};
-    for (u32 l = tid; l < rows; l += CT) {
-      const u32 i = row0 + l;
-      const double xi = x[l], bi = h.mass[i] * xi, dd = h.dg[i] * xi;
-      const double qi = row_times(h, i, h.x, dd);
-      const double di = dinv_at(l), rv = di != 0.0 ? bi - qi : 0.0, zv = rv * di;
-      r[l] = rv, z[l] = zv, p[l] = 0.0, q[l] = 0.0, h.b[i] = bi;
-      if (ONCHIP) h.z[i] = zv;
-      a3[0] += rv * zv, a3[1] += rv * rv, a3[2] += bi * bi;
-    }
-    if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
-    double rz = s_sum[0], rr = s_sum[1], be = 0.0;
-    const double stop = h.tol * h.tol * s_sum[2];
+    double rz = 0.0, rr = 0.0, be = 0.0, stop = 0.0;
     int it = 0, anew = ANEW;
-    while (rr > stop && it < h.maxit) {
-      bool look = false;
-      while (!look) {
-        double a1[1] = {0.0};
-        for (u32 l = tid; l < rows; l += CT) {
-          // (the diagonal times z is r, up to z's rounding)
-          const double qv = row_times(h, row0 + l, h.z, r[l]) + be * q[l], pv = z[l] + be * p[l];
-          q[l] = qv, p[l] = pv;
-          a1[0] += pv * qv;
-        }
-        if (!grid_sums<1, true>(h, a1, gen, s, s_sum, &s_fail, [] {},
-                                [&](const double* t) { s_k = t[0] != 0.0 ? rz / t[0] : 0.0; }))
-          return;
-        const double al = s_k;
-        ++it;
-        look = (it & 7) == 0 || it == h.maxit;  // the residual is looked at (and summed) every eighth iteration
-        double a2[2] = {0.0, 0.0};
-        for (u32 l0 = tid; l0 < rows; l0 += 3 * CT) {
-          double rv[3], qv[3], dv[3];
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const u32 l = l0 + u * CT;
-            if (l < rows) rv[u] = r[l], qv[u] = q[l], dv[u] = dinv_at(l);
-          }
-#pragma unroll
-          for (int u = 0; u < 3; ++u) {
-            const u32 l = l0 + u * CT;
-            if (l >= rows) continue;
-            const double rn = rv[u] - al * qv[u], zn = rn * dv[u];
-            r[l] = rn, z[l] = zn;
-            if (ONCHIP) h.z[row0 + l] = zn;
-            a2[0] += rn * zn;
-            if (look) a2[1] += rn * rn;
-          }
-        }
-        // (x is not needed before the next step: updated while the sums travel)
-        auto update_x = [&] {
-#pragma unroll 4
-          for (u32 l = tid; l < rows; l += CT) x[l] += al * p[l];
-        };
-        const auto beta = [&](const double* t) { s_k = rz != 0.0 ? t[0] / rz : 0.0; };
-        if (look) {
-          if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail, update_x, beta)) return;
-        } else {
-          const double only[1] = {a2[0]};
-          if (!grid_sums<1, true>(h, only, gen, s, s_sum, &s_fail, update_x, beta)) return;
-        }
-        rz = s_sum[0], be = s_k;
-        if (look) rr = s_sum[1];
-      }
-      if (it == anew && rr > stop) {
-        // r = b - A x again, in the place of the recurrence's (x of all blocks
-        // is there after the barrier); the direction goes on
-        anew *= 4;
+    bool first = true;
+    while (true) {
+      // b = M x; r = b - A x, z = D^-1 r; r.z, r.r, b.b.  Later in the step, r anew in
+      // the place of the recurrence's: the direction goes on
+      if (!first) {
         if (ONCHIP)
           for (u32 l = tid; l < rows; l += CT) h.x[row0 + l] = x[l];
-        const double none[1] = {0.0};
+        const double none[1] = {0.0};  // (x of all blocks is there after the barrier)
         if (!grid_sums<1, false>(h, none, gen, s, s_sum, &s_fail, [] {}, [](const double*) {})) return;
-        double a2[2] = {0.0, 0.0};
-        for (u32 l = tid; l < rows; l += CT) {
-          const u32 i = row0 + l;
-          const double di = dinv_at(l), rv = di != 0.0 ? h.b[i] - row_times(h, i, h.x, h.dg[i] * x[l]) : 0.0, zv = rv * di;
-          r[l] = rv, z[l] = zv;
-          if (ONCHIP) h.z[i] = zv;
-          a2[0] += rv * zv, a2[1] += rv * rv;
-        }
-        if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail, [] {},
-                                [&](const double* t) { s_k = rz != 0.0 ? be * (t[0] / rz) : 0.0; }))
-          return;
-        rz = s_sum[0], rr = s_sum[1], be = s_k;
       }
+      double a3[3] = {0.0, 0.0, 0.0};
+      for (u32 l = tid; l < rows; l += CT) {
+        const u32 i = row0 + l;
+        const double xi = x[l], bi = first ? h.mass[i] * xi : h.b[i], dd = h.dg[i] * xi;
+        const double qi = row_times(h, i, h.x, dd);
+        const double di = dinv_at(l), rv = di != 0.0 ? bi - qi : 0.0, zv = rv * di;
+        r[l] = rv, z[l] = zv;
+        if (first) p[l] = 0.0, q[l] = 0.0, h.b[i] = bi;
+        if (ONCHIP) h.z[i] = zv;
+        a3[0] += rv * zv, a3[1] += rv * rv, a3[2] += bi * bi;
+      }
+      if (!grid_sums<3, true>(h, a3, gen, s, s_sum, &s_fail, [] {},
+                              [&](const double* t) { s_k = rz != 0.0 ? be * (t[0] / rz) : 0.0; }))
+        return;
+      rz = s_sum[0], rr = s_sum[1], be = s_k;
+      if (first) stop = h.tol * h.tol * s_sum[2];
+      first = false;
+      while (rr > stop && it < h.maxit && it != anew) {
+        bool look = false;
+        while (!look) {
+          double a1[1] = {0.0};
+          for (u32 l = tid; l < rows; l += CT) {
+            // (the diagonal times z is r, up to z's rounding)
+            const double qv = row_times(h, row0 + l, h.z, r[l]) + be * q[l], pv = z[l] + be * p[l];
+            q[l] = qv, p[l] = pv;
+            a1[0] += pv * qv;
+          }
+          if (!grid_sums<1, true>(h, a1, gen, s, s_sum, &s_fail, [] {},
+                                  [&](const double* t) { s_k = t[0] != 0.0 ? rz / t[0] : 0.0; }))
+            return;
+          const double al = s_k;
+          ++it;
+          look = (it & 7) == 0 || it == h.maxit;  // the residual is looked at (and summed) every eighth iteration
+          double a2[2] = {0.0, 0.0};
+          for (u32 l0 = tid; l0 < rows; l0 += 3 * CT) {
+            double rv[3], qv[3], dv[3];
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+              const u32 l = l0 + u * CT;
+              if (l < rows) rv[u] = r[l], qv[u] = q[l], dv[u] = dinv_at(l);
+            }
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {
+              const u32 l = l0 + u * CT;
+              if (l >= rows) continue;
+              const double rn = rv[u] - al * qv[u], zn = rn * dv[u];
+              r[l] = rn, z[l] = zn;
+              if (ONCHIP) h.z[row0 + l] = zn;
+              a2[0] += rn * zn;
+              if (look) a2[1] += rn * rn;
+            }
+          }
+          // (x is not needed before the next step: updated while the sums travel)
+          auto update_x = [&] {
+#pragma unroll 4
+            for (u32 l = tid; l < rows; l += CT) x[l] += al * p[l];
+          };
+          const auto beta = [&](const double* t) { s_k = rz != 0.0 ? t[0] / rz : 0.0; };
+          if (look) {
+            if (!grid_sums<2, true>(h, a2, gen, s, s_sum, &s_fail, update_x, beta)) return;
+          } else {
+            const double only[1] = {a2[0]};
+            if (!grid_sums<1, true>(h, only, gen, s, s_sum, &s_fail, update_x, beta)) return;
+          }
+          rz = s_sum[0], be = s_k;
+          if (look) rr = s_sum[1];
+        }
+      }
+      if (!(rr > stop) || it >= h.maxit) break;
+      anew *= 4;
     }
     // the step's peak (positive doubles order as their bits, infinity above all;
     // NaNs are left out, as fmax leaves them), and x for the next step's product
