@@ -421,7 +421,8 @@ int mesh_project(sbmt_ctx* ctx, sbmt_mesh mesh, const sbmt_image* field, float* 
  *    vertex;
  *  - backward Euler: (M + alpha dt K) u_{n+1} = M u_n on the free vertices.
  * Each step is solved by conjugate gradients with the diagonal as
- * preconditioner, started from u_n, until |r| <= tol |b|, in double
+ * preconditioner, started from u_n, until |r| <= tol |b| (r as the iteration
+ * carries it, taken anew as b - A x after 96, 384, ... iterations), in double
  * precision.
  *  u0 = amplitude exp(-|x - (x0, y0)|^2 / (2 sigma^2)) at the free vertices
  *  (pixel units; alpha in px^2 per unit time).

@@ -1776,9 +1776,9 @@ int mesh_query(sbmt_ctx* ctx, sbmt_mesh mesh, int wait_ms, sbmt_mesh_view* out) 
     m = it->second;
   }
   // A wait without a limit polls without a pause for its first 5 ms (a sleep of
-  // 20 us between polls overslept by some 50, a tenth of a small mesh's call; giving
-  // way between them cost 2 to 4 us), and then sleeps between polls like one with a limit, so that a thread in a long
-  // wait leaves its core to others.
+  // 20 us between polls overslept by some 50, a tenth of a small mesh's call;
+  // giving way between them cost 2 to 4 us), and then sleeps between polls like
+  // one with a limit, so that a thread in a long wait leaves its core to others.
   const auto t0 = std::chrono::steady_clock::now();
   while (true) {
     const cudaError_t q = cudaEventQuery(m->done);
