@@ -401,6 +401,9 @@ def _pool_bytes():
     """The bytes in use of the device's stream-ordered allocations."""
     import ctypes
 
+    import torch
+
+    torch.cuda.synchronize()
     cu = ctypes.CDLL("libcuda.so.1")
     pool, used = ctypes.c_void_p(), ctypes.c_uint64()
     assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
